@@ -873,6 +873,10 @@ static int launch_ts_t(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_
 
 int launch_ts(bool fp64, const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_t st) {
   if (a.nq > MAXB || a.gram_left > a.nq || a.r < 1 || a.r > MAX_R) return -1;
+  if (fp64) {
+    const int n = launch_tsx(a, nsm, st);
+    if (n > 0) return n;
+  }
   return fp64 ? launch_ts_t<double>(M, a, nsm, st) : launch_ts_t<float>(M, a, nsm, st);
 }
 
@@ -1083,7 +1087,7 @@ void launch_check_finite(bool fp64, const void *X, long long N, int r, int *stat
 namespace lrei {
 // Raise the dynamic shared-memory limit of every tile kernel once (outside any stream capture).
 int ts_init() {
-  if (hv_tiled_init()) return -1;
+  if (hv_tiled_init() || tsx_init()) return -1;
   const int lim = 210 * 1024;
   cudaError_t e = cudaSuccess;
   auto set = [&](const void *f) {

@@ -28,6 +28,7 @@ struct TSArgs {
   int mode;
   void *coef_scratch;   // device, >= (MAXB+1)*MAX_R*MAX_R*16 bytes (converted coefficients)
   long long zero_rows;  // modes 1, 2: rows < zero_rows of the new block are set to zero
+  int *status;          // device status word (may be NULL)
 };
 
 // Returns the grid size used (number of partials written), or -1 on error.
@@ -35,6 +36,10 @@ int launch_ts(bool fp64, const ModelArgs &M, const TSArgs &a, int nsm, cudaStrea
 int ts_max_grid(int nsm);
 int ts_init();
 size_t ts_partial_doubles(int gram_left, int r);   // per CTA
+
+// The same pass of complex128 blocks on the tensor cores (tsx.cu): the number of partials, 0 when it does not apply.
+int launch_tsx(const TSArgs &a, int nsm, cudaStream_t st);
+int tsx_init();
 
 void launch_reduce(const double *partial, int nparts, int len_doubles, double *out, cudaStream_t st);
 
