@@ -9,7 +9,7 @@
 // invariant subspace (sm_eig_topr), so only r x r Jacobi runs in FP64.
 #include "small.cuh"
 
-#include <cstdlib>
+#include <algorithm>
 
 namespace lrei {
 
@@ -35,43 +35,59 @@ __device__ __forceinline__ zd opget(char op, const zd *A, int ld, int i, int p) 
   return op == 'N' ? A[(size_t)p * ld + i] : conj(A[(size_t)i * ld + p]);
 }
 
-__global__ void gemm_thread_kernel(char opA, char opB, int M, int N, int K, zd alpha, const zd *__restrict__ A, int lda,
-                                   const zd *__restrict__ B, int ldb, zd beta, zd *__restrict__ C, int ldc) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= M * N) return;
-  const int i = e % M, j = e / M;
+// One output per LN lanes of a warp: each lane sums every LN-th term, the lanes are combined by shuffles.  An FP64
+// instruction takes a scheduler 64 cycles here whatever the number of active lanes (measured, also in a dependent
+// chain), so a sum of K terms by one thread is a chain of 4 K x 64 cycles and by LN lanes of 4 K / LN + 2 log2 LN.
+template <int LN>
+__global__ void __launch_bounds__(128) gemm_kernel(char opA, char opB, int M, int N, int K, zd alpha, const zd *__restrict__ A,
+                                                   int lda, const zd *__restrict__ B, int ldb, zd beta, zd *__restrict__ C,
+                                                   int ldc) {
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) / LN, lane = threadIdx.x % LN;
+  const bool in = w < M * N;
+  const int i = in ? w % M : 0, j = in ? w / M : 0;
   zd s = mk<double>(0, 0);
-  for (int p = 0; p < K; ++p) fma_(s, opget(opA, A, lda, i, p), opget(opB, B, ldb, p, j));
-  zd c = alpha * s;
-  if (beta.re != 0.0 || beta.im != 0.0) c = c + beta * C[(size_t)j * ldc + i];
-  C[(size_t)j * ldc + i] = c;
-}
-
-__global__ void gemm_warp_kernel(char opA, char opB, int M, int N, int K, zd alpha, const zd *__restrict__ A, int lda,
-                                 const zd *__restrict__ B, int ldb, zd beta, zd *__restrict__ C, int ldc) {
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (w >= M * N) return;
-  const int i = w % M, j = w / M;
-  zd s = mk<double>(0, 0);
-  for (int p = lane; p < K; p += 32) fma_(s, opget(opA, A, lda, i, p), opget(opB, B, ldb, p, j));
-  s = warp_sum(s);
-  if (lane == 0) {
+  for (int p = lane; p < K; p += LN) fma_(s, opget(opA, A, lda, i, p), opget(opB, B, ldb, p, j));
+#pragma unroll
+  for (int o = LN / 2; o > 0; o >>= 1) {
+    s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
+    s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
+  }
+  if (in && lane == 0) {
     zd c = alpha * s;
     if (beta.re != 0.0 || beta.im != 0.0) c = c + beta * C[(size_t)j * ldc + i];
     C[(size_t)j * ldc + i] = c;
   }
 }
 
+// Lanes per output: the least of the longest chain (its FP64 instructions at 64 cycles) and the SMs' throughput (one
+// FP64 warp instruction in 19 cycles and SM, over 152 SMs).  Measured over an RK4 step at n = 16, r = 8 (K = 8..72):
+// 8.7 us a launch with one thread per output, 4.3 with the lanes chosen here; the step 1.58 ms before, 1.40 after.
+static int gemm_lanes(int M, int N, int K) {
+  int best = 4;
+  double cost = 1e300;
+  for (int ln = 4, lg = 2; ln <= 32; ln *= 2, ++lg) {
+    const double instr = 4.0 * ((K + ln - 1) / ln) + 2.0 * lg + 4.0;
+    const double warps = (double)M * N * ln / 32.0;
+    const double c = std::max(64.0 * instr, warps * instr * 19.0 / 152.0);
+    if (c < cost) {
+      cost = c;
+      best = ln;
+    }
+  }
+  return best;
+}
+
 void sm_gemm(char opA, char opB, int M, int N, int K, zd alpha, const zd *A, int lda, const zd *B, int ldb, zd beta,
              zd *C, int ldc, cudaStream_t st) {
   if (M <= 0 || N <= 0) return;
-  if (K >= 48) {
-    const long long threads = (long long)M * N * 32;
-    ::lrei::count_launch(); gemm_warp_kernel<<<(int)((threads + 127) / 128), 128, 0, st>>>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C,
-                                                                    ldc);
-  } else {
-    ::lrei::count_launch(); gemm_thread_kernel<<<(M * N + 63) / 64, 64, 0, st>>>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
-  }
+  const int ln = gemm_lanes(M, N, K);
+  const int grid = (int)(((long long)M * N * ln + 127) / 128);
+  ::lrei::count_launch();
+  auto go = [&](auto kern) { kern<<<grid, 128, 0, st>>>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); };
+  if (ln == 4) go(gemm_kernel<4>);
+  else if (ln == 8) go(gemm_kernel<8>);
+  else if (ln == 16) go(gemm_kernel<16>);
+  else go(gemm_kernel<32>);
 }
 
 // ------------------------------------------------------- triangular solves
