@@ -186,30 +186,16 @@ __global__ void stage_factors_kernel(StagePtrs P, StageCoefs C, const double *__
   }
 }
 
-// Rc = Lr^H with the rows of dead residual columns zeroed, written into Chat.
-__global__ void store_rc_kernel(const zd *__restrict__ Lr, int r, const int *__restrict__ dead, zd *__restrict__ dst,
-                                int ld) {
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e % r, j = e / r;
-    zd v = (i <= j) ? conj(Lr[(size_t)i * r + j]) : mk<double>(0, 0);
-    if (dead[i]) v = mk<double>(0, 0);
-    dst[(size_t)j * ld + i] = v;
-  }
-}
-
-// New rows k..k+r-1 of the Cholesky factor of Gamma: [Bs^H | L22].  A dead column (numerically
-// dependent on the earlier ones) is decoupled from the later columns; with keep_dead its row keeps
-// the projections onto the earlier frame vectors, else it is zeroed too.  dead_frame (may be NULL)
+// The part of the new rows k..k+r-1 of the Cholesky factor of Gamma left of their diagonal block (which the
+// Cholesky kernel writes): Bs^H.  A dead column (numerically dependent on the earlier ones) is decoupled from the later
+// columns; with keep_dead its row keeps the projections onto the earlier frame vectors, else it is zeroed too.  dead_frame (may be NULL)
 // receives the dead flags of the new columns.
-__global__ void store_lrows_kernel(const zd *__restrict__ Bs, int ldb, const zd *__restrict__ L22, int r, int k,
+__global__ void store_lrows_kernel(const zd *__restrict__ Bs, int ldb, int r, int k,
                                    const int *__restrict__ dead, zd *__restrict__ L, int ldl, int keep_dead,
                                    int *__restrict__ dead_frame) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < r * (k + r); e += gridDim.x * blockDim.x) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < r * k; e += gridDim.x * blockDim.x) {
     const int j = e % r, m = e / r;   // row k + j, column m
-    zd v;
-    if (m < k) v = (dead[j] && !keep_dead) ? mk<double>(0, 0) : conj(Bs[(size_t)j * ldb + m]);
-    else v = L22[(size_t)(m - k) * r + j];
-    L[(size_t)m * ldl + (k + j)] = v;
+    L[(size_t)m * ldl + (k + j)] = (dead[j] && !keep_dead) ? mk<double>(0, 0) : conj(Bs[(size_t)j * ldb + m]);
   }
   if (dead_frame && blockIdx.x == 0)
     for (int j = threadIdx.x; j < r; j += blockDim.x) dead_frame[k + j] = dead[j];
@@ -744,7 +730,7 @@ struct lrei_ctx {
   // second stream of the RK step: the stage algebra of stage j runs on it while the N-length
   // passes of the later Krylov blocks run on st (events: fork, Krylov block j done, join)
   cudaStream_t st2 = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_kry[4] = {};
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_inv = nullptr, ev_kry[4] = {};
   int nsm_pass = 0;   // SMs the N-length passes of the RK step use (the rest serve the stage algebra)
   int eig_sweeps = 30;   // FP64 Jacobi sweep limit of each partial eigendecomposition
   ModelArgs M;
@@ -758,7 +744,7 @@ struct lrei_ctx {
   double *partial = nullptr;
   double *red = nullptr;
   void *coef_scratch = nullptr;
-  zd *Gam = nullptr, *L = nullptr, *Chat = nullptr, *Tbar = nullptr, *Xh = nullptr, *Cc = nullptr, *GR = nullptr,
+  zd *Gam = nullptr, *L = nullptr, *Li = nullptr, *Tr = nullptr, *Chat = nullptr, *Tbar = nullptr, *Cc = nullptr, *GR = nullptr,
      *Lr = nullptr, *Ainv = nullptr, *coefQ = nullptr, *Bs = nullptr, *Dm = nullptr, *L22 = nullptr, *Mm = nullptr,
      *Uf = nullptr, *Vf = nullptr, *Yc = nullptr, *ts = nullptr, *G = nullptr, *X11 = nullptr, *Gh = nullptr;
   zd *ys[5] = {}, *zs[4] = {}, *wsv[4] = {};
@@ -874,27 +860,51 @@ void *qblock(lrei_ctx *c, int m) { return m == 0 ? c->V : c->blk[m - 1]; }
 // Gamma[0:r,0:r] <- red (V^*V), L[0:r,0:r] <- chol.
 void set_gamma00(lrei_ctx *c) {
   const int r = c->r, KM = c->KM;
-  sm_copy(reinterpret_cast<zd *>(c->red), r, r, r, c->Gam, KM, c->st);
-  sm_hermitize(c->Gam, KM, r, c->st);
-  sm_chol(c->Gam, KM, r, c->L22, r, TOL_GAM, 1, c->dead_dev, c->status_dev, 1, c->st);
-  sm_copy(c->L22, r, r, r, c->L, KM, c->st);
+  sm_herm_copy(reinterpret_cast<zd *>(c->red), r, r, c->Gam, KM, c->st);
+  sm_chol(c->Gam, KM, r, c->L, KM, TOL_GAM, 1, c->dead_dev, c->status_dev, 1, c->st);
+}
+
+// Li[0:r,0:r] <- L[0:r,0:r]^{-1}, on stream st.  Li is the inverse of the frame's Cholesky factor L (lower triangular,
+// well conditioned: the frame's blocks are normalised or their columns scaled by L itself), kept block by block, so that
+// a triangular solve is a product spread over the GPU (about 4 us) instead of a chain of k steps in
+// one warp (24 us at k = 16..64).  Recomputed from L in every step, so a step depends on the stored L only.
+void start_inverse(lrei_ctx *c, cudaStream_t st) {
+  const int r = c->r, KM = c->KM;
+  sm_set_identity(c->Li, KM, r, r, st);
+  sm_trsv('N', c->L, KM, r, c->Li, KM, r, st);
+}
+
+// The frame extended by block Q_i (k = i r earlier columns), from its measured Gram column in red: the new rows of L
+// and of its inverse.  ref: the squared norms the pivots are judged against (NULL: the largest diagonal entry).
+void extend_frame(lrei_ctx *c, int k, bool keep_dead, int *dead_frame, const zd *ref, int ldref) {
+  const int r = c->r, KM = c->KM, ldr = k + r;
+  cudaStream_t st = c->st;
+  const zd *red = reinterpret_cast<const zd *>(c->red);
+  zd *L22 = c->L + (size_t)k * KM + k, *I22 = c->Li + (size_t)k * KM + k;
+  sm_gemm('N', 'N', k, r, k, ONE, c->Li, KM, red, ldr, ZERO, c->Bs, KM, st);                       // Bs = L^{-1} Gamma_col
+  sm_gemm_herm('C', 'N', r, k, MONE, c->Bs, KM, c->Bs, KM, ONE, red + k, ldr, c->Dm, r, st);       // Schur complement
+  sm_chol(c->Dm, r, r, L22, KM, TOL_GAM, keep_dead ? 0 : 1, c->dead_dev, c->status_dev, 0, st, ref, ldref, I22, KM);
+  ::lrei::count_launch();
+  store_lrows_kernel<<<8, 256, 0, st>>>(c->Bs, KM, r, k, c->dead_dev, c->L, KM, keep_dead ? 1 : 0, dead_frame);
+  // rows k.. of the inverse: -L22^{-1} (L21 L11^{-1})
+  sm_gemm('N', 'N', r, k, k, ONE, c->L + k, KM, c->Li, KM, ZERO, c->Tr, r, st);
+  sm_gemm('N', 'N', r, k, r, MONE, I22, KM, c->Tr, r, ZERO, c->Li + k, KM, st);
 }
 
 // Stage j of an RK step, on stream st2: the stage quantities in the orthonormal frame (G_j, X11,
 // W_j, Z_j), the stage matrix of K_{j+2} (or of rho_{k+1} for the last stage) and its top-r
 // eigenpairs.  It needs the frame of Q_0..Q_{j+1} only: with a = (j+2) r and b = (j+1) r,
 // Tbar[0:a, 0:b] = L_a^H Chat[0:a, 0:b] L_b^{-H}, because L is lower triangular and H Q_m lies
-// in span(Q_0..Q_{m+1}).
+// in span(Q_0..Q_{m+1}); for the same reason stage j adds the last r columns only (the entries below them
+// are zero, set at the step's start).
 void enqueue_stage(lrei_ctx *c, const Tableau &tb, int j, cudaStream_t st2) {
   const int s = tb.s, r = c->r, KM = c->KM, K = (s + 1) * r;
   const int a = (j + 2) * r, b = (j + 1) * r;
-  sm_conj_transpose(c->Chat, KM, a, b, c->Xh, KM, st2);
-  sm_trsv('N', c->L, KM, b, c->Xh, KM, a, st2);
-  sm_gemm('C', 'C', a, b, a, ONE, c->L, KM, c->Xh, KM, ZERO, c->Tbar, KM, st2);
+  sm_gemm('N', 'C', a, r, b, ONE, c->Chat, KM, c->Li + (size_t)j * r, KM, ZERO, c->Yc, KM, st2);
+  sm_gemm('C', 'N', a, r, a, ONE, c->L, KM, c->Yc, KM, ZERO, c->Tbar + (size_t)j * r * KM, KM, st2);
   sm_hermitize(c->Tbar, KM, b, st2);
-  // H V_j in the frame (ys[j] has no rows beyond b); rows a..K of ts are zero
-  if (a < K) sm_zero(c->ts + a, KM, K - a, r, st2);
-  sm_gemm('N', 'N', a, r, b, ONE, c->Tbar, KM, c->ys[j], KM, ZERO, c->ts, KM, st2);
+  // H V_j in the frame (ys[j] has no rows beyond b)
+  sm_gemm('N', 'N', K, r, b, ONE, c->Tbar, KM, c->ys[j], KM, ZERO, c->ts, KM, st2);
   sm_gemm('C', 'N', r, r, b, ONE, c->ys[j], KM, c->ts, KM, ZERO, c->G, r, st2);
   ::lrei::count_launch();
   stage_xwz_kernel<<<r, 128, 2 * r * sizeof(zd), st2>>>(c->G, r, c->lam0_dev, c->kappa, c->model, c->ys[j], c->ts, K,
@@ -917,10 +927,8 @@ void enqueue_stage(lrei_ctx *c, const Tableau &tb, int j, cudaStream_t st2) {
   const int kk = last ? K : (j + 2) * r;
   ::lrei::count_launch();
   stage_factors_kernel<<<64, 256, 0, st2>>>(P, C, c->lam0_dev, c->dt_dev, r, K, KM, c->Uf, c->Vf);
-  sm_gemm('N', 'C', kk, kk, nf, ONE, c->Uf, KM, c->Vf, KM, ZERO, c->Mm, KM, st2);
-  sm_hermitize(c->Mm, KM, kk, st2);
-  zd *dst = last ? c->yfin : c->ys[j + 1];
-  sm_zero(dst, KM, K, r, st2);
+  sm_gemm_herm('N', 'C', kk, nf, ONE, c->Uf, KM, c->Vf, KM, ZERO, c->Mm, KM, c->Mm, KM, st2);
+  zd *dst = last ? c->yfin : c->ys[j + 1];   // rows beyond kk: zero, set at the step's start
   sm_eig_topr(c->Mm, KM, kk, r, dst, KM, c->mu_dev, c->eig_ws, c->status_dev, st2, c->eig_sweeps);
 }
 
@@ -936,8 +944,13 @@ int enqueue_rk_step(lrei_ctx *c, int scheme) {
   zd *red = reinterpret_cast<zd *>(c->red);
   LREI_CUDA_TRY(cudaEventRecord(c->ev_fork, st));
   LREI_CUDA_TRY(cudaStreamWaitEvent(st2, c->ev_fork, 0));
-  sm_zero(c->ys[0], KM, K, r, st2);
-  sm_set_identity(c->ys[0], KM, r, r, st2);
+  // beside the first Krylov block: the inverse of L_00, and the zeros the stages count on
+  start_inverse(c, st2);
+  LREI_CUDA_TRY(cudaEventRecord(c->ev_inv, st2));
+  sm_set_identity(c->ys[0], KM, K, r, st2);
+  for (int j = 1; j < s; ++j) sm_zero(c->ys[j], KM, K, r, st2);
+  sm_zero(c->yfin, KM, K, r, st2);
+  sm_zero(c->Tbar, KM, K, K, st2);
   for (int l = 0; l < s; ++l) {
     const int k = (l + 1) * r, ldr = (l + 2) * r;
     // pass A: S = H Q_l (formed once by the H.V kernel; both passes read it), then
@@ -952,21 +965,16 @@ int enqueue_rk_step(lrei_ctx *c, int scheme) {
     a.mode = 0;
     int rc = ts_pass(c, a, c->nsm_pass);
     if (rc) return rc;
-    // C = Gamma^{-1} P
-    sm_copy(red, ldr, k, r, c->Cc, KM, st);
-    sm_trsv('N', c->L, KM, k, c->Cc, KM, r, st);
-    sm_trsv('C', c->L, KM, k, c->Cc, KM, r, st);
-    // GR = S^*S - P^* C (Gram of the projected residual)
-    sm_copy(red + k, ldr, r, r, c->GR, r, st);
-    sm_gemm('C', 'N', r, r, k, MONE, red, ldr, c->Cc, KM, ONE, c->GR, r, st);
-    sm_hermitize(c->GR, r, r, st);
-    sm_chol(c->GR, r, r, c->Lr, r, tol_rc(c), 0, c->dead_dev, c->status_dev, 0, st, red + k, ldr);
-    // A = (Lr^H)^{-1}; coefQ = -C A; Chat column block l = [C; Lr^H]
-    sm_set_identity(c->Ainv, r, r, r, st);
-    sm_trsv('C', c->Lr, r, r, c->Ainv, r, r, st);
-    sm_gemm('N', 'N', k, r, r, MONE, c->Cc, KM, c->Ainv, r, ZERO, c->coefQ, k, st);
-    sm_copy(c->Cc, KM, k, r, c->Chat + (size_t)l * r * KM, KM, st);
-    ::lrei::count_launch(); store_rc_kernel<<<1, 256, 0, st>>>(c->Lr, r, c->dead_dev, c->Chat + (size_t)l * r * KM + k, KM);
+    if (l == 0) LREI_CUDA_TRY(cudaStreamWaitEvent(st, c->ev_inv, 0));
+    // T = L^{-1} P; the Gram of the projected residual GR = S^*S - P^* Gamma^{-1} P = S^*S - T^*T = Lr Lr^H;
+    // A = (Lr^H)^{-1}; Chat column block l = [C; Lr^H], C = Gamma^{-1} P = L^{-H} T; coefQ = -C A
+    zd *Cl = c->Chat + (size_t)l * r * KM;
+    sm_gemm('N', 'N', k, r, k, ONE, c->Li, KM, red, ldr, ZERO, c->Cc, KM, st);
+    sm_gemm_herm('C', 'N', r, k, MONE, c->Cc, KM, c->Cc, KM, ONE, red + k, ldr, c->GR, r, st);
+    sm_chol(c->GR, r, r, nullptr, 0, tol_rc(c), 0, c->dead_dev, c->status_dev, 0, st, red + k, ldr, c->Ainv, r, 1,
+            Cl + k, KM);
+    sm_gemm('C', 'N', k, r, k, ONE, c->Li, KM, c->Cc, KM, ZERO, Cl, KM, st);
+    sm_gemm('N', 'N', k, r, r, MONE, Cl, KM, c->Ainv, r, ZERO, c->coefQ, k, st);
     // pass B: Q_{l+1} = S A - Q C A, Gram column [Q_0..Q_l, Q_{l+1}]^* Q_{l+1}
     TSArgs b = a;
     b.mode = 1;
@@ -975,16 +983,7 @@ int enqueue_rk_step(lrei_ctx *c, int scheme) {
     b.out = qblock(c, l + 1);
     rc = ts_pass(c, b, c->nsm_pass);
     if (rc) return rc;
-    sm_store_gram_cols(red, ldr, k, r, c->Gam, KM, st);
-    // extend the Cholesky factor of Gamma
-    sm_copy(c->Gam + (size_t)k * KM, KM, k, r, c->Bs, KM, st);
-    sm_trsv('N', c->L, KM, k, c->Bs, KM, r, st);
-    sm_copy(c->Gam + (size_t)k * KM + k, KM, r, r, c->Dm, r, st);
-    sm_gemm('C', 'N', r, r, k, MONE, c->Bs, KM, c->Bs, KM, ONE, c->Dm, r, st);
-    sm_hermitize(c->Dm, r, r, st);
-    sm_chol(c->Dm, r, r, c->L22, r, TOL_GAM, 1, c->dead_dev, c->status_dev, 0, st);
-    ::lrei::count_launch(); store_lrows_kernel<<<8, 256, 0, st>>>(c->Bs, KM, c->L22, r, k, c->dead_dev, c->L, KM, 0,
-                                                                       nullptr);
+    extend_frame(c, k, false, nullptr, nullptr, 0);
     // the frame of Q_0..Q_{l+1} is complete: stage l can run
     LREI_CUDA_TRY(cudaEventRecord(c->ev_kry[l], st));
     LREI_CUDA_TRY(cudaStreamWaitEvent(st2, c->ev_kry[l], 0));
@@ -993,9 +992,7 @@ int enqueue_rk_step(lrei_ctx *c, int scheme) {
   LREI_CUDA_TRY(cudaEventRecord(c->ev_join, st2));
   LREI_CUDA_TRY(cudaStreamWaitEvent(st, c->ev_join, 0));
   // V_{k+1} = Qbar Yfin = Q (L^{-H} Yfin), formed in place over Q_0 = V
-  sm_copy(c->yfin, KM, K, r, c->Yc, KM, st);
-  sm_trsv('C', c->L, KM, K, c->Yc, KM, r, st);
-  sm_copy(c->Yc, KM, K, r, c->coefQ, K, st);
+  sm_gemm('C', 'N', K, r, K, ONE, c->Li, KM, c->yfin, KM, ZERO, c->coefQ, K, st);
   TSArgs cmb{};
   cmb.nq = s + 1;
   cmb.gram_left = 0;
@@ -1148,13 +1145,11 @@ int orth_block(lrei_ctx *c, int i, const void *src, void *const *qb, zd *R) {
   a.mode = 0;
   int rc = ts_pass(c, a);
   if (rc) return rc;
-  // C = Gamma^{-1} P; Q_i = raw_i - Q C
-  sm_copy(red, ldr, k, r, c->Cc, KM, st);
-  sm_trsv('N', c->L, KM, k, c->Cc, KM, r, st);
-  sm_trsv('C', c->L, KM, k, c->Cc, KM, r, st);
+  // C = Gamma^{-1} P = L^{-H} L^{-1} P; Q_i = raw_i - Q C
+  sm_gemm('N', 'N', k, r, k, ONE, c->Li, KM, red, ldr, ZERO, c->Cc, KM, st);
+  sm_gemm('C', 'N', k, r, k, ONE, c->Li, KM, c->Cc, KM, ZERO, R + (size_t)i * r * KM, KM, st);
+  sm_gemm('C', 'N', k, r, k, MONE, c->Li, KM, c->Cc, KM, ZERO, c->coefQ, k, st);
   sm_set_identity(c->Ainv, r, r, r, st);
-  sm_gemm('N', 'N', k, r, r, MONE, c->Cc, KM, c->Ainv, r, ZERO, c->coefQ, k, st);
-  sm_copy(c->Cc, KM, k, r, R + (size_t)i * r * KM, KM, st);
   sm_set_identity(R + (size_t)i * r * KM + k, KM, r, r, st);
   TSArgs b = a;
   b.mode = 1;
@@ -1162,16 +1157,8 @@ int orth_block(lrei_ctx *c, int i, const void *src, void *const *qb, zd *R) {
   b.coefS = c->Ainv;
   b.coefQ = c->coefQ;
   if ((rc = ts_pass(c, b))) return rc;
-  sm_store_gram_cols(red, ldr, k, r, c->Gam, KM, st);
   // extend the Cholesky factor of Gamma: pivots judged against each column's own squared norm
-  sm_copy(c->Gam + (size_t)k * KM, KM, k, r, c->Bs, KM, st);
-  sm_trsv('N', c->L, KM, k, c->Bs, KM, r, st);
-  sm_copy(c->Gam + (size_t)k * KM + k, KM, r, r, c->Dm, r, st);
-  sm_gemm('C', 'N', r, r, k, MONE, c->Bs, KM, c->Bs, KM, ONE, c->Dm, r, st);
-  sm_hermitize(c->Dm, r, r, st);
-  sm_chol(c->Dm, r, r, c->L22, r, TOL_GAM, 0, c->dead_dev, c->status_dev, 0, st, c->Gam + (size_t)k * KM + k, KM);
-  ::lrei::count_launch();
-  store_lrows_kernel<<<8, 256, 0, st>>>(c->Bs, KM, c->L22, r, k, c->dead_dev, c->L, KM, 1, c->dead_frame);
+  extend_frame(c, k, true, c->dead_frame, red + k, ldr);
   return LREI_OK;
 }
 
@@ -1195,6 +1182,7 @@ int enqueue_ab_step(lrei_ctx *c, int m) {
   sm_zero(c->Rraw, KM, K, K, st);
   sm_set_identity(c->Rraw, KM, r, r, st);
   LREI_CUDA_TRY(cudaMemsetAsync(c->dead_frame, 0, (size_t)K * sizeof(int), st));
+  start_inverse(c, st);
   for (int i = 1; i < nb; ++i) {
     if (i == 1) launch_hv(c->fp64, c->M, c->V, yk, c->N, r, c->nsm, st, c->status_dev);
     const int rc = orth_block(c, i, raw[i], qb, c->Rraw);
@@ -1207,13 +1195,11 @@ int enqueue_ab_step(lrei_ctx *c, int m) {
   zero_dead_rows_kernel<<<8, 256, 0, st>>>(c->Bbar, KM, K, K, c->dead_frame);
   for (int l = 0; l < m; ++l) {
     // the state of step k-l is V_l orthonormalised: vbar = v Lv^{-H}, H vbar = y Lv^{-H}
-    sm_copy(c->Bbar + (size_t)(2 * l) * r * KM, KM, K, r, c->ys[l], KM, st);
-    sm_copy(c->Bbar + (size_t)(2 * l + 1) * r * KM, KM, K, r, c->tys[l], KM, st);
-    sm_gemm('C', 'N', r, r, K, ONE, c->ys[l], KM, c->ys[l], KM, ZERO, c->G, r, st);
-    sm_hermitize(c->G, r, r, st);
-    sm_chol(c->G, r, r, c->Lr, r, 0.0, 0, nullptr, nullptr, 0, st);
-    sm_rtrsm_lh_ws(c->ys[l], KM, K, c->Lr, r, r, c->Ainv, c->Uf, st);
-    sm_rtrsm_lh_ws(c->tys[l], KM, K, c->Lr, r, r, c->Ainv, c->Uf, st);
+    const zd *vb = c->Bbar + (size_t)(2 * l) * r * KM, *yb = vb + (size_t)r * KM;
+    sm_gemm_herm('C', 'N', r, K, ONE, vb, KM, vb, KM, ZERO, c->G, r, c->G, r, st);
+    sm_chol(c->G, r, r, nullptr, 0, 0.0, 0, nullptr, nullptr, 0, st, nullptr, 0, c->Ainv, r, 1);
+    sm_gemm('N', 'N', K, r, r, ONE, vb, KM, c->Ainv, r, ZERO, c->ys[l], KM, st);
+    sm_gemm('N', 'N', K, r, r, ONE, yb, KM, c->Ainv, r, ZERO, c->tys[l], KM, st);
     sm_gemm('C', 'N', r, r, K, ONE, c->ys[l], KM, c->tys[l], KM, ZERO, c->G, r, st);
     ::lrei::count_launch(); stage_xwz_kernel<<<r, 128, 2 * r * sizeof(zd), st>>>(c->G, r, c->lam0_dev, c->kappa, c->model, c->ys[l],
                                                          c->tys[l], K, KM, c->X11, c->zs[l], c->wsv[l],
@@ -1229,13 +1215,10 @@ int enqueue_ab_step(lrei_ctx *c, int m) {
     P.w[l] = c->wsv[l];
   }
   ::lrei::count_launch(); stage_factors_kernel<<<64, 256, 0, st>>>(P, C, c->lam0_dev, c->dt_dev, r, K, KM, c->Uf, c->Vf);
-  sm_gemm('N', 'C', K, K, r * (1 + 2 * m), ONE, c->Uf, KM, c->Vf, KM, ZERO, c->Mm, KM, st);
-  sm_hermitize(c->Mm, KM, K, st);
+  sm_gemm_herm('N', 'C', K, r * (1 + 2 * m), ONE, c->Uf, KM, c->Vf, KM, ZERO, c->Mm, KM, c->Mm, KM, st);
   sm_zero(c->yfin, KM, K, r, st);
   sm_eig_topr(c->Mm, KM, K, r, c->yfin, KM, c->mu_dev, c->eig_ws, c->status_dev, st, c->eig_sweeps);
-  sm_copy(c->yfin, KM, K, r, c->Yc, KM, st);
-  sm_trsv('C', c->L, KM, K, c->Yc, KM, r, st);
-  sm_copy(c->Yc, KM, K, r, c->coefQ, K, st);
+  sm_gemm('C', 'N', K, r, K, ONE, c->Li, KM, c->yfin, KM, ZERO, c->coefQ, K, st);
   TSArgs cmb{};
   cmb.nq = nb;
   cmb.gram_left = 0;
@@ -1568,6 +1551,7 @@ int lrei_create(int n, const lrei_bonds *J, const double B[3], double lambda, lr
   cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming);
   cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
   cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
+  cudaEventCreateWithFlags(&c->ev_inv, cudaEventDisableTiming);
   for (int i = 0; i < 4; ++i) cudaEventCreateWithFlags(&c->ev_kry[i], cudaEventDisableTiming);
   c->nsm_use = c->nsm;
   // the complex64 N-length passes of the RK step leave one SM in 32 to the stage algebra running
@@ -1599,10 +1583,10 @@ int lrei_create(int n, const lrei_bonds *J, const double B[3], double lambda, lr
   if ((rc = dalloc_t(c, &c->rdm_out, (size_t)34 * LREI_RDM_MAX_PAIRS * sizeof(double)))) return fail(rc);
   if ((rc = dalloc_t(c, &c->red, (size_t)(MAXB + 1) * R * R * 2 * sizeof(double)))) return fail(rc);
   if ((rc = dalloc(c, &c->coef_scratch, (size_t)(MAXB + 1) * MAX_R * MAX_R * zs))) return fail(rc);
-  zd **kk[] = {&c->Gam, &c->L, &c->Chat, &c->Tbar, &c->Xh, &c->Mm};
+  zd **kk[] = {&c->Gam, &c->L, &c->Li, &c->Chat, &c->Tbar, &c->Mm};
   for (auto p : kk)
     if ((rc = dalloc_t(c, p, (size_t)KM * KM * zs))) return fail(rc);
-  zd **kr[] = {&c->Cc, &c->coefQ, &c->Bs, &c->Yc, &c->ts, &c->yfin};
+  zd **kr[] = {&c->Cc, &c->coefQ, &c->Bs, &c->Yc, &c->Tr, &c->ts, &c->yfin};
   for (auto p : kr)
     if ((rc = dalloc_t(c, p, (size_t)KM * R * zs))) return fail(rc);
   for (int i = 0; i < 5; ++i)
@@ -1644,6 +1628,7 @@ int lrei_destroy(lrei_ctx *c) {
   if (c->ev_out) cudaEventDestroy(c->ev_out);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->ev_inv) cudaEventDestroy(c->ev_inv);
   for (int i = 0; i < 4; ++i)
     if (c->ev_kry[i]) cudaEventDestroy(c->ev_kry[i]);
   if (c->st2) cudaStreamDestroy(c->st2);
@@ -1672,6 +1657,7 @@ int lrei_set_state(lrei_ctx *c, const void *V_dev, int r, int ld, int dtype, con
   LREI_CUDA_TRY(cudaMemsetAsync(c->status_dev, 0, sizeof(int), c->st));
   LREI_CUDA_TRY(cudaMemsetAsync(c->L, 0, (size_t)KM * KM * sizeof(zd), c->st));
   LREI_CUDA_TRY(cudaMemsetAsync(c->Gam, 0, (size_t)KM * KM * sizeof(zd), c->st));
+  LREI_CUDA_TRY(cudaMemsetAsync(c->Chat, 0, (size_t)KM * KM * sizeof(zd), c->st));   // its zero blocks depend on r
   launch_convert(V_dev, dtype == LREI_C64, ld, c->V, c->fp64, c->N, r, c->st);
   launch_check_finite(c->fp64, c->V, c->N, r, c->status_dev, c->st);
   // R^H R = V^*V (Cholesky), rho_0 = Q (R Lambda R^H) Q^*, Q = V R^{-1}
@@ -2220,6 +2206,7 @@ int lrei_truncate_rank(lrei_ctx *c, double tol_r, int *r_out, double *dropped_ou
   int rc = ts_pass(c, a);
   if (!rc) {
     LREI_CUDA_TRY(cudaMemsetAsync(c->L, 0, (size_t)c->KM * c->KM * sizeof(zd), c->st));
+    LREI_CUDA_TRY(cudaMemsetAsync(c->Chat, 0, (size_t)c->KM * c->KM * sizeof(zd), c->st));
     set_gamma00(c);
   }
   if (c->ab_alloc) ab_clear(c);
@@ -2323,6 +2310,7 @@ int lrei_checkpoint_load(lrei_ctx *c, const void *buf, long long bytes) {
   p += r * sizeof(double);
   LREI_CUDA_TRY(cudaMemsetAsync(c->Gam, 0, (size_t)KM * KM * sizeof(zd), c->st));
   LREI_CUDA_TRY(cudaMemsetAsync(c->L, 0, (size_t)KM * KM * sizeof(zd), c->st));
+  LREI_CUDA_TRY(cudaMemsetAsync(c->Chat, 0, (size_t)KM * KM * sizeof(zd), c->st));
   LREI_CUDA_TRY(cudaMemcpy2DAsync(c->Gam, KM * sizeof(zd), p, r * sizeof(zd), r * sizeof(zd), r, cudaMemcpyHostToDevice, c->st));
   p += (size_t)r * r * sizeof(zd);
   LREI_CUDA_TRY(cudaMemcpy2DAsync(c->L, KM * sizeof(zd), p, r * sizeof(zd), r * sizeof(zd), r, cudaMemcpyHostToDevice, c->st));

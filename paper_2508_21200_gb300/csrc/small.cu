@@ -40,11 +40,22 @@ __device__ __forceinline__ zd opget(char op, const zd *A, int ld, int i, int p) 
 // chain), so a sum of K terms by one thread is a chain of 4 K x 64 cycles and by LN lanes of 4 K / LN + 2 log2 LN.
 template <int LN>
 __global__ void __launch_bounds__(128) gemm_kernel(char opA, char opB, int M, int N, int K, zd alpha, const zd *__restrict__ A,
-                                                   int lda, const zd *__restrict__ B, int ldb, zd beta, zd *__restrict__ C,
-                                                   int ldc) {
+                                                   int lda, const zd *__restrict__ B, int ldb, zd beta, const zd *Cin,
+                                                   int ldin, zd *C, int ldc, int herm) {
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) / LN, lane = threadIdx.x % LN;
-  const bool in = w < M * N;
-  const int i = in ? w % M : 0, j = in ? w / M : 0;
+  int i, j;
+  bool in;
+  if (herm) {   // the upper triangle (i <= j) and its mirror; column j holds the outputs j (j + 1) / 2 + i
+    in = w < M * (M + 1) / 2;
+    j = in ? (int)((sqrtf(8.f * (float)w + 1.f) - 1.f) * 0.5f) : 0;
+    while ((j + 1) * (j + 2) / 2 <= w && in) ++j;
+    while (j * (j + 1) / 2 > w) --j;
+    i = in ? w - j * (j + 1) / 2 : 0;
+  } else {
+    in = w < M * N;
+    i = in ? w % M : 0;
+    j = in ? w / M : 0;
+  }
   zd s = mk<double>(0, 0);
   for (int p = lane; p < K; p += LN) fma_(s, opget(opA, A, lda, i, p), opget(opB, B, ldb, p, j));
 #pragma unroll
@@ -54,20 +65,22 @@ __global__ void __launch_bounds__(128) gemm_kernel(char opA, char opB, int M, in
   }
   if (in && lane == 0) {
     zd c = alpha * s;
-    if (beta.re != 0.0 || beta.im != 0.0) c = c + beta * C[(size_t)j * ldc + i];
+    if (beta.re != 0.0 || beta.im != 0.0) c = c + beta * Cin[(size_t)j * ldin + i];
+    if (herm && i == j) c.im = 0.0;
     C[(size_t)j * ldc + i] = c;
+    if (herm && i != j) C[(size_t)i * ldc + j] = conj(c);
   }
 }
 
 // Lanes per output: the least of the longest chain (its FP64 instructions at 64 cycles) and the SMs' throughput (one
 // FP64 warp instruction in 19 cycles and SM, over 152 SMs).  Measured over an RK4 step at n = 16, r = 8 (K = 8..72):
 // 8.7 us a launch with one thread per output, 4.3 with the lanes chosen here; the step 1.58 ms before, 1.40 after.
-static int gemm_lanes(int M, int N, int K) {
+static int gemm_lanes(double outputs, int K) {
   int best = 4;
   double cost = 1e300;
   for (int ln = 4, lg = 2; ln <= 32; ln *= 2, ++lg) {
     const double instr = 4.0 * ((K + ln - 1) / ln) + 2.0 * lg + 4.0;
-    const double warps = (double)M * N * ln / 32.0;
+    const double warps = outputs * ln / 32.0;
     const double c = std::max(64.0 * instr, warps * instr * 19.0 / 152.0);
     if (c < cost) {
       cost = c;
@@ -77,17 +90,30 @@ static int gemm_lanes(int M, int N, int K) {
   return best;
 }
 
-void sm_gemm(char opA, char opB, int M, int N, int K, zd alpha, const zd *A, int lda, const zd *B, int ldb, zd beta,
-             zd *C, int ldc, cudaStream_t st) {
+static void gemm_launch(char opA, char opB, int M, int N, int K, zd alpha, const zd *A, int lda, const zd *B, int ldb,
+                        zd beta, const zd *Cin, int ldin, zd *C, int ldc, int herm, cudaStream_t st) {
   if (M <= 0 || N <= 0) return;
-  const int ln = gemm_lanes(M, N, K);
-  const int grid = (int)(((long long)M * N * ln + 127) / 128);
+  const int outputs = herm ? M * (M + 1) / 2 : M * N;
+  const int ln = gemm_lanes(outputs, K);
+  const int grid = (int)(((long long)outputs * ln + 127) / 128);
   ::lrei::count_launch();
-  auto go = [&](auto kern) { kern<<<grid, 128, 0, st>>>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); };
+  auto go = [&](auto kern) {
+    kern<<<grid, 128, 0, st>>>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, Cin, ldin, C, ldc, herm);
+  };
   if (ln == 4) go(gemm_kernel<4>);
   else if (ln == 8) go(gemm_kernel<8>);
   else if (ln == 16) go(gemm_kernel<16>);
   else go(gemm_kernel<32>);
+}
+
+void sm_gemm(char opA, char opB, int M, int N, int K, zd alpha, const zd *A, int lda, const zd *B, int ldb, zd beta,
+             zd *C, int ldc, cudaStream_t st) {
+  gemm_launch(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, C, ldc, 0, st);
+}
+
+void sm_gemm_herm(char opA, char opB, int M, int K, zd alpha, const zd *A, int lda, const zd *B, int ldb, zd beta,
+                  const zd *Cin, int ldin, zd *C, int ldc, cudaStream_t st) {
+  gemm_launch(opA, opB, M, M, K, alpha, A, lda, B, ldb, beta, Cin, ldin, C, ldc, 1, st);
 }
 
 // ------------------------------------------------------- triangular solves
@@ -158,34 +184,31 @@ void sm_trsv(char op, const zd *L, int ldl, int k, zd *B, int ldb, int ncols, cu
   trsv_kernel<<<(ncols + 3) / 4, 128, bytes, st>>>(op, L, ldl, k, B, ldb, ncols);
 }
 
-// X <- X (L^H)^{-1}: the inverse (L^H)^{-1} is formed by triangular solves on the identity and
-// applied with one GEMM, so no FP64 dependency chain runs per row.  Needs a k x k scratch and a
-// copy of X (both from the caller's workspace).
-void sm_rtrsm_lh_ws(zd *X, int ldx, int nrows, const zd *L, int ldl, int k, zd *inv, zd *xcopy, cudaStream_t st) {
-  if (nrows <= 0) return;
-  sm_set_identity(inv, k, k, k, st);
-  sm_trsv('C', L, ldl, k, inv, k, k, st);                 // inv = (L^H)^{-1}
-  sm_copy(X, ldx, nrows, k, xcopy, nrows, st);
-  sm_gemm('N', 'N', nrows, k, k, mk<double>(1, 0), xcopy, nrows, inv, k, mk<double>(0, 0), X, ldx, st);
-}
-
 // ------------------------------------------------------------- Cholesky
-// Right-looking Cholesky A = L L^H of a Hermitian k x k matrix (k <= 64) in one CTA: after each
-// pivot the trailing matrix gets a rank-one update, one element per thread, so the dependency
-// chain is k steps of one fused multiply-add (FP64 latency, not dot products, sets the time).
-// Column j is dead when its pivot is below tol times a reference: the j-th diagonal entry of
-// `ref` when given (the squared norm of the raw column), else the largest diagonal entry of A.
-// A dead column gets L[j][j] = 1 and a zero sub-column (and, with zero_row, a zero row).
-__global__ void chol_kernel(const zd *__restrict__ A, int lda, int k, zd *__restrict__ Lout, int ldl, double tol,
-                            int zero_row, int *dead, int *status, int flag_rank, const zd *__restrict__ ref, int ldref) {
-  extern __shared__ zd Ls[];   // k x k, ld = k (lower part used)
-  __shared__ double maxdiag, piv;
-  __shared__ int isdead, ndead;
+// Cholesky A = L L^H of a Hermitian k x k matrix (k <= 64) and the inverse of L, in one CTA.  Gaussian elimination on
+// [A | I]: step j takes the multiple A_ij / A_jj of row j off every row i > j, one entry per thread (the entries of
+// the trailing lower triangle and of the inverse's columns c <= j), and the columns are scaled by A_jj^{-1/2} at the
+// end.  An FP64 instruction takes 64 cycles in a dependent chain (a division 445, a square root 690), so the chain of a
+// step is one division and one multiply-add group, with the square roots taken together at the end, and the inverse
+// rides along: k = 16 took 33 us with the square root in the chain, and 24 us more for each triangular solve.
+// Column j is dead when its pivot is below tol times a reference: the j-th diagonal entry of `ref` when given (the
+// squared norm of the raw column), else the largest diagonal entry of A.  A dead column gets L[j][j] = 1 and a zero
+// sub-column (and, with zero_row, a zero row).
+__global__ void __launch_bounds__(256) chol_kernel(const zd *__restrict__ A, int lda, int k, zd *__restrict__ Lout, int ldl,
+                                                   zd *__restrict__ Iout, int ldi, int inv_h, zd *__restrict__ Rc, int ldrc, double tol,
+                                                   int zero_row, int *dead, int *status, int flag_rank,
+                                                   const zd *__restrict__ ref, int ldref) {
+  extern __shared__ zd Ls[];   // k x k: A's lower triangle, then L before scaling; and k x k: the inverse before scaling
+  zd *X = Ls + (size_t)k * k;
+  __shared__ double maxdiag, rs[64], refs[64];
+  __shared__ int deads[64], ndead;
   const int t = threadIdx.x, nt = blockDim.x;
   for (int e = t; e < k * k; e += nt) {
     const int i = e % k, j = e / k;
     Ls[e] = (i >= j) ? A[(size_t)j * lda + i] : mk<double>(0, 0);
+    X[e] = mk<double>(i == j ? 1.0 : 0.0, 0);
   }
+  for (int i = t; i < k; i += nt) refs[i] = ref ? ref[(size_t)i * ldref + i].re : 0.0;
   if (t < 32) {
     double m = 0.0;
     for (int i = t; i < k; i += 32) m = fmax(m, A[(size_t)i * lda + i].re);
@@ -194,45 +217,73 @@ __global__ void chol_kernel(const zd *__restrict__ A, int lda, int k, zd *__rest
   }
   __syncthreads();
   for (int j = 0; j < k; ++j) {
+    const double piv = Ls[j * k + j].re, refj = ref ? refs[j] : maxdiag;
+    const bool dj = !(piv > tol * refj) || !isfinite(piv) || !(refj > 0.0);
     if (t == 0) {
-      piv = Ls[j * k + j].re;
-      const double refj = ref ? ref[(size_t)j * ldref + j].re : maxdiag;
-      isdead = !(piv > tol * refj) || !isfinite(piv) || !(refj > 0.0);
-      if (isdead) ndead++;
-      if (dead) dead[j] = isdead;
+      deads[j] = dj;
+      if (dj) ndead++;
     }
-    __syncthreads();
-    const double d = isdead ? 1.0 : sqrt(piv);
-    const double inv = 1.0 / d;
-    for (int i = j + t; i < k; i += nt) {
-      if (isdead) Ls[j * k + i] = (i == j) ? mk<double>(1, 0) : mk<double>(0, 0);
-      else Ls[j * k + i] = (i == j) ? mk<double>(d, 0) : mk<double>(Ls[j * k + i].re * inv, Ls[j * k + i].im * inv);
-    }
-    if (isdead && zero_row)
-      for (int m = t; m < j; m += nt) Ls[m * k + j] = mk<double>(0, 0);
-    __syncthreads();
-    if (!isdead) {
-      // trailing update: A[i][c] -= L[i][j] conj(L[c][j]) for j < c <= i
-      const int nrem = k - j - 1;
-      for (int e = t; e < nrem * nrem; e += nt) {
-        const int i = j + 1 + e % nrem, cc = j + 1 + e / nrem;
-        if (i >= cc) Ls[cc * k + i] = Ls[cc * k + i] - Ls[j * k + i] * conj(Ls[j * k + cc]);
+    const int nrem = k - j - 1, ntri = nrem * (nrem + 1) / 2;
+    if (!dj) {
+      const double inv = 1.0 / piv;
+      // entries 0 .. ntri - 1: the trailing triangle by rows (row a has a + 1 entries); then nrem x (j + 1) of X
+      for (int e = t; e < ntri + nrem * (j + 1); e += nt) {
+        int i, c;
+        zd *dst;
+        zd f;
+        if (e < ntri) {
+          int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+          while ((a + 1) * (a + 2) / 2 <= e) ++a;
+          while (a * (a + 1) / 2 > e) --a;
+          i = j + 1 + a;
+          c = j + 1 + e - a * (a + 1) / 2;
+          dst = Ls + c * k + i;
+          f = conj(Ls[j * k + c]);
+        } else {
+          const int x = e - ntri;
+          i = j + 1 + x % nrem;
+          c = x / nrem;
+          dst = X + c * k + i;
+          f = X[c * k + j];
+        }
+        const zd l = Ls[j * k + i];
+        *dst = *dst - mk<double>(l.re * inv, l.im * inv) * f;
       }
     }
     __syncthreads();
   }
+  for (int j = t; j < k; j += nt) rs[j] = deads[j] ? 1.0 : 1.0 / sqrt(Ls[j * k + j].re);
+  __syncthreads();
   for (int e = t; e < k * k; e += nt) {
     const int i = e % k, j = e / k;
-    Lout[(size_t)j * ldl + i] = (i >= j) ? Ls[e] : mk<double>(0, 0);
+    const bool row0 = zero_row && deads[i];   // a dead row without its part left of the diagonal
+    zd l = mk<double>(0, 0);
+    if (i > j) {
+      if (!deads[j] && !row0) l = mk<double>(Ls[e].re * rs[j], Ls[e].im * rs[j]);
+    } else if (i == j) {
+      l.re = deads[j] ? 1.0 : Ls[e].re * rs[j];
+    }
+    if (Lout) Lout[(size_t)j * ldl + i] = l;
+    if (Iout) {
+      zd x = mk<double>(0, 0);
+      if (i > j && !row0) x = mk<double>(X[e].re * rs[i], X[e].im * rs[i]);
+      else if (i == j) x.re = rs[i];
+      if (inv_h) Iout[(size_t)i * ldi + j] = conj(x);
+      else Iout[(size_t)j * ldi + i] = x;
+    }
+    // Rc = L^H with the rows of dead columns zeroed: entry (j, i)
+    if (Rc) Rc[(size_t)i * ldrc + j] = deads[j] ? mk<double>(0, 0) : conj(l);
   }
+  if (dead)
+    for (int j = t; j < k; j += nt) dead[j] = deads[j];
   if (t == 0 && ndead > 0 && flag_rank && status) atomicOr(status, ST_RANK);
 }
 
 void sm_chol(const zd *A, int lda, int k, zd *L, int ldl, double tol, int zero_row, int *dead, int *status,
-             int flag_rank, cudaStream_t st, const zd *ref, int ldref) {
+             int flag_rank, cudaStream_t st, const zd *ref, int ldref, zd *Linv, int ldi, int inv_h, zd *Rc, int ldrc) {
   ::lrei::count_launch();
-  chol_kernel<<<1, 256, (size_t)k * k * sizeof(zd), st>>>(A, lda, k, L, ldl, tol, zero_row, dead, status, flag_rank,
-                                                          ref, ldref);
+  chol_kernel<<<1, 256, 2 * (size_t)k * k * sizeof(zd), st>>>(A, lda, k, L, ldl, Linv, ldi, inv_h, Rc, ldrc, tol, zero_row, dead,
+                                                              status, flag_rank, ref, ldref);
 }
 
 // --------------------------------------------------------------- Jacobi
@@ -619,7 +670,6 @@ __global__ void copy_kernel(const zd *A, int lda, int M, int N, zd *B, int ldb, 
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < M * N; e += gridDim.x * blockDim.x) {
     const int i = e % M, j = e / M;
     if (mode == 0) B[(size_t)j * ldb + i] = A[(size_t)j * lda + i];
-    else if (mode == 1) B[(size_t)i * ldb + j] = conj(A[(size_t)j * lda + i]);   // B = A^H (N x M)
     else if (mode == 2) B[(size_t)j * ldb + i] = mk<double>(0, 0);
     else B[(size_t)j * ldb + i] = mk<double>(i == j ? 1 : 0, 0);
   }
@@ -627,9 +677,6 @@ __global__ void copy_kernel(const zd *A, int lda, int M, int N, zd *B, int ldb, 
 static int grid_for(long long n) { long long g = (n + 255) / 256; return (int)(g < 1 ? 1 : (g > 1024 ? 1024 : g)); }
 void sm_copy(const zd *A, int lda, int M, int N, zd *B, int ldb, cudaStream_t st) {
   ::lrei::count_launch(); copy_kernel<<<grid_for((long long)M * N), 256, 0, st>>>(A, lda, M, N, B, ldb, 0);
-}
-void sm_conj_transpose(const zd *A, int lda, int M, int N, zd *B, int ldb, cudaStream_t st) {
-  ::lrei::count_launch(); copy_kernel<<<grid_for((long long)M * N), 256, 0, st>>>(A, lda, M, N, B, ldb, 1);
 }
 void sm_zero(zd *A, int lda, int M, int N, cudaStream_t st) {
   ::lrei::count_launch(); copy_kernel<<<grid_for((long long)M * N), 256, 0, st>>>(nullptr, 0, M, N, A, lda, 2);
@@ -661,26 +708,16 @@ void sm_scale_cols(zd *A, int lda, int M, int N, double s, cudaStream_t st) {
   ::lrei::count_launch(); scale_kernel<<<grid_for((long long)M * N), 256, 0, st>>>(A, lda, M, N, s);
 }
 
-// Columns k..k+r-1 of the Hermitian Gram G from the measured block R ((k + r) x r) and their
-// mirror rows.  Inside the new r x r diagonal block only R's upper triangle is used (the lower one
-// is its conjugate), so every entry of G has exactly one writer: R's two triangles differ in the
-// last bit, and two threads storing both into one entry would make the result depend on which
-// store lands last.
-__global__ void store_gram_cols_kernel(const zd *R, int ldr, int k, int r, zd *G, int ldg) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < (k + r) * r; e += gridDim.x * blockDim.x) {
-    const int i = e % (k + r), j = e / (k + r);
-    if (i > k + j) continue;   // below the diagonal of the new block: written as the mirror of (k + j, i)
-    const zd v = R[(size_t)j * ldr + i];
-    if (i == k + j) {
-      G[(size_t)(k + j) * ldg + i] = mk<double>(v.re, 0);
-    } else {
-      G[(size_t)(k + j) * ldg + i] = v;
-      G[(size_t)i * ldg + (k + j)] = conj(v);
-    }
+// B = (A + A^H)/2, k x k.
+__global__ void herm_copy_kernel(const zd *__restrict__ A, int lda, int k, zd *__restrict__ B, int ldb) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < k * k; e += gridDim.x * blockDim.x) {
+    const int i = e % k, j = e / k;
+    const zd a = A[(size_t)j * lda + i], b = A[(size_t)i * lda + j];
+    B[(size_t)j * ldb + i] = mk<double>(0.5 * (a.re + b.re), i == j ? 0.0 : 0.5 * (a.im - b.im));
   }
 }
-void sm_store_gram_cols(const zd *R, int ldr, int k, int r, zd *G, int ldg, cudaStream_t st) {
-  ::lrei::count_launch(); store_gram_cols_kernel<<<grid_for((long long)(k + r) * r), 256, 0, st>>>(R, ldr, k, r, G, ldg);
+void sm_herm_copy(const zd *A, int lda, int k, zd *B, int ldb, cudaStream_t st) {
+  ::lrei::count_launch(); herm_copy_kernel<<<grid_for((long long)k * k), 256, 0, st>>>(A, lda, k, B, ldb);
 }
 
 }  // namespace lrei
@@ -689,6 +726,7 @@ namespace lrei {
 int sm_init() {
   const int lim = 210 * 1024;
   cudaFuncSetAttribute(trsv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   cudaError_t a = cudaFuncSetAttribute(jacobi_kernel<double, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   cudaError_t b = cudaFuncSetAttribute(jacobi_kernel<float, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   cudaError_t c = cudaFuncSetAttribute(newton_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
