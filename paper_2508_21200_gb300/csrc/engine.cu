@@ -1674,7 +1674,7 @@ int lrei_set_state(lrei_ctx *c, const void *V_dev, int r, int ld, int dtype, con
   sm_chol(red, r, r, c->L22, r, 1e-24, 1, c->dead_dev, c->status_dev, 1, c->st);
   LREI_CUDA_TRY(cudaMemcpyAsync(c->lam0_dev, lam_in.data(), r * sizeof(double), cudaMemcpyHostToDevice, c->st));
   ::lrei::count_launch(); lhl_kernel<<<1, 256, 0, c->st>>>(c->L22, r, c->lam0_dev, c->Dm);
-  sm_jacobi(true, c->Dm, r, r, c->Lr, r, c->mu_dev, c->eig_ws, 60, 1e-15, c->status_dev, c->st);
+  sm_jacobi64(c->Dm, r, r, c->Lr, r, c->mu_dev, 60, 1e-15, c->status_dev, c->st);
   // coefficients R^{-1} E = L^{-H} E
   sm_copy(c->Lr, r, r, r, c->coefQ, r, c->st);
   sm_trsv('C', c->L22, r, r, c->coefQ, r, r, c->st);

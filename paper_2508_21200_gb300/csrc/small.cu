@@ -30,6 +30,20 @@ __device__ __forceinline__ zd warp_sum(zd v) {
   return v;
 }
 
+// State of an eigensolve on the device: [META_ROUNDS] rounds of its FP32 Jacobi, [META_D + p - 1] largest component of the p-th
+// Newton correction (float bits).
+enum { META_ROUNDS = 0, META_D = 1, META_INTS = 8 };
+constexpr int NEWTON_PASSES = 4;
+// Whether the corrections up to pass p (1-based) leave nothing to correct: they shrink by a constant factor per pass
+// (the FP32 error of Ur), so after pass q about D_q^2 / D_{q-1} is left.
+__device__ __forceinline__ bool newton_done(const int *meta, int p) {
+  for (int q = 2; q <= p; ++q) {
+    const float d = __int_as_float(meta[META_D + q - 1]);
+    if (d * d <= 1e-17f * __int_as_float(meta[META_D + q - 2])) return true;
+  }
+  return false;
+}
+
 // ------------------------------------------------------------------ GEMM
 __device__ __forceinline__ zd opget(char op, const zd *A, int ld, int i, int p) {
   return op == 'N' ? A[(size_t)p * ld + i] : conj(A[(size_t)i * ld + p]);
@@ -41,7 +55,8 @@ __device__ __forceinline__ zd opget(char op, const zd *A, int ld, int i, int p) 
 template <int LN>
 __global__ void __launch_bounds__(128) gemm_kernel(char opA, char opB, int M, int N, int K, zd alpha, const zd *__restrict__ A,
                                                    int lda, const zd *__restrict__ B, int ldb, zd beta, const zd *Cin,
-                                                   int ldin, zd *C, int ldc, int herm) {
+                                                   int ldin, zd *C, int ldc, int herm, const int *meta, int pass) {
+  if (meta && newton_done(meta, pass)) return;
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) / LN, lane = threadIdx.x % LN;
   int i, j;
   bool in;
@@ -91,14 +106,15 @@ static int gemm_lanes(double outputs, int K) {
 }
 
 static void gemm_launch(char opA, char opB, int M, int N, int K, zd alpha, const zd *A, int lda, const zd *B, int ldb,
-                        zd beta, const zd *Cin, int ldin, zd *C, int ldc, int herm, cudaStream_t st) {
+                        zd beta, const zd *Cin, int ldin, zd *C, int ldc, int herm, cudaStream_t st,
+                        const int *meta = nullptr, int pass = 0) {
   if (M <= 0 || N <= 0) return;
   const int outputs = herm ? M * (M + 1) / 2 : M * N;
   const int ln = gemm_lanes(outputs, K);
   const int grid = (int)(((long long)outputs * ln + 127) / 128);
   ::lrei::count_launch();
   auto go = [&](auto kern) {
-    kern<<<grid, 128, 0, st>>>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, Cin, ldin, C, ldc, herm);
+    kern<<<grid, 128, 0, st>>>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, Cin, ldin, C, ldc, herm, meta, pass);
   };
   if (ln == 4) go(gemm_kernel<4>);
   else if (ln == 8) go(gemm_kernel<8>);
@@ -287,229 +303,408 @@ void sm_chol(const zd *A, int lda, int k, zd *L, int ldl, double tol, int zero_r
 }
 
 // --------------------------------------------------------------- Jacobi
-template <typename T>
-struct Rot {
-  T c;
-  cx<T> s;
-  int p, q;
-};
+// Cyclic Jacobi of a Hermitian matrix in one CTA, round-robin pairs (circle method: position 0 stays, positions
+// 1 .. kp-1 rotate by one per round).  A rotation J = [[c, s], [-conj(s), c]] on (p, q) annihilates A_pq; a round applies the kp / 2
+// disjoint rotations of its pairs as A <- J^H A J on 2 x 2 blocks of pairs.  Only the upper triangle is kept
+// (an element below the diagonal is its mirror's conjugate), so a round touches each pair of pairs once.
+__device__ __forceinline__ void round_pair(int pos, int round, int kp, int *p, int *q) {
+  auto player = [&](int x) {
+    if (x == 0) return 0;
+    int y = x - 1 + round;
+    if (y >= kp - 1) y -= kp - 1;
+    return y + 1;
+  };
+  const int a = player(pos), b = player(kp - 1 - pos);
+  *p = min(a, b);
+  *q = max(a, b);
+}
+template <typename T> __device__ __forceinline__ cx<T> tri_get(const cx<T> *A, int ld, int i, int j) {
+  return i <= j ? A[j * ld + i] : conj(A[i * ld + j]);
+}
+template <typename T> __device__ __forceinline__ void tri_put(cx<T> *A, int ld, int i, int j, cx<T> v) {
+  if (i <= j) A[j * ld + i] = v;
+  else A[i * ld + j] = conj(v);
+}
+// item e of the pairs of positions a < b, e = b (b - 1) / 2 + a; with diag = 1 of a <= b, e = b (b + 1) / 2 + a
+__device__ __forceinline__ void tri_item(int e, int *a, int *b, int diag = 0) {
+  int y = (int)((sqrtf(8.f * (float)e + 1.f) + 1.f) * 0.5f);
+  while (y * (y + 1) / 2 <= e) ++y;
+  while (y * (y - 1) / 2 > e) --y;
+  *b = y - diag;
+  *a = e - y * (y - 1) / 2;
+}
 
-// One CTA.  A (k x k Hermitian, FP64 input) -> eigenpairs in working precision T.
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT) jacobi_kernel(const zd *__restrict__ Ain, int lda, int k, zd *__restrict__ Uout,
-                                                     int ldu, double *__restrict__ wout, cx<T> *Ug, int max_sweeps,
-                                                     double tol, int *status, cx<float> *__restrict__ Uf, int nout) {
+constexpr int J32_ITEMS = 8;        // pairs of pairs per thread: enough for k = 162, where A fills the shared memory
+constexpr int J32_SWEEPS = 12;
+constexpr int J32_KMAX = 162;
+
+// FP32.  A round is latency: the angle, the blocks, two barriers.  The eigenvectors are not accumulated here: the
+// rotations (c, s, p | q << 16) of every round go to rots, and replay_kernel applies them to the rows of U on many SMs.
+// The odd leading dimension keeps mirrored (row-wise) accesses free of bank conflicts.
+// order[i]: rank of diagonal entry i in decreasing order.
+__global__ void __launch_bounds__(512) jacobi32_kernel(const zd *__restrict__ Ain, int lda, int k, double *__restrict__ wout,
+                                                       int *__restrict__ order, float4 *__restrict__ rots,
+                                                       int *__restrict__ meta, float tol) {
   extern __shared__ __align__(16) unsigned char sm[];
-  const int kp = k + (k & 1);
-  const int np = kp / 2;
-  cx<T> *A = reinterpret_cast<cx<T> *>(sm);
-  Rot<T> *rot = reinterpret_cast<Rot<T> *>(A + (size_t)kp * kp);
-  cx<T> *U = Ug ? Ug : reinterpret_cast<cx<T> *>(rot + np);
-  __shared__ double red[32];
-  __shared__ int done;
-  const int t = threadIdx.x, nt = blockDim.x;
+  const int kp = k + (k & 1), ld = kp + 1, np = kp / 2, nitem = np * (np - 1) / 2;
+  float4 *rot = reinterpret_cast<float4 *>(sm);
+  cx<float> *A = reinterpret_cast<cx<float> *>(rot + np);    // upper triangle
+  __shared__ float red[2][16];
+  const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wp = t >> 5;
   for (int e = t; e < kp * kp; e += nt) {
     const int i = e % kp, j = e / kp;
-    if (i < k && j < k) {
-      zd v = Ain[(size_t)j * lda + i];
-      A[e] = mk<T>((T)v.re, (T)v.im);
-    } else {
-      A[e] = mk<T>(0, 0);
-    }
-    U[e] = mk<T>(i == j ? 1 : 0, 0);
+    cx<float> v = mk<float>(0.f, 0.f);
+    if (i < k && j < k && i <= j) v = cvt<float>(Ain[(size_t)j * lda + i]);
+    A[j * ld + i] = v;
   }
+  int item[J32_ITEMS];
+#pragma unroll
+  for (int x = 0; x < J32_ITEMS; ++x) {
+    int a = 0, b = 0;
+    if (t + x * nt < nitem) tri_item(t + x * nt, &a, &b);
+    item[x] = a | b << 16;
+  }
+  if (t < META_INTS) meta[t] = 0;
   __syncthreads();
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    // convergence test: off-diagonal vs total Frobenius norm (summed in T per thread: the FP32
-    // solver's test needs no FP64 arithmetic, which is slow on this part)
-    T offt = 0, tott = 0;
+  int rounds = 0, sweeps = 0;
+  for (; sweeps < J32_SWEEPS; ++sweeps) {
+    // convergence test: off-diagonal vs total Frobenius norm
+    float off = 0.f, tot = 0.f;
     for (int e = t; e < kp * kp; e += nt) {
       const int i = e % kp, j = e / kp;
-      const T v = norm2(A[e]);
-      tott += v;
-      if (i != j) offt += v;
+      if (i > j) continue;
+      const float v = norm2(A[j * ld + i]);
+      if (i == j) tot += v;
+      else off += 2.f * v;
     }
-    double off = (double)offt, tot = (double)tott;
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       off += __shfl_xor_sync(0xffffffffu, off, o);
       tot += __shfl_xor_sync(0xffffffffu, tot, o);
     }
-    if ((t & 31) == 0) red[t >> 5] = off;
+    if (lane == 0) { red[0][wp] = off; red[1][wp] = tot; }
     __syncthreads();
-    if (t == 0) {
-      double s = 0.0;
-      for (int w = 0; w < (nt + 31) / 32; ++w) s += red[w];
-      off = s;
-    }
-    __syncthreads();
-    if ((t & 31) == 0) red[t >> 5] = tot;
-    __syncthreads();
-    if (t == 0) {
-      double s = 0.0;
-      for (int w = 0; w < (nt + 31) / 32; ++w) s += red[w];
-      done = (off <= tol * tol * s) || !(s == s);
-    }
-    __syncthreads();
-    if (done) break;
-    for (int round = 0; round < kp - 1; ++round) {
+    off = tot = 0.f;
+    for (int w = 0; w < nt / 32; ++w) { off += red[0][w]; tot += red[1][w]; }
+    tot += off;
+    if (off <= tol * tol * tot || !(tot == tot)) break;
+    for (int round = 0; round < kp - 1; ++round, ++rounds) {
       for (int pi = t; pi < np; pi += nt) {
-        // circle-method tournament: position 0 fixed, positions 1..kp-1 rotate
-        auto player = [&](int pos) { return pos == 0 ? 0 : 1 + ((pos - 1 + round) % (kp - 1)); };
-        int p = player(pi), q = player(kp - 1 - pi);
-        if (p > q) { const int tmp = p; p = q; q = tmp; }
-        const cx<T> b = A[(size_t)q * kp + p];
-        const T ab = sqrt(b.re * b.re + b.im * b.im);
-        const T a = A[(size_t)p * kp + p].re, d = A[(size_t)q * kp + q].re;
-        Rot<T> R;
-        R.p = p;
-        R.q = q;
-        const T small = (sizeof(T) == 4) ? (T)1e-30 : (T)1e-280;
-        if (ab <= small) {
-          R.c = 1;
-          R.s = mk<T>(0, 0);
-        } else {
-          const T tau = (d - a) / (2 * ab);
-          T tt;
-          if (fabs((double)tau) > ((sizeof(T) == 4) ? 1e7 : 1e150)) tt = (T)0.5 / tau;
-          else tt = (tau >= 0 ? (T)1 : (T)-1) / (fabs(tau) + sqrt((T)1 + tau * tau));
-          const T c = (T)1 / sqrt((T)1 + tt * tt);
-          R.c = c;
-          R.s = mk<T>(tt * c * b.re / ab, tt * c * b.im / ab);
+        int p, q;
+        round_pair(pi, round, kp, &p, &q);
+        const cx<float> b = A[q * ld + p];
+        const float n2 = norm2(b), a = A[p * ld + p].re, d = A[q * ld + q].re;
+        float c = 1.f, f = 0.f;
+        if (n2 > 1e-37f) {   // tan = f |b| with f = sign(d - a) / (|h| + sqrt(h^2 + |b|^2)), h = (d - a) / 2
+          const float h = 0.5f * (d - a), g = fmaf(h, h, n2);
+          f = copysignf(__fdividef(1.f, fabsf(h) + g * rsqrtf(g)), h);
+          c = rsqrtf(fmaf(n2 * f, f, 1.f));
+          A[p * ld + p] = mk<float>(fmaf(-f, n2, a), 0.f);   // the pair's own block: A_pp - tan |b|, A_qq + tan |b|, 0
+          A[q * ld + q] = mk<float>(fmaf(f, n2, d), 0.f);
+          A[q * ld + p] = mk<float>(0.f, 0.f);
         }
+        const float4 R = make_float4(c, c * f * b.re, c * f * b.im, __int_as_float(p | q << 16));
         rot[pi] = R;
+        rots[(size_t)rounds * np + pi] = R;
       }
       __syncthreads();
-      // A <- J^H A J on 2x2 blocks (pairs a, b): every element is read and written once;
-      // U <- U J on the pairs' columns.  J = [[c, s], [-conj(s), c]] on (p, q).
-      for (int e = t; e < np * np + np * kp; e += nt) {
-        if (e < np * np) {
-          const Rot<T> Ra = rot[e % np], Rb = rot[e / np];
-          cx<T> *a0 = A + (size_t)Rb.p * kp, *a1 = A + (size_t)Rb.q * kp;
-          const cx<T> x00 = a0[Ra.p], x10 = a0[Ra.q], x01 = a1[Ra.p], x11 = a1[Ra.q];
-          // Y = X J_b
-          const cx<T> y00 = Rb.c * x00 - conj(Rb.s) * x01, y01 = Rb.s * x00 + Rb.c * x01;
-          const cx<T> y10 = Rb.c * x10 - conj(Rb.s) * x11, y11 = Rb.s * x10 + Rb.c * x11;
-          // X' = J_a^H Y
-          a0[Ra.p] = Ra.c * y00 - Ra.s * y10;
-          a1[Ra.p] = Ra.c * y01 - Ra.s * y11;
-          a0[Ra.q] = conj(Ra.s) * y00 + Ra.c * y10;
-          a1[Ra.q] = conj(Ra.s) * y01 + Ra.c * y11;
-        } else {
-          const int f = e - np * np;
-          const Rot<T> R = rot[f / kp];
-          const int i = f % kp;
-          if (R.s.re == 0 && R.s.im == 0) continue;
-          cx<T> *up = U + (size_t)R.p * kp, *uq = U + (size_t)R.q * kp;
-          const cx<T> ux = up[i], uy = uq[i];
-          up[i] = R.c * ux - conj(R.s) * uy;
-          uq[i] = R.s * ux + R.c * uy;
+#pragma unroll
+      for (int x = 0; x < J32_ITEMS; ++x)
+        if (t + x * nt < nitem) {
+          const float4 Ra = rot[item[x] & 0xffff], Rb = rot[item[x] >> 16];
+          const int pa = __float_as_int(Ra.w) & 0xffff, qa = __float_as_int(Ra.w) >> 16;
+          const int pb = __float_as_int(Rb.w) & 0xffff, qb = __float_as_int(Rb.w) >> 16;
+          const cx<float> sa = mk<float>(Ra.y, Ra.z), sb = mk<float>(Rb.y, Rb.z);
+          const cx<float> x00 = tri_get(A, ld, pa, pb), x10 = tri_get(A, ld, qa, pb), x01 = tri_get(A, ld, pa, qb),
+                          x11 = tri_get(A, ld, qa, qb);
+          const cx<float> y00 = Rb.x * x00 - conj(sb) * x01, y01 = sb * x00 + Rb.x * x01;    // Y = X J_b
+          const cx<float> y10 = Rb.x * x10 - conj(sb) * x11, y11 = sb * x10 + Rb.x * x11;
+          tri_put(A, ld, pa, pb, Ra.x * y00 - sa * y10);                                     // X' = J_a^H Y
+          tri_put(A, ld, pa, qb, Ra.x * y01 - sa * y11);
+          tri_put(A, ld, qa, pb, conj(sa) * y00 + Ra.x * y10);
+          tri_put(A, ld, qa, qb, conj(sa) * y01 + Ra.x * y11);
+        }
+      __syncthreads();
+    }
+  }
+  // eigenvalues and their order (decreasing, ties by index)
+  for (int i = t; i < k; i += nt) {
+    const float wi = A[i * ld + i].re;
+    int rank = 0;
+    for (int j = 0; j < k; ++j) {
+      const float wj = A[j * ld + j].re;
+      rank += (wj > wi) || (wj == wi && j < i);
+    }
+    wout[rank] = (double)wi;
+    order[i] = rank;
+  }
+  if (t == 0) {
+    meta[META_ROUNDS] = rounds;
+    atomicAdd(&g_jacobi_counters[0], 1ull);
+    atomicAdd(&g_jacobi_counters[1], (unsigned long long)sweeps);
+  }
+}
+
+// U = J_1 J_2 ... applied to the rows of the identity (a row sees every rotation, and no other row): one warp per row,
+// eight rows per CTA, the rotations of REPLAY rounds at a time through shared memory.  Writes U with its columns in
+// decreasing order of eigenvalue: all of them in FP32, the first nout also in FP64.
+constexpr int REPLAY = 16;
+__global__ void __launch_bounds__(256) replay_kernel(int k, const float4 *__restrict__ rots, const int *__restrict__ meta,
+                                                     const int *__restrict__ order, cx<float> *__restrict__ Uf,
+                                                     zd *__restrict__ Uout, int ldu, int nout) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const int kp = k + (k & 1), np = kp / 2;
+  float4 *R = reinterpret_cast<float4 *>(sm);                       // [REPLAY][np]
+  const int t = threadIdx.x, lane = t & 31, wp = t >> 5, row = blockIdx.x * 8 + wp;
+  cx<float> *u = reinterpret_cast<cx<float> *>(R + REPLAY * np) + wp * kp;
+  for (int i = lane; i < kp; i += 32) u[i] = mk<float>(i == row ? 1.f : 0.f, 0.f);
+  const int rounds = meta[0];
+  for (int r0 = 0; r0 < rounds; r0 += REPLAY) {
+    const int nr = min(REPLAY, rounds - r0);
+    __syncthreads();
+    for (int e = t; e < nr * np; e += 256) R[e] = rots[(size_t)r0 * np + e];
+    __syncthreads();
+    for (int rd = 0; rd < nr; ++rd) {
+      for (int pi = lane; pi < np; pi += 32) {
+        const float4 r = R[rd * np + pi];
+        const int p = __float_as_int(r.w) & 0xffff, q = __float_as_int(r.w) >> 16;
+        const cx<float> s = mk<float>(r.y, r.z), x = u[p], y = u[q];
+        u[p] = r.x * x - conj(s) * y;
+        u[q] = s * x + r.x * y;
+      }
+      __syncwarp();
+    }
+  }
+  if (row < k)
+    for (int i = lane; i < k; i += 32) {
+      const int rk = order[i];
+      Uf[(size_t)rk * k + row] = u[i];
+      if (rk < nout) Uout[(size_t)rk * ldu + row] = cvt<double>(u[i]);
+    }
+}
+
+static size_t j32_smem(int k) {
+  const int kp = k + (k & 1);
+  return (size_t)kp * (kp + 1) * sizeof(cx<float>) + (size_t)(kp / 2) * sizeof(float4);
+}
+static size_t replay_smem(int k) {
+  const int kp = k + (k & 1);
+  return (size_t)REPLAY * (kp / 2) * sizeof(float4) + (size_t)8 * kp * sizeof(cx<float>);
+}
+
+// Conversions by their bits (a conversion instruction runs at the FP64 rate): x truncated to FP32 (zero below
+// 2^-126; x is finite and below 2^128), and back (normal numbers and zero).
+__device__ __forceinline__ float f32_bits(double x) {
+  const int hi = __double2hiint(x), e = ((hi >> 20) & 0x7ff) - 896;
+  return e <= 0 ? 0.f : __int_as_float((hi & 0x80000000) | e << 23 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double f64_bits(float x) {
+  const int b = __float_as_int(x), e = (b >> 23) & 0xff;
+  return e == 0 ? 0.0 : __hiloint2double((b & 0x80000000) | (e + 896) << 20 | ((b >> 3) & 0xfffff), b << 29);
+}
+__device__ __forceinline__ double flip_if(double x, bool c) {
+  return __hiloint2double(__double2hiint(x) ^ (c ? 0x80000000 : 0), __double2loint(x));
+}
+
+// FP64, k <= 32, one CTA.  An FP64 instruction occupies a scheduler for 64 cycles, a division or square root for 7 to 11 of
+// these, so (a) the angle of a rotation is taken in FP32: it annihilates its entry to 1e-7 instead of 1e-16, which leaves the
+// number of sweeps as it is, and the rotation is made unitary in FP64, c = sqrt(1 - |s|^2) by two Newton steps from its
+// FP32 value; (b) one thread computes one real component (three multiply-adds for A J, three for J^H (A J), the
+// neighbours' components by shuffles), eight threads a 2 x 2 block.  A is scaled by a power of two to entries below
+// 2, so that FP32 has the range.  (One thread per block and FP64 angles: 55 us a call at k = 8.)
+__global__ void __launch_bounds__(512) jacobi64_kernel(const zd *__restrict__ Ain, int lda, int k, zd *__restrict__ Uout,
+                                                       int ldu, double *__restrict__ wout, int max_sweeps, double tol,
+                                                       int *status) {
+  __shared__ double A[2 * 32 * 33], U[2 * 32 * 33];   // (re, im) pairs, leading dimension ld
+  __shared__ double rc[16], rsr[16], rsi[16];
+  __shared__ int rpq[16];
+  __shared__ unsigned red[2][16];
+  const int kp = k + (k & 1), ld = kp + 1, np = kp / 2;
+  const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wp = t >> 5, nw = nt >> 5;
+  unsigned emax = 0;
+  for (int e = t; e < kp * kp; e += nt) {
+    const int i = e % kp, j = e / kp;
+    const zd a = (i < k && j < k && i <= j) ? Ain[(size_t)j * lda + i] : mk<double>(0, 0);
+    A[2 * (j * ld + i)] = a.re;
+    A[2 * (j * ld + i) + 1] = a.im;
+    U[2 * (j * ld + i)] = i == j ? 1.0 : 0.0;
+    U[2 * (j * ld + i) + 1] = 0.0;
+    emax = max(emax, max((unsigned)__double2hiint(a.re) >> 20 & 0x7ffu, (unsigned)__double2hiint(a.im) >> 20 & 0x7ffu));
+  }
+  emax = __reduce_max_sync(0xffffffffu, emax);
+  if (lane == 0) red[0][wp] = emax;
+  __syncthreads();
+  for (int w = 0; w < nw; ++w) emax = max(emax, red[0][w]);
+  const bool finite = emax < 0x7ff;
+  const int es = emax == 0 || !finite ? 1023 : max(1, 2046 - (int)emax);
+  const double scale = __hiloint2double(es << 20, 0), unscale = __hiloint2double((2046 - es) << 20, 0);
+  for (int e = t; e < kp * kp; e += nt) {   // each thread its own elements of the loop above
+    A[2 * ((e / kp) * ld + e % kp)] *= scale;
+    A[2 * ((e / kp) * ld + e % kp) + 1] *= scale;
+  }
+  __syncthreads();
+  // off-diagonal Frobenius norm <= k max |re|, |im| (off-diagonal) * sqrt(2); total >= max |diagonal|
+  const float thr = (float)tol / (1.5f * (float)k);
+  const int nA = (np * (np + 1) / 2 * 8 + 31) & ~31, nU = (np * kp * 4 + 31) & ~31;
+  int sweep = 0;
+  for (; finite && sweep < max_sweeps; ++sweep) {
+    unsigned off = 0, dia = 0;
+    for (int e = t; e < kp * kp; e += nt) {
+      const int i = e % kp, j = e / kp;
+      if (i > j) continue;
+      const unsigned m = max(__float_as_uint(fabsf(f32_bits(A[2 * (j * ld + i)]))),
+                             __float_as_uint(fabsf(f32_bits(A[2 * (j * ld + i) + 1]))));
+      if (i == j) dia = max(dia, m);
+      else off = max(off, m);
+    }
+    off = __reduce_max_sync(0xffffffffu, off);
+    dia = __reduce_max_sync(0xffffffffu, dia);
+    if (lane == 0) { red[0][wp] = off; red[1][wp] = dia; }
+    __syncthreads();
+    for (int w = 0; w < nw; ++w) { off = max(off, red[0][w]); dia = max(dia, red[1][w]); }
+    if (__uint_as_float(off) <= thr * __uint_as_float(dia)) break;
+    for (int round = 0; round < kp - 1; ++round) {
+      if (t < np) {
+        int p, q;
+        round_pair(t, round, kp, &p, &q);
+        const float br = f32_bits(A[2 * (q * ld + p)]), bi = f32_bits(A[2 * (q * ld + p) + 1]), n2 = fmaf(br, br, bi * bi);
+        double c = 1.0, sr = 0.0, si = 0.0;
+        if (n2 > 1e-37f) {
+          const float h = 0.5f * f32_bits(A[2 * (q * ld + q)] - A[2 * (p * ld + p)]), g = fmaf(h, h, n2);
+          const float f = copysignf(__fdividef(1.f, fabsf(h) + g * rsqrtf(g)), h), v = fmaf(n2 * f, f, 1.f);
+          const float cf = rsqrtf(v);
+          sr = f64_bits(cf * f * br);
+          si = f64_bits(cf * f * bi);
+          const double x = fma(-sr, sr, fma(-si, si, 1.0)), hc = f64_bits(0.5f * v * cf);   // c^2, 1 / (2 c)
+          c = f64_bits(cf);
+          c = fma(fma(-c, c, x), hc, c);
+          c = fma(fma(-c, c, x), hc, c);
+        }
+        rc[t] = c;
+        rsr[t] = sr;
+        rsi[t] = si;
+        rpq[t] = p | q << 16;
+      }
+      __syncthreads();
+      for (int base = wp * 32; base < nA + nU; base += nt) {
+        const bool isA = base < nA;
+        const int f = isA ? base + lane : base - nA + lane;
+        const int cm = f & 1, j = (f >> 1) & 1;
+        if (isA) {   // component cm of entry (i, j) of the block of pairs a <= b
+          const int i = (f >> 2) & 1;
+          int a, b;
+          const bool in = (f >> 3) < np * (np + 1) / 2;
+          tri_item(in ? f >> 3 : 0, &a, &b, 1);
+          const int ra = i ? rpq[a] >> 16 : rpq[a] & 0xffff;
+          const int cj = j ? rpq[b] >> 16 : rpq[b] & 0xffff, co = j ? rpq[b] & 0xffff : rpq[b] >> 16;
+          const double *own = ra <= cj ? A + 2 * (cj * ld + ra) : A + 2 * (ra * ld + cj);
+          const double *oth = ra <= co ? A + 2 * (co * ld + ra) : A + 2 * (ra * ld + co);
+          // an element below the diagonal is its mirror's conjugate
+          const double u = flip_if(own[cm], cm && ra > cj), v = flip_if(oth[cm], cm && ra > co),
+                       w = flip_if(oth[1 - cm], !cm && ra > co);
+          // Y_0 = c X_0 - conj(s) X_1, Y_1 = c X_1 + s X_0
+          const double y = fma(rc[b], u, fma(flip_if(rsr[b], !j), v, flip_if(rsi[b], !cm) * w));
+          const double v2 = __shfl_xor_sync(0xffffffffu, y, 4), w2 = __shfl_xor_sync(0xffffffffu, y, 5);
+          // X'_0 = c Y_0 - s Y_1, X'_1 = c Y_1 + conj(s) Y_0
+          double z = fma(rc[a], y, fma(flip_if(rsr[a], !i), v2, flip_if(rsi[a], cm) * w2));
+          double *dst = ra <= cj ? A + 2 * (cj * ld + ra) : A + 2 * (ra * ld + cj);
+          if (a == b && i == j && cm) z = 0.0;
+          if (in && (a != b || i == j || ra < cj)) dst[cm] = flip_if(z, cm && ra > cj);
+        } else {   // U <- U J
+          const bool in = (f >> 2) < np * kp;
+          const int row = in ? (f >> 2) % kp : 0, b = in ? (f >> 2) / kp : 0;
+          const int cj = j ? rpq[b] >> 16 : rpq[b] & 0xffff, co = j ? rpq[b] & 0xffff : rpq[b] >> 16;
+          const double u = U[2 * (cj * ld + row) + cm], v = U[2 * (co * ld + row) + cm], w = U[2 * (co * ld + row) + 1 - cm];
+          const double y = fma(rc[b], u, fma(flip_if(rsr[b], !j), v, flip_if(rsi[b], !cm) * w));
+          __syncwarp();
+          if (in) U[2 * (cj * ld + row) + cm] = y;
         }
       }
       __syncthreads();
     }
     if (sweep == max_sweeps - 1 && t == 0 && status) atomicOr(status, ST_EIG_NOCONV);
-    if (t == 0) atomicAdd(&g_jacobi_counters[sizeof(T) == 4 ? 1 : 3], 1ull);
   }
-  if (t == 0) atomicAdd(&g_jacobi_counters[sizeof(T) == 4 ? 0 : 2], 1ull);
+  if (t == 0) {
+    atomicAdd(&g_jacobi_counters[2], 1ull);
+    atomicAdd(&g_jacobi_counters[3], (unsigned long long)sweep);
+  }
   // sort eigenvalues decreasing (ties by index) and write out
-  for (int i = t; i < k; i += nt) {
-    const T wi = A[(size_t)i * kp + i].re;
+  for (int e = t; e < k * k; e += nt) {
+    const int i = e / k, row = e % k;
+    const double wi = A[2 * (i * ld + i)];
     int rank = 0;
     for (int j = 0; j < k; ++j) {
-      const T wj = A[(size_t)j * kp + j].re;
+      const double wj = A[2 * (j * ld + j)];
       rank += (wj > wi) || (wj == wi && j < i);
     }
-    wout[rank] = (double)wi;
-    if (rank < nout)
-      for (int row = 0; row < k; ++row) {
-        const cx<T> u = U[(size_t)i * kp + row];
-        Uout[(size_t)rank * ldu + row] = mk<double>((double)u.re, (double)u.im);
-      }
-    if (Uf)
-      for (int row = 0; row < k; ++row) {
-        const cx<T> u = U[(size_t)i * kp + row];
-        Uf[(size_t)rank * k + row] = mk<float>((float)u.re, (float)u.im);
-      }
+    if (row == 0) wout[rank] = wi * unscale;
+    Uout[(size_t)rank * ldu + row] = mk<double>(U[2 * (i * ld + row)], U[2 * (i * ld + row) + 1]);
   }
 }
 
-template <typename T>
-static size_t jacobi_smem(int k, bool u_in_smem) {
-  const int kp = k + (k & 1);
-  return (size_t)kp * kp * sizeof(cx<T>) * (u_in_smem ? 2 : 1) + (size_t)(kp / 2) * sizeof(Rot<T>) + 64;
-}
-
-size_t sm_jacobi_scratch_bytes(int k) {
-  const int kp = k + (k & 1);
-  return (size_t)kp * kp * sizeof(cx<double>);
-}
-
-void sm_jacobi(bool fp64, const zd *A, int lda, int k, zd *U, int ldu, double *w, void *scratch, int max_sweeps,
-               double tol, int *status, cudaStream_t st, void *Uf32, int nout) {
-  const size_t lim = 200 * 1024;
-  if (nout < 0 || nout > k) nout = k;
-  if (fp64) {
-    const bool in_smem = jacobi_smem<double>(k, true) <= lim;
-    const size_t bytes = jacobi_smem<double>(k, in_smem);
-    ::lrei::count_launch(); jacobi_kernel<double, 512><<<1, 512, bytes, st>>>(A, lda, k, U, ldu, w, in_smem ? nullptr : (cx<double> *)scratch,
-                                                 max_sweeps, tol, status, reinterpret_cast<cx<float> *>(Uf32), nout);
-  } else {
-    const bool in_smem = jacobi_smem<float>(k, true) <= lim;
-    const size_t bytes = jacobi_smem<float>(k, in_smem);
-    ::lrei::count_launch();
-    jacobi_kernel<float, 1024><<<1, 1024, bytes, st>>>(A, lda, k, U, ldu, w, in_smem ? nullptr : (cx<float> *)scratch,
-                                                       max_sweeps, tol, status, reinterpret_cast<cx<float> *>(Uf32), nout);
-  }
+void sm_jacobi64(const zd *A, int lda, int k, zd *U, int ldu, double *w, int max_sweeps, double tol, int *status,
+                 cudaStream_t st) {
+  const int np = (k + 1) / 2, slots = np * (np + 1) * 4 + 8 * np * np + 64;
+  const int nt = slots >= 512 ? 512 : slots / 32 * 32;
+  ::lrei::count_launch();
+  jacobi64_kernel<<<1, nt, 0, st>>>(A, lda, k, U, ldu, w, max_sweeps, tol, status);
 }
 
 // ------------------------------------------------------------ top-r eig
-// Block-Newton correction of the top-r invariant subspace (one column per CTA):
-// X_ij = (Ur^H R)_ij / (d_j - w_{r+i}), with R = M E - E (E^H M E) the residual of the current
-// basis E, d_j = (E^H M E)_jj its Rayleigh quotients, and Ur, w_{r+i} the FP32 eigenpairs of the
-// other k - r eigenvalues.  Because the correction is driven by the residual (which vanishes
-// exactly on the invariant subspace), repeated passes converge to FP64 accuracy even though Ur
-// is only FP32-accurate.
-// One CTA per column j of E; every step below is local to that column once W1 = M E is known:
+// Whether pass p ends with an orthonormalisation: E + D has Gram I + D^H D (D is orthogonal to E), so only after
+// the first pass (E is orthonormal to FP32 before it), a large correction, and the last one.
+__device__ __forceinline__ bool newton_orth(const int *meta, int p) {
+  return p == 1 || p == NEWTON_PASSES || !(__int_as_float(meta[META_D + p - 1]) <= 1e-9f) || newton_done(meta, p);
+}
+
+// Block-Newton correction of the top-r invariant subspace, one CTA per column j of E; everything below is local to that
+// column once W1 = M E is known:
 //   a = E^H W1[:, j],  R = W1[:, j] - E a                  (FP64: the residual is a small difference)
 //   X_i = (Ur^H R)_i / (a_j - w_{r+i}),  D = Ur X           (FP32: only the correction's leading digits
 //   Enew[:, j] = E[:, j] + D - E (E^H D)                      matter; Ur is FP32-accurate anyway)
-// Ur is read from the FP32 eigenvectors (k x k, ld k, column r + i).  E is read by all CTAs, so the
-// result goes to a separate array.  FP64 work is kept to the residual: on this part FP64
-// (including conversions) runs at 1/58 of the FP32 rate.
-__global__ void __launch_bounds__(256) newton_chain_kernel(const zd *__restrict__ W1, int ldw, const zd *__restrict__ E,
-                                                           int lde, const cx<float> *__restrict__ Uf,
-                                                           const double *__restrict__ w, int k, int r,
-                                                           zd *__restrict__ Enew, int ldn) {
+// Ur, w_{r+i}: the FP32 eigenpairs of the other k - r eigenvalues (columns r + i of Uf).  Because the correction is driven
+// by the residual (which vanishes exactly on the invariant subspace), repeated passes converge to FP64 accuracy although
+// Ur is only FP32-accurate.  Ef: E in FP32.  The FP64 sums are chains of 64 cycles per
+// instruction, so each is split over lanes: 32 per entry of a, 8 (4 parts x re, im) per entry of R.
+constexpr int NEWTON_THREADS = 512;
+__global__ void __launch_bounds__(NEWTON_THREADS) newton_chain_kernel(
+    const zd *__restrict__ W1, const zd *__restrict__ E, const cx<float> *__restrict__ Ef, const cx<float> *__restrict__ Uf,
+    const double *__restrict__ w, int k, int r, zd *__restrict__ Enew, int *meta, int pass) {
+  if (newton_done(meta, pass - 1)) return;
   extern __shared__ __align__(16) unsigned char nsm[];
-  zd *w1 = reinterpret_cast<zd *>(nsm);                    // k
-  zd *av = w1 + k;                                          // r
+  zd *av = reinterpret_cast<zd *>(nsm);                     // r
   cx<float> *rf = reinterpret_cast<cx<float> *>(av + r);    // k: residual (FP32)
   cx<float> *x = rf + k;                                    // k - r
   cx<float> *d2 = x + k;                                    // k
-  cx<float> *ef = d2 + k;                                   // k x r: E in FP32 (for the projection)
-  cx<float> *g1 = ef + (size_t)k * r;                       // r
-  const int j = blockIdx.x, t = threadIdx.x, lane = t & 31, wp = t >> 5, nw = blockDim.x >> 5;
-  for (int p = t; p < k; p += blockDim.x) w1[p] = W1[(size_t)j * ldw + p];
-  __syncthreads();
-  for (int i = wp; i < r; i += nw) {          // a = E^H w1
+  cx<float> *g1 = d2 + k;                                   // r
+  cx<float> *pd = g1 + r;                                   // 4 x k: parts of D
+  float *den = reinterpret_cast<float *>(pd + 4 * k);       // k - r
+  const int j = blockIdx.x, t = threadIdx.x, lane = t & 31, wp = t >> 5;
+  constexpr int NW = NEWTON_THREADS / 32;
+  const zd *w1 = W1 + (size_t)j * k;
+  for (int i = wp; i < r; i += NW) {          // a = E^H w1
     zd s = mk<double>(0, 0);
-    for (int p = lane; p < k; p += 32) fmac_(s, E[(size_t)i * lde + p], w1[p]);
+    for (int p = lane; p < k; p += 32) fmac_(s, E[(size_t)i * k + p], w1[p]);
     s = warp_sum(s);
     if (lane == 0) av[i] = s;
   }
   __syncthreads();
-  for (int p = t; p < k; p += blockDim.x) {   // R = w1 - E a; E to FP32 for the projection below
-    zd s = w1[p];
-    for (int i = 0; i < r; ++i) {
-      const zd e = E[(size_t)i * lde + p];
-      s = s - e * av[i];
-      ef[(size_t)i * k + p] = cvt<float>(e);
-    }
-    rf[p] = cvt<float>(s);
+  for (int i = t; i < k - r; i += NEWTON_THREADS) den[i] = (float)(av[j].re - w[r + i]);
+  for (int base = 0; base < k; base += NEWTON_THREADS / 8) {   // R = w1 - E a
+    const int p = base + (t >> 3), cm = t & 1, q = (t >> 1) & 3;
+    double s = 0.0;
+    if (p < k)
+      for (int i = q; i < r; i += 4) {
+        const zd e = E[(size_t)i * k + p], a = av[i];
+        s = fma(e.re, cm ? a.im : a.re, fma(e.im, cm ? a.re : -a.im, s));
+      }
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 4);
+    if (p < k && q == 0) reinterpret_cast<float *>(rf)[2 * p + cm] = (float)((cm ? w1[p].im : w1[p].re) - s);
   }
   __syncthreads();
-  const double dj = av[j].re;
-  for (int i = wp; i < k - r; i += nw) {      // X = (Ur^H R) ./ (d_j - w)
+#pragma unroll 2
+  for (int i = wp; i < k - r; i += NW) {      // X = (Ur^H R) ./ (d_j - w)
     cx<float> s = mk<float>(0.f, 0.f);
     const cx<float> *u = Uf + (size_t)(r + i) * k;
     for (int p = lane; p < k; p += 32) fmac_(s, u[p], rf[p]);
@@ -518,22 +713,24 @@ __global__ void __launch_bounds__(256) newton_chain_kernel(const zd *__restrict_
       s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
       s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
     }
-    if (lane == 0) {
-      const float den = (float)(dj - w[r + i]);
-      x[i] = (fabsf(den) > 1e-30f) ? mk<float>(s.re / den, s.im / den) : mk<float>(0.f, 0.f);
+    if (lane == 0) x[i] = (fabsf(den[i]) > 1e-30f) ? mk<float>(s.re / den[i], s.im / den[i]) : mk<float>(0.f, 0.f);
+  }
+  __syncthreads();
+  {                                           // D = Ur X, in four parts
+    const int c = t / (NEWTON_THREADS / 4), n4 = (k - r + 3) / 4, i1 = min(k - r, (c + 1) * n4);
+    for (int p = t % (NEWTON_THREADS / 4); p < k; p += NEWTON_THREADS / 4) {
+      cx<float> s = mk<float>(0.f, 0.f);
+#pragma unroll 8
+      for (int i = c * n4; i < i1; ++i) fma_(s, Uf[(size_t)(r + i) * k + p], x[i]);
+      pd[c * k + p] = s;
     }
   }
   __syncthreads();
-  for (int p = t; p < k; p += blockDim.x) {   // D = Ur X
-    cx<float> s = mk<float>(0.f, 0.f);
-#pragma unroll 8
-    for (int i = 0; i < k - r; ++i) fma_(s, Uf[(size_t)(r + i) * k + p], x[i]);
-    d2[p] = s;
-  }
+  for (int p = t; p < k; p += NEWTON_THREADS) d2[p] = (pd[p] + pd[k + p]) + (pd[2 * k + p] + pd[3 * k + p]);
   __syncthreads();
-  for (int i = wp; i < r; i += nw) {          // g = E^H D
+  for (int i = wp; i < r; i += NW) {          // g = E^H D
     cx<float> s = mk<float>(0.f, 0.f);
-    for (int p = lane; p < k; p += 32) fmac_(s, ef[(size_t)i * k + p], d2[p]);
+    for (int p = lane; p < k; p += 32) fmac_(s, Ef[(size_t)i * k + p], d2[p]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
@@ -542,76 +739,123 @@ __global__ void __launch_bounds__(256) newton_chain_kernel(const zd *__restrict_
     if (lane == 0) g1[i] = s;
   }
   __syncthreads();
-  for (int p = t; p < k; p += blockDim.x) {   // Enew = E + D - E g
+  unsigned big = 0;
+  for (int p = t; p < k; p += NEWTON_THREADS) {   // Enew = E + D - E g
     cx<float> s = d2[p];
-    for (int i = 0; i < r; ++i) s = s - ef[(size_t)i * k + p] * g1[i];
-    const zd e = E[(size_t)j * lde + p];
-    Enew[(size_t)j * ldn + p] = mk<double>(e.re + (double)s.re, e.im + (double)s.im);
+#pragma unroll 8
+    for (int i = 0; i < r; ++i) s = s - Ef[(size_t)i * k + p] * g1[i];
+    const zd e = E[(size_t)j * k + p];
+    Enew[(size_t)j * k + p] = mk<double>(e.re + (double)s.re, e.im + (double)s.im);
+    big = max(big, max(__float_as_uint(fabsf(s.re)), __float_as_uint(fabsf(s.im))));
   }
+  big = __reduce_max_sync(0xffffffffu, big);
+  if (lane == 0 && big) atomicMax(reinterpret_cast<unsigned *>(meta + META_D + pass - 1), big);
 }
 
 size_t newton_chain_smem(int k, int r) {
-  return (size_t)(k + r) * sizeof(zd) + (size_t)(3 * k + (size_t)k * r + r) * sizeof(cx<float>) + 64;
+  return (size_t)r * sizeof(zd) + (size_t)(7 * k + r) * sizeof(cx<float>) + (size_t)k * sizeof(float);
 }
 
-// T = (15/8) I - (5/4) G + (3/8) G^2 for G = E^H E = I + d: then E T = E (E^H E)^{-1/2} + O(d^3),
-// the orthonormal polar factor of E (same span).  One CTA per column j; the sum over m of
-// (G^2)_{ij} is split over the CTA's threads and combined in shared memory.
-__global__ void __launch_bounds__(256) polar_t_kernel(const zd *__restrict__ G, int ldg, int r, zd *__restrict__ T,
-                                                      int ldt) {
-  __shared__ zd part[256];
-  const int j = blockIdx.x, t = threadIdx.x;
-  const int i = t % r, q = t / r, nq = blockDim.x / r;
+// Column j of E T for T = (15/8) I - (5/4) G + (3/8) G^2, G = E^H E = I + d: E (E^H E)^{-1/2} + O(d^3), the orthonormal polar
+// factor of E (same span); Ein itself when the pass needs no orthonormalisation.  Also in FP32.
+// Eight lanes (4 parts x re, im) per entry of T and of the product; 32 rows per CTA, r columns.  (T by one kernel,
+// E T by another: 5.5 + 4.7 us at r = 8.)
+__global__ void __launch_bounds__(256) polar_kernel(const zd *__restrict__ G, const zd *__restrict__ Ein, int k, int r,
+                                                    zd *__restrict__ Eout, cx<float> *__restrict__ Eoutf, const int *meta,
+                                                    int pass) {
+  if (pass && newton_done(meta, pass - 1)) return;
+  __shared__ zd T[MAX_R];
+  const int j = blockIdx.x, t = threadIdx.x, cm = t & 1, q = (t >> 1) & 3, row = t >> 3;
+  const int p = blockIdx.y * 32 + row;
+  double s = 0.0;
+  if (!pass || newton_orth(meta, pass)) {
+    if (row < r)
+      for (int m = q; m < r; m += 4) {
+        const zd a = G[(size_t)m * r + row], b = G[(size_t)j * r + m];
+        s = fma(a.re, cm ? b.im : b.re, fma(a.im, cm ? b.re : -b.im, s));
+      }
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 4);
+    if (row < r && q == 0) {
+      const double g = reinterpret_cast<const double *>(G + (size_t)j * r + row)[cm];
+      reinterpret_cast<double *>(T)[2 * row + cm] = fma(0.375, s, fma(-1.25, g, (row == j && !cm) ? 1.875 : 0.0));
+    }
+    __syncthreads();
+    s = 0.0;
+    if (p < k)
+      for (int m = q; m < r; m += 4) {
+        const zd a = Ein[(size_t)m * k + p], b = T[m];
+        s = fma(a.re, cm ? b.im : b.re, fma(a.im, cm ? b.re : -b.im, s));
+      }
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 4);
+  } else if (p < k) {
+    s = reinterpret_cast<const double *>(Ein + (size_t)j * k + p)[cm];
+  }
+  if (p < k && q == 0) {
+    reinterpret_cast<double *>(Eout + (size_t)j * k + p)[cm] = s;
+    reinterpret_cast<float *>(Eoutf + (size_t)j * k + p)[cm] = (float)s;
+  }
+}
+
+// G = E^H E for polar_kernel, where the pass needs it: a warp per entry of the upper triangle.
+__global__ void __launch_bounds__(128) polar_gram_kernel(const zd *__restrict__ E, int k, int r, zd *__restrict__ G,
+                                                         const int *meta, int pass) {
+  if (pass && (newton_done(meta, pass - 1) || !newton_orth(meta, pass))) return;
+  const int e = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (e >= r * (r + 1) / 2) return;
+  int i, j;
+  tri_item(e, &i, &j, 1);
   zd s = mk<double>(0, 0);
-  if (q < nq)
-    for (int m = q; m < r; m += nq) fma_(s, G[(size_t)m * ldg + i], G[(size_t)j * ldg + m]);
-  part[t] = s;
-  __syncthreads();
-  if (t < r) {
-    zd g2 = mk<double>(0, 0);
-    for (int u = 0; u < nq; ++u) g2 = g2 + part[u * r + t];
-    const zd gij = G[(size_t)j * ldg + t];
-    zd v = mk<double>(-1.25 * gij.re + 0.375 * g2.re, -1.25 * gij.im + 0.375 * g2.im);
-    if (t == j) v.re += 1.875;
-    T[(size_t)j * ldt + t] = v;
+  for (int p = lane; p < k; p += 32) fmac_(s, E[(size_t)i * k + p], E[(size_t)j * k + p]);
+  s = warp_sum(s);
+  if (lane == 0) {
+    if (i == j) s.im = 0.0;
+    G[(size_t)j * r + i] = s;
+    if (i != j) G[(size_t)i * r + j] = conj(s);
   }
 }
 
-// Residual check ||M Y - Y diag(mu)||_max <= tol * max|mu|, else flag.
-__global__ void eig_check_kernel(const zd *__restrict__ MY, int ldmy, const zd *__restrict__ Y, int ldy,
-                                 const double *__restrict__ mu, int k, int r, double tol, int *status) {
-  __shared__ double red[8];
-  double m = 0.0, mm = 0.0;
-  for (int e = threadIdx.x; e < k * r; e += blockDim.x) {
-    const int i = e % k, j = e / k;
-    const zd a = MY[(size_t)j * ldmy + i], y = Y[(size_t)j * ldy + i];
-    const double rr = a.re - mu[j] * y.re, ri = a.im - mu[j] * y.im;
-    m = fmax(m, sqrt(rr * rr + ri * ri));
-    if (!isfinite(a.re) || !isfinite(a.im)) m = 1e300;
+// Y = E Wr (column j: blockIdx.x, 32 rows per CTA, eight lanes per entry), the residual M Y - Y diag(mu) from ME = M E, and its check:
+// an entry that may exceed tol * max |mu|, or is not finite, sets ST_EIG_RESID.
+__global__ void __launch_bounds__(256) eig_finish_kernel(const zd *__restrict__ E, const zd *__restrict__ ME,
+                                                         const zd *__restrict__ Wr, const double *__restrict__ mu, int k, int r,
+                                                         zd *__restrict__ Y, int ldy, double tol, int *status) {
+  const int j = blockIdx.x, t = threadIdx.x, cm = t & 1, q = (t >> 1) & 3, p = blockIdx.y * 32 + (t >> 3);
+  double y = 0.0, z = 0.0;
+  if (p < k)
+    for (int m = q; m < r; m += 4) {
+      const zd a = E[(size_t)m * k + p], c = ME[(size_t)m * k + p], b = Wr[(size_t)j * r + m];
+      const double bs = cm ? b.im : b.re, bo = cm ? b.re : -b.im;
+      y = fma(a.re, bs, fma(a.im, bo, y));
+      z = fma(c.re, bs, fma(c.im, bo, z));
+    }
+#pragma unroll
+  for (int o = 2; o <= 4; o <<= 1) {
+    y += __shfl_xor_sync(0xffffffffu, y, o);
+    z += __shfl_xor_sync(0xffffffffu, z, o);
   }
-  for (int j = threadIdx.x; j < r; j += blockDim.x) mm = fmax(mm, fabs(mu[j]));
-  for (int o = 16; o > 0; o >>= 1) {
-    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    mm = fmax(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+  if (p < k && q == 0) {
+    reinterpret_cast<double *>(Y + (size_t)j * ldy + p)[cm] = y;
+    double mm = 1e-300;
+    for (int i = 0; i < r; ++i) mm = fmax(mm, fabs(mu[i]));
+    if (!(fabs(fma(-mu[j], y, z)) <= 0.70710678 * tol * mm)) atomicOr(status, ST_EIG_RESID);
   }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0;
-    for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) a = fmax(a, red[i]);
-    if (!(a <= tol * fmax(mm, 1e-300))) atomicOr(status, ST_EIG_RESID);
-  }
+}
+
+static size_t rots_bytes(int k) {
+  const int kp = std::min(k + (k & 1), J32_KMAX);
+  return (size_t)J32_SWEEPS * (kp - 1) * (kp / 2) * sizeof(float4);
 }
 
 size_t sm_eig_ws_bytes(int kmax, int rmax) {
   size_t z = sizeof(zd);
   size_t b = 0;
-  b += (size_t)kmax * 8;             // w
-  b += 4 * (size_t)kmax * rmax * z;  // W1, A21, E1, W2
-  b += 4 * (size_t)rmax * rmax * z;  // G1, L1, Ar, Wr
-  b += sm_jacobi_scratch_bytes(kmax);
-  b += (size_t)rmax * rmax * z + (size_t)kmax * rmax * z;
-  b += (size_t)kmax * kmax * sizeof(cx<float>) + 256;   // FP32 eigenvectors
+  b += (size_t)kmax * 8;                                  // w
+  b += 3 * (size_t)kmax * rmax * z;                       // W1, E1, W2
+  b += 3 * (size_t)rmax * rmax * z;                       // G, Ar, Wr
+  b += (size_t)kmax * (kmax + rmax) * sizeof(cx<float>);  // FP32 eigenvectors, FP32 copy of E
+  b += (size_t)kmax * sizeof(int) + META_INTS * sizeof(int) + rots_bytes(kmax);
   return b + 4096;
 }
 
@@ -621,48 +865,54 @@ void sm_eig_topr(const zd *M, int ldm, int k, int r, zd *Y, int ldy, double *mu,
   auto take = [&](size_t bytes) { unsigned char *q = p; p += (bytes + 255) & ~(size_t)255; return q; };
   double *w = (double *)take((size_t)k * 8);
   zd *W1 = (zd *)take((size_t)k * r * sizeof(zd));
-  zd *A21 = (zd *)take((size_t)k * r * sizeof(zd));
   zd *E1 = (zd *)take((size_t)k * r * sizeof(zd));
   zd *W2 = (zd *)take((size_t)k * r * sizeof(zd));
-  zd *G1 = (zd *)take((size_t)r * r * sizeof(zd));
-  zd *L1 = (zd *)take((size_t)r * r * sizeof(zd));
+  zd *G = (zd *)take((size_t)r * r * sizeof(zd));
   zd *Ar = (zd *)take((size_t)r * r * sizeof(zd));
   zd *Wr = (zd *)take((size_t)r * r * sizeof(zd));
-  void *jscratch = take(sm_jacobi_scratch_bytes(k));
-  zd *Inv = (zd *)take((size_t)r * r * sizeof(zd));
-  zd *Xc = (zd *)take((size_t)k * r * sizeof(zd));
   cx<float> *U32 = (cx<float> *)take((size_t)k * k * sizeof(cx<float>));
+  cx<float> *E32 = (cx<float> *)take((size_t)k * r * sizeof(cx<float>));
+  int *order = (int *)take((size_t)k * sizeof(int));
+  int *meta = (int *)take(META_INTS * sizeof(int));
+  float4 *rots = (float4 *)take(rots_bytes(k));
   const zd one = mk<double>(1, 0), zero = mk<double>(0, 0);
-  (void)Inv; (void)Xc; (void)A21; (void)L1;
   // 1. FP32 eigendecomposition of the whole k x k matrix: all eigenvectors in FP32 (U32), the
-  //    top r also in FP64 (E1), eigenvalues in FP64 (w)
-  sm_jacobi(false, M, ldm, k, E1, k, w, jscratch, 12, 1e-5, nullptr, st, U32, r);
-  // 2.-3. block-Newton corrections of the top-r invariant subspace, each followed by the polar
-  // re-orthonormalisation E <- E T, T = (E^H E)^{-1/2} to third order (multi-CTA FP64 gemms)
-  const int passes = (k > r) ? 4 : 1;
-  for (int it = 0; it < passes; ++it) {
-    zd *Ecur = E1;
-    if (k > r) {
-      sm_gemm('N', 'N', k, r, k, one, M, ldm, E1, k, zero, W1, k, st);           // W1 = M E
-      ::lrei::count_launch();
-      newton_chain_kernel<<<r, 256, newton_chain_smem(k, r), st>>>(W1, k, E1, k, U32, w, k, r, W2, k);
-      Ecur = W2;
-    }
-    sm_gemm('C', 'N', r, r, k, one, Ecur, k, Ecur, k, zero, G1, r, st);         // G = E^H E
+  //    top r also in FP64 (E1), eigenvalues in FP64 (w).  Threads: one item each while the CTA has them.
+  const int np = (k + 1) / 2, nt = std::min(512, std::max(64, (np * (np - 1) / 2 + 31) / 32 * 32));
+  ::lrei::count_launch();
+  jacobi32_kernel<<<1, nt, j32_smem(k), st>>>(M, ldm, k, w, order, rots, meta, 1e-5f);
+  ::lrei::count_launch();
+  replay_kernel<<<(k + 7) / 8, 256, replay_smem(k), st>>>(k, rots, meta, order, U32, E1, k, r);
+  // 2.-3. block-Newton corrections of the top-r invariant subspace and polar re-orthonormalisations, each pass
+  //       returning at once when the ones before it have converged
+  const dim3 rows(r, (k + 31) / 32);
+  const int grams = (r * (r + 1) / 2 + 3) / 4;
+  auto polar = [&](const zd *in, zd *out, int pass) {
     ::lrei::count_launch();
-    polar_t_kernel<<<r, 256, 0, st>>>(G1, r, r, Ar, r);                        // T
-    sm_gemm('N', 'N', k, r, r, one, Ecur, k, Ar, r, zero, (Ecur == E1) ? W2 : E1, k, st);
-    if (Ecur == E1) sm_copy(W2, k, k, r, E1, k, st);
+    polar_gram_kernel<<<grams, 128, 0, st>>>(in, k, r, G, meta, pass);
+    ::lrei::count_launch();
+    polar_kernel<<<rows, 256, 0, st>>>(G, in, k, r, out, E32, meta, pass);
+  };
+  zd *E = E1;
+  if (k > r) {
+    for (int pass = 1; pass <= NEWTON_PASSES; ++pass) {
+      gemm_launch('N', 'N', k, r, k, one, M, ldm, E1, k, zero, W1, k, W1, k, 0, st, meta, pass - 1);   // W1 = M E
+      ::lrei::count_launch();
+      newton_chain_kernel<<<r, NEWTON_THREADS, newton_chain_smem(k, r), st>>>(W1, E1, pass == 1 ? U32 : E32, U32, w, k, r, W2,
+                                                                             meta, pass);
+      polar(W2, E1, pass);
+    }
+  } else {
+    polar(E1, W2, 0);
+    E = W2;
   }
-  // 4. Rayleigh-Ritz on span(E1) in FP64
-  sm_gemm('N', 'N', k, r, k, one, M, ldm, E1, k, zero, W2, k, st);
-  sm_gemm('C', 'N', r, r, k, one, E1, k, W2, k, zero, Ar, r, st);
-  sm_hermitize(Ar, r, r, st);
-  sm_jacobi(true, Ar, r, r, Wr, r, mu, jscratch, max_sweeps, 1e-14, status, st);
-  sm_gemm('N', 'N', k, r, r, one, E1, k, Wr, r, zero, Y, ldy, st);
-  // 5. residual check of the returned pairs
-  sm_gemm('N', 'N', k, r, k, one, M, ldm, Y, ldy, zero, W1, k, st);
-  ::lrei::count_launch(); eig_check_kernel<<<1, 256, 0, st>>>(W1, k, Y, ldy, mu, k, r, 1e-9, status);
+  // 4. Rayleigh-Ritz on span(E) in FP64
+  sm_gemm('N', 'N', k, r, k, one, M, ldm, E, k, zero, W1, k, st);
+  sm_gemm_herm('C', 'N', r, k, one, E, k, W1, k, zero, Ar, r, Ar, r, st);
+  sm_jacobi64(Ar, r, r, Wr, r, mu, max_sweeps, 1e-14, status, st);
+  // 5. the returned vectors and the residual check of the pairs
+  ::lrei::count_launch();
+  eig_finish_kernel<<<rows, 256, 0, st>>>(E, W1, Wr, mu, k, r, Y, ldy, 1e-9, status);
 }
 
 // ------------------------------------------------------------ elementwise
@@ -727,10 +977,8 @@ int sm_init() {
   const int lim = 210 * 1024;
   cudaFuncSetAttribute(trsv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  cudaError_t a = cudaFuncSetAttribute(jacobi_kernel<double, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  cudaError_t b = cudaFuncSetAttribute(jacobi_kernel<float, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  cudaError_t c = cudaFuncSetAttribute(newton_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  return (a == cudaSuccess && b == cudaSuccess && c == cudaSuccess) ? 0 : -1;
+  cudaError_t a = cudaFuncSetAttribute(jacobi32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  return a == cudaSuccess ? 0 : -1;
 }
 }  // namespace lrei
 

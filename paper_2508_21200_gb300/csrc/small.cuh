@@ -29,14 +29,13 @@ void sm_chol(const zd *A, int lda, int k, zd *L, int ldl, double tol, int zero_r
              int flag_rank, cudaStream_t st, const zd *ref = nullptr, int ldref = 0, zd *Linv = nullptr, int ldi = 0,
              int inv_h = 0, zd *Rc = nullptr, int ldrc = 0);
 
-// Hermitian eigendecomposition by cyclic Jacobi in working precision T (float or double),
-// one CTA.  Eigenvalues w sorted decreasing (ties by index), eigenvectors U (k x k, FP64).
-void sm_jacobi(bool fp64, const zd *A, int lda, int k, zd *U, int ldu, double *w, void *scratch, int max_sweeps,
-               double tol, int *status, cudaStream_t st, void *Uf32 = nullptr, int nout = -1);
-size_t sm_jacobi_scratch_bytes(int k);
+// FP64 eigendecomposition of a Hermitian k x k matrix (k <= 32, its upper triangle is read) by cyclic Jacobi, one CTA.
+// Eigenvalues w sorted decreasing (ties by index), eigenvectors U.  max_sweeps sweeps without convergence: ST_EIG_NOCONV.
+void sm_jacobi64(const zd *A, int lda, int k, zd *U, int ldu, double *w, int max_sweeps, double tol, int *status,
+                 cudaStream_t st);
 
-// Top-r eigenpairs of the Hermitian k x k matrix M to FP64 accuracy: FP32 Jacobi, one
-// block-Newton correction of the top-r invariant subspace, FP64 Rayleigh-Ritz on it
+// Top-r eigenpairs of the Hermitian k x k matrix M to FP64 accuracy: FP32 Jacobi,
+// block-Newton corrections of the top-r invariant subspace, FP64 Rayleigh-Ritz on it
 // (FP64 Jacobi of the r x r projection, at most max_sweeps sweeps; more sets ST_EIG_NOCONV).  Y (k x r, ld ldy) gets the eigenvectors,
 // mu the eigenvalues, both sorted decreasing.  ws: see sm_eig_ws_bytes.
 void sm_eig_topr(const zd *M, int ldm, int k, int r, zd *Y, int ldy, double *mu, void *ws, int *status,
