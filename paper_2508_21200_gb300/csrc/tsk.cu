@@ -492,195 +492,296 @@ __global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__
 
 // ------------------------------------------- fused tile pass, pipelined (complex64 bulk)
 // Same contract as ts_kernel for T = float, split H.V (apply_h == 0) and r in {8, 16, 32}.
-// Each CTA walks its tiles of TR rows with the next tile's blocks already in flight: cp.async
-// copies the rows of every input block into the other half of a double buffer (padded rows,
-// RS = r + 2 complex, so that rows of one column fall in different banks) while the current
-// tile is computed.  Gram work split: a micro-tile is column c of every Gram block against 4
-// consecutive G columns (g x 4 complex accumulators); NPH lanes of one warp take interleaved
-// rows of the same micro-tile and are combined by shuffles at each flush, every FLUSHT tiles
-// (at r = 16: 16 tiles, 128 rows per lane in plain FP32), into compensated FP32 pairs (TwoSum)
-// in shared memory.  Lane = phase * TPW + micro-tile, so
-// the G loads of a quarter-warp are one row (distinct 16-byte columns) and the block loads of
-// a half-warp are two rows of two columns: no bank conflicts at r = 16.
-template <int R, int TR, int GMAX, int MINB = (TR <= 32 ? 2 : 1)>
-__global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ TSArgs a,
-                                                       const cx<float> *__restrict__ coefg) {
-  constexpr int RS = R + 2;
-  constexpr int MTS = R * R / 4;
+// Each CTA walks its tiles of TR rows with the next tiles' blocks already in flight: cp.async copies the rows of every
+// input block into a ring of nst buffers (padded rows of RS complex) while the current tile is computed.
+// What bounds it is the FP32 pipe (at r = 16, 5 blocks: 150 us of multiply-adds against 99 us of bytes), next to it the
+// 128 bytes a cycle that shared memory delivers to registers, and the issue slots of everything else.  So
+//  - Gram micro-tiles are A columns of every Gram block against 8 G columns: 8 (g A + 8) bytes per 4 g A 8
+//    multiply-adds (g = 5, A = 2: 36 cycles of loads under 80 of arithmetic; with 4 columns, A = 1: 18 to 20);
+//    NPH lanes of a warp take interleaved rows of one micro-tile;
+//  - projection tiles are 4 rows x 4 columns, the sum over inputs split over KW lanes and KX warps;
+//  - plain multiply-adds: packed pairs (fma.rn.f32x2) halve the issue slots but need every factor twice in
+//    registers, and were slower (n = 22, r = 32, 5 blocks: Gram 3.9 -> 5.1 ms).
+// Every 16-byte load of a quarter-warp and 8-byte load of a half-warp falls in distinct banks: a thread's columns are
+// 16-byte chunks (2 columns) R / 8 (Gram) or R / 4 (projection) chunks apart, lanes of one sum whose
+// coefficients would share banks read their two chunks in swapped order, and RS is chosen so.
+// At a flush (128 rows per lane in plain FP32 at r = 16) the lanes of a micro-tile are combined by halving
+// shuffles, and each sum is added to its compensated FP32 pair (TwoSum), kept in the CTA's partial (L2).
+// Before (4 columns, one G column group conflicting at r = 32, double buffer): n = 20, r = 16, 5 blocks 337 us, now 262;
+// projection and Gram of 5 blocks 463 (4 inputs) -> 402 us; n = 22, r = 32, 5 blocks 7.7 -> 3.6 ms and 17.2 -> 7.0 ms.
+template <int R> struct TS3 {
+  static constexpr int RS = R == 16 ? 20 : R + 2;  // complex per padded row
+  static constexpr int KW = 32 / R;                // projection: lanes of one sum
+};
+constexpr int TS3_STAGES = 6;
+
+// GMAX: Gram blocks this instance handles (gl + 1 <= GMAX; with EXACT gl + 1 == GMAX)
+template <int R, int TR, int GMAX, bool EXACT, int A, int MINB>
+__global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ TSArgs a, const cx<float> *__restrict__ coefg,
+                                                       int nst) {
+  constexpr int RS = TS3<R>::RS, KW = TS3<R>::KW, KX = 128 / TR;   // KX: warps of one projection sum
+  constexpr int NJ = R / 8;                 // groups of 8 G columns
+  constexpr int MTS = (R / A) * NJ;         // micro-tiles
   constexpr int NPH = 256 / MTS;
   constexpr int TPW = 32 / NPH;
   constexpr int CH = R / 2;                 // 16-byte chunks per row
-  // GMAX: Gram blocks this instance handles (gl + 1 <= GMAX).  Flush period and row-loop unroll
-  // measured at n = 20, r = 16 (16 tiles and 8 / 4 for g = 2 / 5: 7-9% faster than 8 tiles and
-  // 2); the other widths keep the previous 8 and 2
-  constexpr int FLUSHT = R == 16 ? 16 : 8;
-  constexpr int UNR = R == 16 ? (GMAX <= 2 ? 8 : 4) : 2;
-  constexpr int PU = R == 16 ? 16 : 4;      // projection: inputs per block unrolled (measured, r = 16)
-  static_assert(NPH >= 1 && NPH <= 32 && (32 % NPH) == 0 && (RS * 8) % 16 == 0, "r in {8, 16, 32}");
+  constexpr int FLUSHT = (R == 32 ? 256 : (R == 16 ? 128 : 32)) * NPH / TR;   // tiles between flushes
+  constexpr int CNT = R / (KW * KX);
+  static_assert(NPH >= 2 && NPH <= 32 && (RS * 8) % 16 == 0 && FLUSHT >= 1 && TR / 16 * KX == 8, "r in {8, 16, 32}");
   extern __shared__ __align__(16) unsigned char smem3[];
   const int nq = a.nq, gl = a.gram_left, mode = a.mode;
   const int nb = nq + (mode != 2 ? 1 : 0);
-  const int g = gl + 1;
-  const int bstride = TR * RS;
-  cx<float> *buf = reinterpret_cast<cx<float> *>(smem3);       // [2][nb][TR][RS]
-  cx<float> *ns = buf + 2 * nb * bstride;                       // [TR][RS] new tile
-  cx<float> *cs = ns + bstride;                                 // [(nq+1) R][R] coefficients
-  float *slots = reinterpret_cast<float *>(cs + (mode != 0 ? (nq + 1) * R * R : 0));   // [g R][R][4]
+  const int g = EXACT ? GMAX : gl + 1;
+  constexpr int bstride = TR * RS;
+  cx<float> *buf = reinterpret_cast<cx<float> *>(smem3);       // [nst][nb][TR][RS]
+  cx<float> *ns = buf + nst * nb * bstride;                     // [KX][TR][RS] parts of the new tile; then the tile in the first
+  cx<float> *cs = ns + (mode != 0 ? KX * bstride : 0);          // [(nq+1) R][R] coefficients
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ph = lane / TPW;
   const int mt = warp * TPW + lane % TPW;
-  const int c = mt / (R / 4), j0 = (mt % (R / 4)) * 4;
+  const int c0 = mt / NJ * A, jg = mt % NJ;
   const long long N = a.N;
   const long long ntiles = (N + TR - 1) / TR;
+  const int ldg = g * R;
+  double2 *outp = reinterpret_cast<double2 *>(a.partial + (size_t)blockIdx.x * ldg * R * 2);
 
   if (mode != 0)
     for (int e = tid; e < (nq + 1) * R * R; e += 256) cs[e] = coefg[e];
-  for (int e = tid; e < g * R * R * 4; e += 256) slots[e] = 0.f;
 
+  // A tile's rows are contiguous: chunk tid + 256 x of a block.  Rows beyond N (in the last tile only) become zero.
+  const int lr_t = tid / CH;
+  const uint32_t sm_t = (uint32_t)__cvta_generic_to_shared(buf + lr_t * RS + tid % CH * 2);
   auto prefetch = [&](long long tile, int sb) {
     const long long row0 = tile * TR;
-    for (int m = 0; m < nb; ++m) {
-      const cx<float> *base = reinterpret_cast<const cx<float> *>(m < nq ? a.q[m] : a.src);
-      cx<float> *dst = buf + (size_t)(sb * nb + m) * bstride;
-      for (int e = tid; e < TR * CH; e += 256) {
-        const int lr = e / CH, ch = e % CH;
-        const bool ok = row0 + lr < N;
-        const cx<float> *gp = ok ? base + (size_t)(row0 + lr) * R + ch * 2 : base;
-        const uint32_t sa = (uint32_t)__cvta_generic_to_shared(dst + lr * RS + ch * 2);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gp), "r"(ok ? 16 : 0));
+    const size_t off = (size_t)row0 * (R * sizeof(cx<float>)) + tid * 16;
+    uint32_t sa = sm_t + sb * nb * (bstride * 8);
+    const bool full = row0 + TR <= N;
+#pragma unroll 1
+    for (int m = 0; m < nb; ++m, sa += bstride * 8) {
+      const char *gp = reinterpret_cast<const char *>(m < nq ? a.q[m] : a.src) + off;
+#pragma unroll
+      for (int x = 0; x < TR * CH / 256; ++x) {
+        const bool ok = full || row0 + lr_t + x * (256 / CH) < N;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa + x * (256 / CH) * RS * 8),
+                     "l"(ok ? gp + x * 4096 : gp - off), "r"(ok ? 16 : 0));
       }
     }
   };
 
-  cx<float> acc[GMAX][4];
+  cx<float> acc[GMAX][A][8];   // column y: chunk y / 2, i.e. 2 (jg + (y / 2) NJ) + y % 2
 #pragma unroll
   for (int m = 0; m < GMAX; ++m)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) acc[m][y] = mk<float>(0.f, 0.f);
+    for (int x = 0; x < A; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) acc[m][x][y] = mk<float>(0.f, 0.f);
 
-  auto flush = [&]() {
+  // The lanes of a micro-tile (bits TPW .. 16 of the lane) halve their columns three times, further ones are summed
+  // whole; then the pairs in the partial: (sum, error) of re and im, or with last their final values.
+  bool first = true;
+  auto flush = [&](bool last) {
+    constexpr int LV = NPH == 2 ? 1 : (NPH == 4 ? 2 : 3), LEFT = 8 >> LV;
+    int y0 = 0;
+#pragma unroll
+    for (int v = 0; v < LV; ++v) y0 += (lane & (16 >> v)) ? 4 >> v : 0;
 #pragma unroll
     for (int m = 0; m < GMAX; ++m) {
-      if (m < g) {
+      if (EXACT || m < g) {
 #pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          float re = acc[m][y].re, im = acc[m][y].im;
+        for (int x = 0; x < A; ++x) {
+          float2 f[8];
 #pragma unroll
-          for (int o = TPW; o < 32; o <<= 1) {
-            re += __shfl_xor_sync(0xffffffffu, re, o);
-            im += __shfl_xor_sync(0xffffffffu, im, o);
+          for (int y = 0; y < 8; ++y) {
+            f[y] = make_float2(acc[m][x][y].re, acc[m][x][y].im);
+            acc[m][x][y] = mk<float>(0.f, 0.f);
           }
-          if (ph == 0) {
-            float *s = slots + ((size_t)(m * R + c) * R + j0 + y) * 4;
-            two_sum_acc(s[0], s[1], re);
-            two_sum_acc(s[2], s[3], im);
+#pragma unroll
+          for (int v = 0; v < LV; ++v) {
+            const int o = 16 >> v, h = 4 >> v;
+            const bool up = lane & o;
+#pragma unroll
+            for (int y = 0; y < h; ++y) {
+              const float2 send = up ? f[y] : f[y + h], keep = up ? f[y + h] : f[y];
+              f[y].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, o);
+              f[y].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, o);
+            }
           }
-          acc[m][y] = mk<float>(0.f, 0.f);
+#pragma unroll
+          for (int o = 16 >> LV; o >= TPW; o >>= 1) {
+            f[0].x += __shfl_xor_sync(0xffffffffu, f[0].x, o);
+            f[0].y += __shfl_xor_sync(0xffffffffu, f[0].y, o);
+          }
+          if ((lane & ((32 >> LV) - 1)) < TPW) {
+#pragma unroll
+            for (int y = 0; y < LEFT; ++y) {
+              const int yy = y0 + y, col = 2 * (jg + (yy >> 1) * NJ) + (yy & 1);
+              double2 *slot = outp + (size_t)col * ldg + m * R + c0 + x;
+              float4 s = first ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<float4 *>(slot);
+              two_sum_acc(s.x, s.y, f[y].x);
+              two_sum_acc(s.z, s.w, f[y].y);
+              if (last) *slot = make_double2((double)s.x + (double)s.y, (double)s.z + (double)s.w);
+              else *reinterpret_cast<float4 *>(slot) = s;
+            }
+          }
         }
       }
     }
+    first = false;
   };
 
   long long tile = blockIdx.x;
   int sb = 0;
-  if (tile < ntiles) prefetch(tile, 0);
-  asm volatile("cp.async.commit_group;\n" ::);
+  for (int i = 0; i < nst - 1; ++i) {
+    if (tile + (long long)i * gridDim.x < ntiles) prefetch(tile + (long long)i * gridDim.x, i);
+    asm volatile("cp.async.commit_group;\n" ::);
+  }
   int since = 0;
   for (; tile < ntiles; tile += gridDim.x) {
-    const long long nxt = tile + gridDim.x;
-    if (nxt < ntiles) prefetch(nxt, sb ^ 1);
+    switch (nst) {   // all but the newest nst - 2 groups: this tile is there
+      case 2: asm volatile("cp.async.wait_group 0;\n" ::); break;
+      case 3: asm volatile("cp.async.wait_group 1;\n" ::); break;
+      case 4: asm volatile("cp.async.wait_group 2;\n" ::); break;
+      case 5: asm volatile("cp.async.wait_group 3;\n" ::); break;
+      default: asm volatile("cp.async.wait_group 4;\n" ::); break;
+    }
+    __syncthreads();   // also: every thread is done with the tile before this one
+    const long long nxt = tile + (long long)(nst - 1) * gridDim.x;
+    if (nxt < ntiles) prefetch(nxt, sb == 0 ? nst - 1 : sb - 1);
     asm volatile("cp.async.commit_group;\n" ::);
-    asm volatile("cp.async.wait_group 1;\n" ::);
-    __syncthreads();
     const cx<float> *B0 = buf + (size_t)sb * nb * bstride;
     const long long row0 = tile * TR;
     const int rows = (int)((N - row0) < TR ? (N - row0) : TR);
     const cx<float> *G;
     if (mode != 0) {
       const int mlast = (mode == 1) ? nq : nq - 1;
-      cx<float> *out = reinterpret_cast<cx<float> *>(a.out);
-      for (int e = tid; e < TR * (R / 4); e += 256) {
-        const int lr = e / (R / 4), q0 = (e % (R / 4)) * 4;
-        cx<float> o[4];
+      const int kw = lane % KW, q = lane / KW % (R / 4), kx = warp / (TR / 16);
+      const int lr0 = warp % (TR / 16) * 16 + lane / 8;       // rows lr0 + 4 y
+      const int sw = KW == 4 ? kw >> 1 : (KW == 2 ? kw : 0);   // order of the two chunks
+      const int k0 = kx * (CNT * KW) + kw;
+      cx<float> v[4][4];                                       // [row][column, chunks in order sw]
 #pragma unroll
-        for (int y = 0; y < 4; ++y) o[y] = mk<float>(0.f, 0.f);
-        for (int m = 0; m <= mlast; ++m) {
-          const cx<float> *X = B0 + (size_t)m * bstride + lr * RS;
-          const cx<float> *C = cs + (size_t)m * R * R + q0;
-#pragma unroll PU
-          for (int i = 0; i < R; ++i) {
-            const cx<float> x = X[i];
-            const float4 c01 = *reinterpret_cast<const float4 *>(C + i * R);
-            const float4 c23 = *reinterpret_cast<const float4 *>(C + i * R + 2);
-            fma_(o[0], x, mk<float>(c01.x, c01.y));
-            fma_(o[1], x, mk<float>(c01.z, c01.w));
-            fma_(o[2], x, mk<float>(c23.x, c23.y));
-            fma_(o[3], x, mk<float>(c23.z, c23.w));
+      for (int y = 0; y < 4; ++y)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) v[y][x] = mk<float>(0.f, 0.f);
+      for (int m = 0; m <= mlast; ++m) {
+        const cx<float> *X = B0 + (size_t)m * bstride + lr0 * RS + k0;
+        const cx<float> *C = cs + (size_t)(m * R + k0) * R + 2 * q;
+#pragma unroll
+        for (int i = 0; i < CNT; ++i) {
+          const float4 ca = *reinterpret_cast<const float4 *>(C + i * KW * R + sw * (R / 2));
+          const float4 cb = *reinterpret_cast<const float4 *>(C + i * KW * R + (1 - sw) * (R / 2));
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            const cx<float> x = X[4 * y * RS + i * KW];
+            fma_(v[y][0], x, mk<float>(ca.x, ca.y));
+            fma_(v[y][1], x, mk<float>(ca.z, ca.w));
+            fma_(v[y][2], x, mk<float>(cb.x, cb.y));
+            fma_(v[y][3], x, mk<float>(cb.z, cb.w));
           }
         }
-        const bool valid = lr < rows && row0 + lr >= a.zero_rows;
+      }
+      // lanes of one sum: the partner with the other order of chunks keeps the other two rows, the one with the same
+      // order the other chunk
+      if (KW >= 2) {
 #pragma unroll
-        for (int y = 0; y < 4; ++y)
-          if (!valid) o[y] = mk<float>(0.f, 0.f);
-        float4 *nd = reinterpret_cast<float4 *>(ns + lr * RS + q0);
-        nd[0] = make_float4(o[0].re, o[0].im, o[1].re, o[1].im);
-        nd[1] = make_float4(o[2].re, o[2].im, o[3].re, o[3].im);
-        if (out && lr < rows) {
-          float4 *od = reinterpret_cast<float4 *>(out + (size_t)(row0 + lr) * R + q0);
-          od[0] = nd[0];
-          od[1] = nd[1];
+        for (int y = 0; y < 2; ++y) {
+          cx<float> got[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const cx<float> send = sw ? v[y][x] : v[y + 2][x];
+            if (sw) v[y][x] = v[y + 2][x];
+            got[x].re = __shfl_xor_sync(0xffffffffu, send.re, KW / 2);
+            got[x].im = __shfl_xor_sync(0xffffffffu, send.im, KW / 2);
+          }
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            v[y][x].re += got[x ^ 2].re;
+            v[y][x].im += got[x ^ 2].im;
+          }
         }
+      }
+      if (KW == 4) {
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const cx<float> send = (kw & 1) ? v[y][x] : v[y][2 + x], keep = (kw & 1) ? v[y][2 + x] : v[y][x];
+            v[y][x].re = keep.re + __shfl_xor_sync(0xffffffffu, send.re, 1);
+            v[y][x].im = keep.im + __shfl_xor_sync(0xffffffffu, send.im, 1);
+          }
+      }
+      const int half = KW == 4 ? sw ^ (kw & 1) : sw;   // chunk in v[y][0..1]; the other one in v[y][2..3]
+#pragma unroll
+      for (int y = 0; y < (KW == 1 ? 4 : 2); ++y)
+#pragma unroll
+        for (int h = 0; h < (KW == 4 ? 1 : 2); ++h)
+          *reinterpret_cast<float4 *>(ns + (size_t)kx * bstride + (lr0 + 4 * (KW == 1 ? y : 2 * sw + y)) * RS + 2 * q +
+                                      (half ^ h) * (R / 2)) =
+              make_float4(v[y][2 * h].re, v[y][2 * h].im, v[y][2 * h + 1].re, v[y][2 * h + 1].im);
+      __syncthreads();
+      cx<float> *out = reinterpret_cast<cx<float> *>(a.out);
+      for (int e = tid; e < TR * CH; e += 256) {
+        const int lr = e / CH, ch = e % CH;
+        float4 *nd = reinterpret_cast<float4 *>(ns + lr * RS + ch * 2);
+        float4 w = *nd;
+#pragma unroll
+        for (int x = 1; x < KX; ++x) {
+          const float4 u = *reinterpret_cast<const float4 *>(ns + x * bstride + lr * RS + ch * 2);
+          w = make_float4(w.x + u.x, w.y + u.y, w.z + u.z, w.w + u.w);
+        }
+        if (!(lr < rows && row0 + lr >= a.zero_rows)) w = make_float4(0.f, 0.f, 0.f, 0.f);
+        *nd = w;
+        if (out && lr < rows) *reinterpret_cast<float4 *>(out + (size_t)(row0 + lr) * R + ch * 2) = w;
       }
       __syncthreads();
       G = ns;
     } else {
       G = B0 + (size_t)nq * bstride;
     }
-#pragma unroll UNR
+#pragma unroll 2
     for (int lr = ph; lr < TR; lr += NPH) {
-      const float4 ga = *reinterpret_cast<const float4 *>(G + lr * RS + j0);
-      const float4 gb = *reinterpret_cast<const float4 *>(G + lr * RS + j0 + 2);
-      const cx<float> gv0 = mk<float>(ga.x, ga.y), gv1 = mk<float>(ga.z, ga.w);
-      const cx<float> gv2 = mk<float>(gb.x, gb.y), gv3 = mk<float>(gb.z, gb.w);
+      cx<float> gv[8];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const float4 t = *reinterpret_cast<const float4 *>(G + lr * RS + 2 * (jg + x * NJ));
+        gv[2 * x] = mk<float>(t.x, t.y);
+        gv[2 * x + 1] = mk<float>(t.z, t.w);
+      }
 #pragma unroll
       for (int m = 0; m < GMAX; ++m) {
-        if (m < g) {
-          const cx<float> *L = (m < gl) ? B0 + (size_t)m * bstride : G;
-          const cx<float> lv = L[lr * RS + c];
-          fmac_(acc[m][0], lv, gv0);
-          fmac_(acc[m][1], lv, gv1);
-          fmac_(acc[m][2], lv, gv2);
-          fmac_(acc[m][3], lv, gv3);
+        if (EXACT || m < g) {
+          const cx<float> *L = ((EXACT ? m < GMAX - 1 : m < gl) ? B0 + (size_t)m * bstride : G) + lr * RS + c0;
+          cx<float> l[A];
+          if (A == 2) {
+            const float4 t = *reinterpret_cast<const float4 *>(L);
+            l[0] = mk<float>(t.x, t.y);
+            l[A - 1] = mk<float>(t.z, t.w);
+          } else {
+            l[0] = L[0];
+          }
+#pragma unroll
+          for (int x = 0; x < A; ++x)
+#pragma unroll
+            for (int y = 0; y < 8; ++y) fmac_(acc[m][x][y], l[x], gv[y]);
         }
       }
     }
     if (++since >= FLUSHT) {
       since = 0;
-      flush();
+      flush(false);
     }
-    __syncthreads();
-    sb ^= 1;
+    if (++sb == nst) sb = 0;
   }
   asm volatile("cp.async.wait_group 0;\n" ::);
-  flush();
-  __syncthreads();
-  const int ldg_ = g * R, nent = ldg_ * R;
-  double *outp = a.partial + (size_t)blockIdx.x * nent * 2;
-  for (int e = tid; e < nent; e += 256) {
-    const int j = e / ldg_, row = e % ldg_;
-    const float *s = slots + ((size_t)row * R + j) * 4;
-    outp[2 * e] = (double)s[0] + (double)s[1];
-    outp[2 * e + 1] = (double)s[2] + (double)s[3];
-  }
+  flush(true);
 }
 
-template <int R, int TR>
-__host__ inline size_t ts3_bytes(int nq, int gl, int mode) {
+// Shared memory with tiles of tr rows and nst stages.
+static size_t ts3_bytes(int r, int nq, int mode, int tr, int nst) {
   const int nb = nq + (mode != 2 ? 1 : 0);
-  const size_t bstride = (size_t)TR * (R + 2) * sizeof(cx<float>);
-  size_t b = (2 * (size_t)nb + 1) * bstride;
-  if (mode != 0) b += (size_t)(nq + 1) * R * R * sizeof(cx<float>);
-  b += (size_t)(gl + 1) * R * R * 16;
+  const size_t bstride = (size_t)tr * (r == 16 ? TS3<16>::RS : r + 2) * sizeof(cx<float>);
+  size_t b = ((size_t)nst * nb + (mode != 0 ? 128 / tr : 0)) * bstride;
+  if (mode != 0) b += (size_t)(nq + 1) * r * r * sizeof(cx<float>);
   return b;
 }
 
@@ -768,35 +869,65 @@ static int launch_ts_v1(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream
 }
 
 
-// Shared memory of the pipelined pass for the given arguments, or 0 if it does not apply.
-static size_t ts3_plan(const TSArgs &a, int *tr) {
-  if (a.apply_h) return 0;
-  if (a.mode == 0 && a.out) return 0;
+// Tile rows, CTAs per SM, stages and shared memory of the pipelined pass for the given arguments; 0 bytes if it does
+// not apply.  Two CTAs per SM (128 registers: A = 1 from 3 Gram blocks on) hide more latency than one with the larger
+// micro-tile up to 4 Gram blocks at r = 16 (4: 206 against 256 us at n = 20) and 3 at r = 32 (3: 2.4 against 2.6 ms at
+// n = 22; 4: 3.3 against 3.15); 64-row tiles halve the barriers of 32-row ones (r = 16, one block: 79 -> 71 us) and are
+// taken where two stages of them fit.
+struct TS3Plan {
+  int tr, two, nst;
+  size_t bytes;
+};
+static TS3Plan ts3_plan(const TSArgs &a) {
+  TS3Plan p{0, 0, 0, 0};
+  if (a.apply_h) return p;
+  if (a.mode == 0 && a.out) return p;
   const int r = a.r, nq = a.nq, gl = a.gram_left, mode = a.mode;
   const int nb = nq + (mode != 2 ? 1 : 0);
-  if (nb < 1 || nb > 8 || gl + 1 > 8 || gl > nq || (mode == 2 && nq < 1)) return 0;
-  auto al = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  if (nb < 1 || nb > 8 || gl + 1 > 8 || gl > nq || (mode == 2 && nq < 1)) return p;
+  auto al = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
   for (int m = 0; m < nq; ++m)
-    if (!al(a.q[m])) return 0;
-  if (mode != 2 && !al(a.src)) return 0;
-  if (a.out && !al(a.out)) return 0;
-  size_t b = 0;
-  if (r == 16) {
-    *tr = 32;
-    b = ts3_bytes<16, 32>(nq, gl, mode);
-  } else if (r == 8) {
-    *tr = 64;
-    b = ts3_bytes<8, 64>(nq, gl, mode);
-  } else if (r == 32) {
-    *tr = 32;
-    b = ts3_bytes<32, 32>(nq, gl, mode);
-  } else {
-    return 0;
-  }
-  return b <= 227 * 1024 ? b : 0;
+    if (!al(a.q[m])) return p;
+  if (mode != 2 && !al(a.src)) return p;
+  if (a.out && !al(a.out)) return p;
+  if (r != 8 && r != 16 && r != 32) return p;
+  const int two = r == 16 ? gl + 1 <= 4 : (r == 32 ? gl + 1 <= 3 : 0);
+  for (int t = two; t >= 0; --t)
+    for (int tr = 64; tr >= (r == 8 ? 64 : 32); tr /= 2) {
+      const size_t lim = (t ? 113 : 227) * 1024;
+      if (ts3_bytes(r, nq, mode, tr, 2) > lim) continue;
+      p.tr = tr;
+      p.two = t;
+      p.nst = 2;
+      while (p.nst < TS3_STAGES && ts3_bytes(r, nq, mode, tr, p.nst + 1) <= lim) ++p.nst;
+      p.bytes = ts3_bytes(r, nq, mode, tr, p.nst);
+      return p;
+    }
+  return p;
 }
 
-static int launch_ts3(const TSArgs &a, int nsm, cudaStream_t st, size_t bytes, int tr) {
+using TS3Kernel = void (*)(TSArgs, const cx<float> *, int);
+template <int R, int TR> static TS3Kernel ts3_instance(int g, bool two) {
+  if (g > 5) return ts3_kernel<R, TR, 8, false, 1, 1>;
+  if (two) {
+    if (g == 1) return ts3_kernel<R, TR, 1, true, 2, 2>;
+    if (g == 2) return ts3_kernel<R, TR, 2, true, 2, 2>;
+    if (g == 3) return ts3_kernel<R, TR, 3, true, 1, 2>;
+    if (g == 4) return ts3_kernel<R, TR, 4, true, 1, 2>;
+  }
+  if (g == 1) return ts3_kernel<R, TR, 1, true, 2, 2>;
+  if (g <= 3) return ts3_kernel<R, TR, 3, false, 2, 1>;
+  if (g == 4) return ts3_kernel<R, TR, 4, true, 2, 1>;
+  return ts3_kernel<R, TR, 5, true, 2, 1>;
+}
+static TS3Kernel ts3_pick(int r, int tr, int g, bool two) {
+  if (r == 16) return tr == 64 ? ts3_instance<16, 64>(g, two) : ts3_instance<16, 32>(g, two);
+  if (r == 32) return tr == 64 ? ts3_instance<32, 64>(g, two) : ts3_instance<32, 32>(g, two);
+  if (g <= 2) return ts3_kernel<8, 64, 2, false, 1, 1>;
+  return g <= 5 ? ts3_kernel<8, 64, 5, false, 1, 1> : ts3_kernel<8, 64, 8, false, 1, 1>;
+}
+
+static int launch_ts3(const TSArgs &a, int nsm, cudaStream_t st, const TS3Plan &p) {
   const cx<float> *coefg = nullptr;
   if (a.mode != 0) {
     if (!a.coef_scratch) return -1;
@@ -805,34 +936,21 @@ static int launch_ts3(const TSArgs &a, int nsm, cudaStream_t st, size_t bytes, i
     coef_convert2_kernel<float><<<8, 256, 0, st>>>(a.coefQ, a.coefS, a.nq, a.r, a.mode,
                                                   reinterpret_cast<cx<float> *>(a.coef_scratch));
   }
-  // persistent, each CTA walking tiles blockIdx.x, + gridDim.x, ...: one CTA per SM at 64-row
-  // tiles, two at 32-row tiles (at most 128 registers per thread and 110 KB of shared memory)
-  const long long ntiles = (a.N + tr - 1) / tr;
-  const long long cap = (tr <= 32 && bytes <= 110 * 1024) ? 2LL * nsm : (long long)nsm;
+  // persistent, each CTA walking tiles blockIdx.x, + gridDim.x, ...: one or two CTAs per SM (ts3_plan)
+  const long long ntiles = (a.N + p.tr - 1) / p.tr;
+  const long long cap = p.two ? 2LL * nsm : (long long)nsm;
   int grid = (int)(ntiles < cap ? ntiles : cap);
   if (grid < 1) grid = 1;
   ::lrei::count_launch();
-  const int g = a.gram_left + 1;
-  if (a.r == 16) {
-    if (g <= 2) ts3_kernel<16, 32, 2><<<grid, 256, bytes, st>>>(a, coefg);
-    else if (g <= 3) ts3_kernel<16, 32, 3><<<grid, 256, bytes, st>>>(a, coefg);
-    else if (g <= 4) ts3_kernel<16, 32, 4><<<grid, 256, bytes, st>>>(a, coefg);
-    else if (g <= 5) ts3_kernel<16, 32, 5><<<grid, 256, bytes, st>>>(a, coefg);
-    else ts3_kernel<16, 32, 8><<<grid, 256, bytes, st>>>(a, coefg);
-  } else if (a.r == 8) {
-    ts3_kernel<8, 64, 8><<<grid, 256, bytes, st>>>(a, coefg);
-  } else {
-    ts3_kernel<32, 32, 8><<<grid, 256, bytes, st>>>(a, coefg);
-  }
+  ts3_pick(a.r, p.tr, a.gram_left + 1, p.two)<<<grid, 256, p.bytes, st>>>(a, coefg, p.nst);
   return grid;
 }
 
 template <typename T>
 static int launch_ts_t(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_t st) {
   if (sizeof(T) == 4) {
-    int tr3 = 0;
-    const size_t b3 = ts3_plan(a, &tr3);
-    if (b3) return launch_ts3(a, nsm, st, b3, tr3);
+    const TS3Plan p = ts3_plan(a);
+    if (p.bytes) return launch_ts3(a, nsm, st, p);
   }
   const int r = a.r, rp = ts2_rp(r);
   const int NMT = (a.gram_left + 1) * rp / TS2<T>::MI * (rp / TS2<T>::MJ);
@@ -1098,13 +1216,14 @@ int ts_init() {
     cudaError_t x = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (x != cudaSuccess) e = x;
   };
-  set3((const void *)ts3_kernel<16, 32, 2>);
-  set3((const void *)ts3_kernel<16, 32, 3>);
-  set3((const void *)ts3_kernel<16, 32, 4>);
-  set3((const void *)ts3_kernel<16, 32, 5>);
-  set3((const void *)ts3_kernel<16, 32, 8>);
-  set3((const void *)ts3_kernel<8, 64, 8>);
-  set3((const void *)ts3_kernel<32, 32, 8>);
+  for (int g = 1; g <= 8; ++g)
+    for (int two = 0; two < 2; ++two) {
+      set3((const void *)ts3_pick(8, 64, g, two));
+      set3((const void *)ts3_pick(16, 64, g, two));
+      set3((const void *)ts3_pick(16, 32, g, two));
+      set3((const void *)ts3_pick(32, 64, g, two));
+      set3((const void *)ts3_pick(32, 32, g, two));
+    }
   set((const void *)ts_kernel<double, 2>);
   set((const void *)ts_kernel<double, 1>);
   set((const void *)ts_kernel<float, 4>);
