@@ -24,6 +24,7 @@
 #include "lrei.h"
 #include "common.cuh"
 #include "small.cuh"
+#include "small_dev.cuh"
 #include "tsk.cuh"
 
 namespace lrei { int sm_read_counters(unsigned long long *out); }
@@ -233,129 +234,150 @@ __global__ void rhs_coef_kernel(const zd *__restrict__ G, int r, const double *_
   }
 }
 
-// B = L^H diag(lam) L (r x r) for set_state.
+// B = L^H diag(lam) L (r x r) for set_state: eight lanes per entry.
 __global__ void lhl_kernel(const zd *__restrict__ L, int r, const double *__restrict__ lam, zd *__restrict__ B) {
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e % r, j = e / r;
-    zd s = mk<double>(0, 0);
-    for (int m = 0; m < r; ++m) {
-      // (L^H)_{im} = conj(L_{mi}), L_{mj}
-      const zd a = conj(L[(size_t)i * r + m]);
-      fma_(s, a, lam[m] * L[(size_t)j * r + m]);
-    }
-    B[e] = s;
+  const int e = (blockIdx.x * blockDim.x + threadIdx.x) / 8, q = threadIdx.x & 7;
+  const int i = e % r, j = e / r;
+  zd s = mk<double>(0, 0);
+  if (e < r * r)
+    for (int m = q; m < r; m += 8) fma_(s, conj(L[(size_t)i * r + m]), lam[m] * L[(size_t)j * r + m]);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
+    s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
   }
+  if (e < r * r && q == 0) B[e] = s;
 }
 
 // Observables from the Gram blocks of the observable pass (one CTA, r <= 32).
 // The stored factor V is orthonormalised implicitly: with V^*V = L L^H and X = L^{-1},
-// Tr(rho A) = Tr(Lambda X (V^*AV) X^H).
+// Tr(rho A) = Tr(Lambda X (V^*AV) X^H) = Tr(W V^*AV), W = X^H Lambda X: the products by X are done once (W, and
+// W2 = X^H Lambda^2 X for Tr(rho^2 H^2)), each observable is a sum over r^2 entries, and Tr(rho H rho H) the one of P P,
+// P = W V^*HV.  FP64 instructions bound it (an SM issues one per 19 cycles): an entry's sum is split over four lanes.
+// (With X A X^H formed per observable and square roots in the factor's chain: 179 us at r = 8, 2310 us at r = 32.)
 // With Werner weight p (Sec. 5, eq. werner-sol) the state is rho = p I/N + (1 - p) rho_hat, rho_hat the
 // stored low-rank state: H and the magnetisations are traceless, so their expectations and [rho, H] scale
 // by q = 1 - p; Tr rho = p + q Tr rho_hat; Tr rho^2 = p^2/N + 2 p q Tr(rho_hat)/N + q^2 Tr rho_hat^2; each
 // eigenvalue mu of rho_hat becomes p/N + q mu.  When mu is given, out[16 + i] receives the mapped Ritz
 // values and out[48 + i] the mapped spectrum.
-__global__ void obs_final_kernel(const double *__restrict__ red, int r, const double *__restrict__ lam,
-                                 double *__restrict__ out, double p, double inv_n, const double *__restrict__ mu) {
+__device__ __forceinline__ zd quad_sum(zd v) {
+#pragma unroll
+  for (int o = 1; o <= 2; o <<= 1) {
+    v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
+    v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
+  }
+  return v;
+}
+__global__ void __launch_bounds__(512) obs_final_kernel(const double *__restrict__ red, int r, const double *__restrict__ lam,
+                                                        double *__restrict__ out, double p, double inv_n,
+                                                        const double *__restrict__ mu) {
   // blocks: 0 V^*HV, 1 (HV)^*(HV), 2 V^*V, 3 V^*MxV, 4 V^*MyV, 5 V^*MzV
   extern __shared__ zd s[];
-  zd *Lg = s, *X = s + r * r, *T = s + 2 * r * r, *Ab = s + 3 * r * r;
-  __shared__ double part[6][32];
+  const int rr = r * r;
+  zd *P = s, *X = s + rr, *W = s + 2 * rr, *W2 = s + 3 * rr;
+  constexpr int NSUM = 8, NMAX = 3;
+  __shared__ double part[NSUM][16];
+  __shared__ unsigned long long pmax[NMAX][16];
+  __shared__ double tot[NSUM], lams[MAX_R];
   const zd *B = reinterpret_cast<const zd *>(red);
-  const int t = threadIdx.x, nt = blockDim.x;
-  for (int e = t; e < r * r; e += nt) Lg[e] = B[2 * r * r + e];
-  __syncthreads();
-  // Cholesky of Gamma (column by column, rows in parallel)
-  for (int j = 0; j < r; ++j) {
-    if (t == 0) {
-      double d = Lg[j * r + j].re;
-      for (int m = 0; m < j; ++m) d -= norm2(Lg[m * r + j]);
-      Lg[j * r + j] = mk<double>(sqrt(fmax(d, 1e-300)), 0);
-    }
-    __syncthreads();
-    for (int i = j + 1 + t; i < r; i += nt) {
-      zd v = Lg[j * r + i];
-      for (int m = 0; m < j; ++m) v = v - Lg[m * r + i] * conj(Lg[m * r + j]);
-      const double d = Lg[j * r + j].re;
-      Lg[j * r + i] = mk<double>(v.re / d, v.im / d);
-    }
-    __syncthreads();
-  }
-  // X = L^{-1}: column j by forward substitution, columns in parallel
-  for (int j = t; j < r; j += nt) {
-    for (int i = 0; i < r; ++i) {
-      if (i < j) { X[j * r + i] = mk<double>(0, 0); continue; }
-      zd v = mk<double>(i == j ? 1.0 : 0.0, 0);
-      for (int m = j; m < i; ++m) v = v - Lg[m * r + i] * X[j * r + m];
-      const double d = Lg[i * r + i].re;
-      X[j * r + i] = mk<double>(v.re / d, v.im / d);
-    }
-  }
-  __syncthreads();
-  const int which[5] = {0, 1, 3, 4, 5};
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int w = 0; w < 5; ++w) {
-    const zd *A = B + which[w] * r * r;
-    for (int e = t; e < r * r; e += nt) {          // T = X A
-      const int i = e % r, j = e / r;
-      zd v = mk<double>(0, 0);
-      for (int m = 0; m <= i; ++m) fma_(v, X[m * r + i], A[j * r + m]);
-      T[e] = v;
-    }
-    __syncthreads();
-    for (int e = t; e < r * r; e += nt) {          // Abar = T X^H
-      const int i = e % r, j = e / r;
-      zd v = mk<double>(0, 0);
-      for (int m = 0; m <= j; ++m) v = v + T[m * r + i] * conj(X[m * r + j]);
-      Ab[e] = v;
-    }
-    __syncthreads();
-    for (int i = t; i < r; i += nt) acc[w] += ((w == 1) ? lam[i] * lam[i] : lam[i]) * Ab[i * r + i].re;
-    if (w == 0)   // Tr(Lambda Gbar Lambda Gbar)
-      for (int e = t; e < r * r; e += nt) acc[5] += lam[e % r] * lam[e / r] * norm2(Ab[e]);
-    __syncthreads();
-  }
-  for (int q = 0; q < 6; ++q) {
-    double v = acc[q];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((t & 31) == 0) part[q][t >> 5] = v;
-  }
-  __syncthreads();
-  if (t == 0) {
-    double tot[6];
-    for (int q = 0; q < 6; ++q) {
-      tot[q] = 0.0;
-      for (int w = 0; w < (nt + 31) / 32; ++w) tot[q] += part[q][w];
-    }
-    const zd *Gam = B + 2 * r * r;
-    double trace = 0.0, purity = 0.0, orth = 0.0, herm = 0.0, gmax = 0.0;
-    for (int i = 0; i < r; ++i) {
-      trace += lam[i] * Gam[i * r + i].re;
-      for (int j = 0; j < r; ++j) {
-        purity += lam[i] * lam[j] * norm2(Gam[j * r + i]);
-        orth = fmax(orth, sqrt(norm2(Gam[j * r + i] - mk<double>(i == j ? 1.0 : 0.0, 0))));
-        const zd a = B[j * r + i], b = B[i * r + j];
-        herm = fmax(herm, sqrt(norm2(a - conj(b))));
-        gmax = fmax(gmax, sqrt(norm2(a)));
+  const zd *Gam = B + 2 * rr;
+  const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wp = t >> 5, q4 = t & 3;
+  for (int i = t; i < r; i += nt) lams[i] = lam[i];
+  chol_inv_cta(Gam, r, r, P, X);
+  for (int base = 0; base < rr; base += nt / 4) {      // W and W2, i <= j: sums over m >= j (X is lower triangular)
+    const int e = base + (t >> 2), i = e % r, j = e / r;
+    zd w = mk<double>(0, 0), w2 = w;
+    if (e < rr && i <= j)
+      for (int m = j + q4; m < r; m += 4) {
+        const zd a = conj(X[i * r + m]), b = lams[m] * X[j * r + m];
+        fma_(w, a, b);
+        fma_(w2, a, lams[m] * b);
       }
+    w = quad_sum(w);
+    w2 = quad_sum(w2);
+    if (e < rr && i <= j && q4 == 0) {
+      W[j * r + i] = w;
+      W[i * r + j] = conj(w);
+      W2[j * r + i] = w2;
+      W2[i * r + j] = conj(w2);
     }
+  }
+  __syncthreads();
+  for (int base = 0; base < rr; base += nt / 4) {      // P = W V^*HV
+    const int e = base + (t >> 2), i = e % r, j = e / r;
+    zd v = mk<double>(0, 0);
+    if (e < rr)
+      for (int m = q4; m < r; m += 4) fma_(v, W[m * r + i], B[j * r + m]);
+    v = quad_sum(v);
+    if (e < rr && q4 == 0) P[e] = v;
+  }
+  __syncthreads();
+  // sums: 0 Tr P, 1 Tr(W2 A1), 2..4 Tr(W A3..5), 5 Tr(P P), 6 trace, 7 purity; maxima (squares): V^*V - I, V^*HV - its
+  // conjugate transpose, V^*HV
+  double acc[NSUM] = {0, 0, 0, 0, 0, 0, 0, 0};
+  double mx[NMAX] = {0, 0, 0};
+  auto dot = [](double &a, zd x, zd y) { a = fma(x.re, y.re, fma(-x.im, y.im, a)); };   // a += Re(x y)
+  for (int e = t; e < rr; e += nt) {
+    const int i = e % r, j = e / r, et = i * r + j;
+    const zd w = W[et], g = Gam[e], h = B[e], ht = B[et];
+    dot(acc[1], W2[et], B[rr + e]);
+    dot(acc[2], w, B[3 * rr + e]);
+    dot(acc[3], w, B[4 * rr + e]);
+    dot(acc[4], w, B[5 * rr + e]);
+    dot(acc[5], P[e], P[et]);
+    acc[7] = fma(lams[i] * lams[j], norm2(g), acc[7]);
+    if (i == j) {
+      acc[0] += P[e].re;
+      acc[6] = fma(lams[i], g.re, acc[6]);
+    }
+    mx[0] = fmax(mx[0], norm2(i == j ? mk<double>(g.re - 1.0, g.im) : g));
+    mx[1] = fmax(mx[1], norm2(h - conj(ht)));
+    mx[2] = fmax(mx[2], norm2(h));
+  }
+#pragma unroll
+  for (int x = 0; x < NSUM; ++x) {
+    double v = acc[x];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) part[x][wp] = v;
+  }
+#pragma unroll
+  for (int x = 0; x < NMAX; ++x) {   // not negative: ordered as integers, which run at full rate
+    unsigned long long v = __double_as_longlong(mx[x]);
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0) pmax[x][wp] = v;
+  }
+  __syncthreads();
+  if (t < NSUM) {
+    double v = 0.0;
+    for (int w = 0; w < nt / 32; ++w) v += part[t][w];
+    tot[t] = v;
+  }
+  __syncthreads();
+  if (t < 9) {
     const double q = 1.0 - p;
-    out[0] = q * tot[0];
-    out[1] = q * tot[2];
-    out[2] = q * tot[3];
-    out[3] = q * tot[4];
-    out[4] = p * p * inv_n + 2.0 * p * q * inv_n * trace + q * q * purity;
-    out[5] = p + q * trace;
-    out[6] = orth;
-    out[7] = gmax > 0 ? herm / gmax : 0.0;
-    out[8] = q * sqrt(fmax(0.0, 2.0 * tot[1] - 2.0 * tot[5]));
+    double v = 0.0;
+    if (t == 0) v = q * tot[0];
+    else if (t <= 3) v = q * tot[t + 1];
+    else if (t == 4) v = p * p * inv_n + 2.0 * p * q * inv_n * tot[6] + q * q * tot[7];
+    else if (t == 5) v = p + q * tot[6];
+    else {
+      unsigned long long m[NMAX] = {0, 0, 0};
+      for (int w = 0; w < nt / 32; ++w)
+        for (int x = 0; x < NMAX; ++x) m[x] = max(m[x], pmax[x][w]);
+      const double orth = __longlong_as_double(m[0]), herm = __longlong_as_double(m[1]), g = __longlong_as_double(m[2]);
+      v = sqrt(t == 6 ? orth : (t == 7 ? (g > 0 ? herm / g : 0.0) : fmax(0.0, 2.0 * tot[1] - 2.0 * tot[5])));
+      if (t == 8) v *= q;
+    }
+    out[t] = v;
   }
   if (mu)
     for (int i = t; i < r; i += nt) {
       out[16 + i] = p * inv_n + (1.0 - p) * mu[i];
-      out[48 + i] = p * inv_n + (1.0 - p) * lam[i];
+      out[48 + i] = p * inv_n + (1.0 - p) * lams[i];
     }
 }
+// Threads: an entry each in the elementwise part.
+static int obs_final_threads(int r) { return r * r >= 512 ? 512 : (r * r < 64 ? 64 : (r * r + 31) / 32 * 32); }
 
 // ----------------------------------------------------------- controller features
 // ||[rho, H]||_F^2 = 2 Tr(Lambda^2 V^*H^2V) - 2 Tr(Lambda G Lambda G); in the Krylov frame H V_1 has
@@ -419,40 +441,14 @@ __global__ void feat_final_kernel(const double *__restrict__ mu, const double *_
 // Frobenius distance between two states rho_a = Va La Va^*, rho_b (same spectrum Lambda), from
 // C = Va^*Vb and the Grams of the stored factors (implicit Cholesky orthonormalisation):
 // ||rho_a - rho_b||_F^2 = 2 sum lam^2 - 2 sum_ij lam_i lam_j |Cbar_ij|^2, Cbar = La^{-1} C Lb^{-H}.
-__device__ void chol_inv_small(const zd *A, int lda, int r, zd *L, zd *X) {
-  // single thread: L = chol(A) lower, X = L^{-1}
-  for (int j = 0; j < r; ++j) {
-    double d = A[(size_t)j * lda + j].re;
-    for (int m = 0; m < j; ++m) d -= norm2(L[m * r + j]);
-    d = sqrt(fmax(d, 1e-300));
-    L[j * r + j] = mk<double>(d, 0);
-    for (int i = j + 1; i < r; ++i) {
-      zd v = A[(size_t)j * lda + i];
-      for (int m = 0; m < j; ++m) v = v - L[m * r + i] * conj(L[m * r + j]);
-      L[j * r + i] = mk<double>(v.re / d, v.im / d);
-    }
-    for (int i = 0; i < j; ++i) L[j * r + i] = mk<double>(0, 0);
-  }
-  for (int j = 0; j < r; ++j)
-    for (int i = 0; i < r; ++i) {
-      if (i < j) { X[j * r + i] = mk<double>(0, 0); continue; }
-      zd v = mk<double>(i == j ? 1.0 : 0.0, 0);
-      for (int m = j; m < i; ++m) v = v - L[m * r + i] * X[j * r + m];
-      const double d = L[i * r + i].re;
-      X[j * r + i] = mk<double>(v.re / d, v.im / d);
-    }
-}
-
 __global__ void dist_kernel(const zd *__restrict__ red, int r, const zd *__restrict__ Ga, int lda_,
                             const double *__restrict__ lam, double *__restrict__ out) {
   extern __shared__ zd sd[];
   zd *La = sd, *Xa = sd + r * r, *Lb = sd + 2 * r * r, *Xb = sd + 3 * r * r, *T = sd + 4 * r * r;
   const int t = threadIdx.x;
   const int ldr = 2 * r;   // red: rows 0..r-1 = Va^*Vb, rows r..2r-1 = Vb^*Vb (column-major)
-  if (t == 0) chol_inv_small(Ga, lda_, r, La, Xa);
-  if (t == 32 % blockDim.x && blockDim.x > 32) chol_inv_small(red + r, ldr, r, Lb, Xb);
-  if (blockDim.x <= 32 && t == 0) chol_inv_small(red + r, ldr, r, Lb, Xb);
-  __syncthreads();
+  chol_inv_cta(Ga, lda_, r, La, Xa);
+  chol_inv_cta(red + r, ldr, r, Lb, Xb);
   for (int e = t; e < r * r; e += blockDim.x) {   // T = Xa C
     const int i = e % r, j = e / r;
     zd v = mk<double>(0, 0);
@@ -460,7 +456,7 @@ __global__ void dist_kernel(const zd *__restrict__ red, int r, const zd *__restr
     T[e] = v;
   }
   __syncthreads();
-  __shared__ double acc[256];
+  __shared__ double acc[32];
   double s = 0.0;
   for (int e = t; e < r * r; e += blockDim.x) {   // Cbar = T Xb^H
     const int i = e % r, j = e / r;
@@ -468,11 +464,9 @@ __global__ void dist_kernel(const zd *__restrict__ red, int r, const zd *__restr
     for (int m = 0; m <= j; ++m) v = v + T[m * r + i] * conj(Xb[m * r + j]);
     s += lam[i] * lam[j] * norm2(v);
   }
-  acc[t] = s;
-  __syncthreads();
+  const double a = cta_sum(s, acc);
   if (t == 0) {
-    double a = 0, l2 = 0;
-    for (int w = 0; w < (int)blockDim.x; ++w) a += acc[w];
+    double l2 = 0;
     for (int i = 0; i < r; ++i) l2 += lam[i] * lam[i];
     out[0] = sqrt(fmax(2.0 * l2 - 2.0 * a, 0.0));
     out[1] = sqrt(l2);
@@ -493,19 +487,8 @@ __global__ void dist_prep_kernel(const zd *__restrict__ red, int r, const zd *__
   const int ldr = 2 * r;   // red rows 0..r-1: V_b^* V
   for (int e = t; e < r * r; e += blockDim.x) Lc[e] = Lcur[(size_t)(e / r) * ldl + (e % r)];
   __syncthreads();
-  if (t == 0) chol_inv_small(Gb, r, r, Lb, Xb);
-  if (t == (blockDim.x > 32 ? 32 : 0)) {
-    // Xc = Lc^{-1} from the current factor's Cholesky factor
-    for (int j = 0; j < r; ++j)
-      for (int i = 0; i < r; ++i) {
-        if (i < j) { Xc[j * r + i] = mk<double>(0, 0); continue; }
-        zd v = mk<double>(i == j ? 1.0 : 0.0, 0);
-        for (int m = j; m < i; ++m) v = v - Lc[m * r + i] * Xc[j * r + m];
-        const double d = Lc[i * r + i].re;
-        Xc[j * r + i] = mk<double>(v.re / d, v.im / d);
-      }
-  }
-  __syncthreads();
+  chol_inv_cta(Gb, r, r, Lb, Xb);
+  tri_inv_cta(Lc, r, Xc);   // Xc = Lc^{-1} from the current factor's Cholesky factor
   for (int e = t; e < r * r; e += blockDim.x) {   // T = Xb (V_b^* V)
     const int i = e % r, j = e / r;
     zd v = mk<double>(0, 0);
@@ -529,7 +512,7 @@ __global__ void dist_prep_kernel(const zd *__restrict__ red, int r, const zd *__
     coef[(size_t)j * 2 * r + r + i] = mk<double>(-v.re, -v.im);
   }
   // off-diagonal part of C Lambda C^H
-  __shared__ double acc[256];
+  __shared__ double acc[32];
   double s = 0.0;
   for (int e = t; e < r * r; e += blockDim.x) {
     const int i = e % r, j = e / r;
@@ -538,11 +521,9 @@ __global__ void dist_prep_kernel(const zd *__restrict__ red, int r, const zd *__
     for (int m = 0; m < r; ++m) v = v + lam[m] * (C[m * r + i] * conj(C[m * r + j]));
     s += norm2(v);
   }
-  acc[t] = s;
-  __syncthreads();
+  const double a = cta_sum(s, acc);
   if (t == 0) {
-    double a = 0, l2 = 0;
-    for (int w = 0; w < (int)blockDim.x; ++w) a += acc[w];
+    double l2 = 0;
     for (int i = 0; i < r; ++i) l2 += lam[i] * lam[i];
     out[0] = a;
     out[1] = l2;
@@ -707,7 +688,7 @@ __global__ void obs_assemble_kernel(const zd *__restrict__ R1, const zd *__restr
 
 void launch_obs_final(const double *red, int r, const double *lam, double *out, cudaStream_t st) {
   ::lrei::count_launch();
-  obs_final_kernel<<<1, 256, 4 * r * r * sizeof(zd), st>>>(red, r, lam, out, 0.0, 0.0, nullptr);
+  obs_final_kernel<<<1, obs_final_threads(r), 4 * r * r * sizeof(zd), st>>>(red, r, lam, out, 0.0, 0.0, nullptr);
 }
 
 }  // namespace lrei
@@ -1673,7 +1654,7 @@ int lrei_set_state(lrei_ctx *c, const void *V_dev, int r, int ld, int dtype, con
   sm_hermitize(red, r, r, c->st);
   sm_chol(red, r, r, c->L22, r, 1e-24, 1, c->dead_dev, c->status_dev, 1, c->st);
   LREI_CUDA_TRY(cudaMemcpyAsync(c->lam0_dev, lam_in.data(), r * sizeof(double), cudaMemcpyHostToDevice, c->st));
-  ::lrei::count_launch(); lhl_kernel<<<1, 256, 0, c->st>>>(c->L22, r, c->lam0_dev, c->Dm);
+  ::lrei::count_launch(); lhl_kernel<<<(r * r + 31) / 32, 256, 0, c->st>>>(c->L22, r, c->lam0_dev, c->Dm);
   sm_jacobi64(c->Dm, r, r, c->Lr, r, c->mu_dev, 60, 1e-15, c->status_dev, c->st);
   // coefficients R^{-1} E = L^{-H} E
   sm_copy(c->Lr, r, r, r, c->coefQ, r, c->st);
@@ -1859,7 +1840,7 @@ int lrei_observables(lrei_ctx *c, lrei_obs *out) {
     launch_reduce(c->partial, g, 6 * r * r * 2, c->red, c->st);
   }
   ::lrei::count_launch();
-  obs_final_kernel<<<1, 256, 4 * r * r * sizeof(zd), c->st>>>(c->red, r, c->lam0_dev, c->obs_dev, c->werner_p,
+  obs_final_kernel<<<1, obs_final_threads(r), 4 * r * r * sizeof(zd), c->st>>>(c->red, r, c->lam0_dev, c->obs_dev, c->werner_p,
                                                                1.0 / (double)c->N, c->mu_dev);
   LREI_CUDA_TRY(cudaMemcpyAsync(c->obs_host, c->obs_dev, 80 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
   leave(c);
@@ -2143,10 +2124,10 @@ int lrei_two_spin_rdm(lrei_ctx *c, int npairs, const int *site_k, const int *sit
   const long long groups = c->N / 4;
   const long long per_cta = 256 / r;
   int ncta = (int)std::min<long long>(64, std::max<long long>(1, (groups + per_cta - 1) / per_cta));
-  int chunk = (int)std::min<size_t>((size_t)npairs, c->partial_doubles / ((size_t)ncta * 20));
+  int chunk = (int)std::min<size_t>((size_t)npairs, c->partial_doubles / ((size_t)ncta * 16));
   while (chunk < 1 && ncta > 1) {
     ncta /= 2;
-    chunk = (int)std::min<size_t>((size_t)npairs, c->partial_doubles / ((size_t)ncta * 20));
+    chunk = (int)std::min<size_t>((size_t)npairs, c->partial_doubles / ((size_t)ncta * 16));
   }
   for (int q0 = 0; q0 < npairs && !rc; q0 += chunk) {
     const int nq = std::min(chunk, npairs - q0);

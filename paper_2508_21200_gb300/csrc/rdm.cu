@@ -10,8 +10,8 @@
 // over the factor computes the ten entries s <= s'; each thread owns one column c of a group
 // (threads of consecutive columns read consecutive words of a row) and keeps running sums,
 // compensated (TwoSum) in the complex64 path, combined per CTA and written as FP64 partials.
-// A one-thread-per-pair FP64 kernel then sums the partials in a fixed order, applies the Werner
-// weight p (R -> p I/4 + (1 - p) R) and evaluates the two measures by 4 x 4 Jacobi.
+// One CTA per pair then sums the partials in a fixed order, applies the Werner weight p (R -> p I/4 + (1 - p) R) and
+// evaluates the two measures by 4 x 4 Jacobi, a warp each.
 #include "common.cuh"
 
 namespace lrei {
@@ -26,21 +26,21 @@ __device__ __forceinline__ void two_sum(float &hi, float &lo, float b) {
 
 template <typename T> struct RAcc;
 template <> struct RAcc<double> {
-  double v[20];
+  double v[16];
   __device__ void zero() {
 #pragma unroll
-    for (int i = 0; i < 20; ++i) v[i] = 0.0;
+    for (int i = 0; i < 16; ++i) v[i] = 0.0;
   }
-  __device__ void add(int i, double x) { v[i] += x; }
+  __device__ void add(int i, double a, double b, double c, double d) { v[i] = fma(a, b, fma(c, d, v[i])); }   // += a b + c d
   __device__ double get(int i) const { return v[i]; }
 };
 template <> struct RAcc<float> {
-  float v[20], e[20];
+  float v[16], e[16];
   __device__ void zero() {
 #pragma unroll
-    for (int i = 0; i < 20; ++i) v[i] = e[i] = 0.f;
+    for (int i = 0; i < 16; ++i) v[i] = e[i] = 0.f;
   }
-  __device__ void add(int i, float x) { two_sum(v[i], e[i], x); }
+  __device__ void add(int i, float a, float b, float c, float d) { two_sum(v[i], e[i], fmaf(a, b, c * d)); }
   __device__ double get(int i) const { return (double)v[i] + (double)e[i]; }
 };
 
@@ -52,12 +52,13 @@ __device__ __forceinline__ uint32_t insert_zero(uint32_t x, int pos) {
 }  // namespace
 
 // pairs: 2 ints per pair, the bit positions of sites k and l in the basis index.
-// partial: [npairs][gridDim.x][20] doubles (entries (s, s') with s <= s' in row order, re/im).
+// partial: [npairs][gridDim.x][16] doubles: the diagonal entries, then (s, s') with s < s' in row order, re/im.
+// FP64 multiply-adds bound it (n = 16, r = 7, 120 pairs: 40 per group and column, 1.85 ms with 80).
 template <typename T>
 __global__ void __launch_bounds__(256) rdm_kernel(const cx<T> *__restrict__ V, long long N, int r,
                                                   const double *__restrict__ lam, const int *__restrict__ pairs,
                                                   double *__restrict__ partial) {
-  __shared__ double red[8][20];
+  __shared__ double red[8][16];
   const int p = blockIdx.y;
   const int bk = pairs[2 * p], bl = pairs[2 * p + 1];
   const int lo = bk < bl ? bk : bl, hi = bk < bl ? bl : bk;
@@ -77,167 +78,190 @@ __global__ void __launch_bounds__(256) rdm_kernel(const cx<T> *__restrict__ V, l
         const uint32_t b = b0 | ((uint32_t)(s >> 1) << bk) | ((uint32_t)(s & 1) << bl);
         v[s] = V[(size_t)b * r + c];
       }
-      int e = 0;
+      int e = 4;
 #pragma unroll
-      for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 4; ++s) {   // lambda_c v_s conj(v_t)
+        const cx<T> w = lc * v[s];
+        acc.add(s, w.re, v[s].re, w.im, v[s].im);
 #pragma unroll
-        for (int t = s; t < 4; ++t) {
-          // lambda_c v_s conj(v_t)
-          const T re = v[s].re * v[t].re + v[s].im * v[t].im;
-          const T im = v[s].im * v[t].re - v[s].re * v[t].im;
-          acc.add(2 * e, lc * re);
-          acc.add(2 * e + 1, lc * im);
-          ++e;
+        for (int t = s + 1; t < 4; ++t) {
+          acc.add(e++, w.re, v[t].re, w.im, v[t].im);
+          acc.add(e++, w.im, v[t].re, -w.re, v[t].im);
         }
+      }
     }
   }
   // combine the CTA's threads: warp shuffles, then the warps in a fixed order
   const int lane = tid & 31, wp = tid >> 5;
 #pragma unroll
-  for (int i = 0; i < 20; ++i) {
+  for (int i = 0; i < 16; ++i) {
     double x = acc.get(i);
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     if (lane == 0) red[wp][i] = x;
   }
   __syncthreads();
-  if (tid < 20) {
+  if (tid < 16) {
     double s = 0.0;
     for (int w = 0; w < 8; ++w) s += red[w][tid];
-    partial[((size_t)p * gridDim.x + blockIdx.x) * 20 + tid] = s;
+    partial[((size_t)p * gridDim.x + blockIdx.x) * 16 + tid] = s;
   }
 }
 
 namespace {
-// Eigenvalues (decreasing) and eigenvectors (columns of U, 4 x 4 column-major) of a Hermitian 4 x 4
-// matrix A (column-major, overwritten) by cyclic complex Jacobi in FP64.
-__device__ void herm4_eig(zd *A, zd *U, double *w) {
-  for (int i = 0; i < 16; ++i) U[i] = mk<double>((i % 5) == 0 ? 1.0 : 0.0, 0.0);
-  for (int sweep = 0; sweep < 30; ++sweep) {
-    double off = 0.0, tot = 0.0;
-    for (int i = 0; i < 16; ++i) {
-      tot += norm2(A[i]);
-      if (i % 5) off += norm2(A[i]);
+// Eigenvalues (w, in the order of the diagonal) and eigenvectors (columns of U, 4 x 4 column-major) of the Hermitian 4 x 4
+// matrix A (column-major) by cyclic complex Jacobi, by one warp: lane 8 i + 2 j + m holds component m of entry
+// (i, j), and a round applies the two rotations of the pairs x, x ^ mask.  An FP64 instruction takes 64 cycles in a
+// chain, a division or square root 7 to 11 of these, so the angle is taken in FP32 (which annihilates to 1e-7 a
+// round) and made unitary in FP64 by two Newton steps for c = sqrt(1 - |s|^2).  A is scaled by a power of two to entries
+// below 2, so that FP32 has the range.  (One thread per matrix with FP64 angles: 5.0 ms for the 120 pairs of n = 16.)
+__device__ __forceinline__ float to_f32(double x) { return (float)x; }
+__device__ __forceinline__ double flip(double x, bool c) { return c ? -x : x; }
+__device__ void herm4_eig(const zd *A, zd *U, double *w) {
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31, m = lane & 1, j = (lane >> 1) & 3, i = lane >> 3;
+  double a = reinterpret_cast<const double *>(A)[2 * (4 * j + i) + m];
+  double u = (i == j && m == 0) ? 1.0 : 0.0;
+  const unsigned emax = __reduce_max_sync(all, ((unsigned)__double2hiint(a) >> 20) & 0x7ffu);
+  const bool finite = emax < 0x7ff;
+  const int es = emax == 0 || !finite ? 1023 : max(1, 2046 - (int)emax);
+  a *= __hiloint2double(es << 20, 0);
+  for (int sweep = 0; finite && sweep < 30; ++sweep) {
+    const unsigned v = __float_as_uint(fabsf(to_f32(a)));
+    const float off = __uint_as_float(__reduce_max_sync(all, i != j ? v : 0u));
+    const float dia = __uint_as_float(__reduce_max_sync(all, i == j ? v : 0u));
+    if (off <= 2e-17f * dia) break;   // off-diagonal norm <= sqrt(24) max |re|, |im| <= 1e-16 of the total
+#pragma unroll
+    for (int mask = 1; mask < 4; ++mask) {
+      const int p = min(j, j ^ mask), q = max(j, j ^ mask);
+      const double app = __shfl_sync(all, a, 8 * p + 2 * p), aqq = __shfl_sync(all, a, 8 * q + 2 * q);
+      const float br = to_f32(__shfl_sync(all, a, 8 * p + 2 * q)), bi = to_f32(__shfl_sync(all, a, 8 * p + 2 * q + 1));
+      const float n2 = fmaf(br, br, bi * bi);
+      double c = 1.0, sr = 0.0, si = 0.0;   // [[c, s], [-conj(s), c]] on (p, q)
+      if (n2 > 1e-37f) {
+        const float h = 0.5f * to_f32(aqq - app), g = fmaf(h, h, n2);
+        const float f = copysignf(__fdividef(1.f, fabsf(h) + g * rsqrtf(g)), h), vv = fmaf(n2 * f, f, 1.f), cf = rsqrtf(vv);
+        sr = (double)(cf * f * br);
+        si = (double)(cf * f * bi);
+        const double x = fma(-sr, sr, fma(-si, si, 1.0)), hc = (double)(0.5f * vv * cf);
+        c = (double)cf;
+        c = fma(fma(-c, c, x), hc, c);
+        c = fma(fma(-c, c, x), hc, c);
+      }
+      const bool jq = j & (mask & 2 ? 2 : 1) ? true : false, iq = i & (mask & 2 ? 2 : 1) ? true : false;   // the larger of its pair
+      // the rotation of this lane's row pair is the one of column i
+      const double ci = __shfl_sync(all, c, 2 * i), sri = __shfl_sync(all, sr, 2 * i), sii = __shfl_sync(all, si, 2 * i);
+      const double srj = flip(sr, !jq), sij = flip(si, !m);
+      // A J and U J: the other column's components
+      const double av = __shfl_xor_sync(all, a, 2 * mask), aw = __shfl_xor_sync(all, a, 2 * mask + 1);
+      const double uv = __shfl_xor_sync(all, u, 2 * mask), uw = __shfl_xor_sync(all, u, 2 * mask + 1);
+      const double y = fma(c, a, fma(srj, av, sij * aw));
+      u = fma(c, u, fma(srj, uv, sij * uw));
+      // J^H (A J): the other row's
+      const double yv = __shfl_xor_sync(all, y, 8 * mask), yw = __shfl_xor_sync(all, y, 8 * mask + 1);
+      a = fma(ci, y, fma(flip(sri, !iq), yv, flip(sii, m) * yw));
+      if (i == j && m) a = 0.0;
     }
-    if (off <= 1e-32 * tot || off == 0.0) break;
-    for (int p = 0; p < 3; ++p)
-      for (int q = p + 1; q < 4; ++q) {
-        const zd apq = A[q * 4 + p];
-        const double ab = sqrt(norm2(apq));
-        if (ab == 0.0) continue;
-        const double app = A[p * 4 + p].re, aqq = A[q * 4 + q].re;
-        // rotate so that the (p, q) entry vanishes: phase e = apq / |apq|
-        const double theta = 0.5 * (aqq - app) / ab;
-        const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-        const double cs = 1.0 / sqrt(t * t + 1.0), sn = t * cs;
-        const zd e = mk<double>(apq.re / ab, apq.im / ab);
-        // columns: A <- A G with G = [[c, s e], [-s conj(e), c]] on (p, q)
-        for (int i = 0; i < 4; ++i) {
-          const zd aip = A[p * 4 + i], aiq = A[q * 4 + i];
-          A[p * 4 + i] = cs * aip - sn * (aiq * conj(e));
-          A[q * 4 + i] = cs * aiq + sn * (aip * e);
-          const zd uip = U[p * 4 + i], uiq = U[q * 4 + i];
-          U[p * 4 + i] = cs * uip - sn * (uiq * conj(e));
-          U[q * 4 + i] = cs * uiq + sn * (uip * e);
-        }
-        // rows: A <- G^H A
-        for (int j = 0; j < 4; ++j) {
-          const zd apj = A[j * 4 + p], aqj = A[j * 4 + q];
-          A[j * 4 + p] = cs * apj - sn * (aqj * e);
-          A[j * 4 + q] = cs * aqj + sn * (apj * conj(e));
-        }
-      }
   }
-  for (int i = 0; i < 4; ++i) w[i] = A[i * 4 + i].re;
-  // sort decreasing (with the vectors)
-  for (int i = 0; i < 4; ++i)
-    for (int j = i + 1; j < 4; ++j)
-      if (w[j] > w[i]) {
-        const double tw = w[i]; w[i] = w[j]; w[j] = tw;
-        for (int m = 0; m < 4; ++m) { const zd tu = U[i * 4 + m]; U[i * 4 + m] = U[j * 4 + m]; U[j * 4 + m] = tu; }
-      }
+  reinterpret_cast<double *>(U)[2 * (4 * j + i) + m] = u;
+  if (i == j && m == 0) w[i] = a * __hiloint2double((2046 - es) << 20, 0);
+  __syncwarp();
+}
+// C = A B (4 x 4) by one warp; B conjugate-transposed with bh.
+__device__ void mul4(const zd *A, const zd *B, bool bh, zd *C) {
+  const int lane = threadIdx.x & 31, m = lane & 1, j = (lane >> 1) & 3, i = lane >> 3;
+  double v = 0.0;
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const zd a = A[4 * x + i], b = bh ? conj(B[4 * x + j]) : B[4 * j + x];
+    v = fma(a.re, m ? b.im : b.re, fma(m ? a.im : -a.im, m ? b.re : b.im, v));
+  }
+  reinterpret_cast<double *>(C)[2 * (4 * j + i) + m] = v;
+  __syncwarp();
 }
 }  // namespace
 
-// One thread per pair: R from the partials, the Werner map, concurrence and negativity.
+// One CTA per pair: R from the partials, the Werner map, then the concurrence by warp 0 and the negativity by warp 1.
 // out: [npairs][32 + 2] doubles: R (4 x 4 complex, column-major), concurrence, negativity.
-__global__ void rdm_final_kernel(const double *__restrict__ partial, int nparts, int npairs, double p_werner,
-                                 double *__restrict__ out) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= npairs) return;
-  double s[20];
-  for (int i = 0; i < 20; ++i) s[i] = 0.0;
-  for (int b = 0; b < nparts; ++b)
-    for (int i = 0; i < 20; ++i) s[i] += partial[((size_t)q * nparts + b) * 20 + i];
-  zd R[16];
-  int e = 0;
-  for (int a = 0; a < 4; ++a)
-    for (int t = a; t < 4; ++t) {
-      const zd v = mk<double>(s[2 * e], s[2 * e + 1]);
-      R[t * 4 + a] = v;            // (a, t)
-      R[a * 4 + t] = conj(v);      // (t, a)
-      ++e;
-    }
-  const double qw = 1.0 - p_werner;
-  for (int i = 0; i < 16; ++i) R[i] = qw * R[i];
-  for (int i = 0; i < 4; ++i) R[i * 5].re += 0.25 * p_werner;
-  double *o = out + (size_t)q * 34;
-  for (int i = 0; i < 16; ++i) {
-    o[2 * i] = R[i].re;
-    o[2 * i + 1] = R[i].im;
+__global__ void __launch_bounds__(256) rdm_final_kernel(const double *__restrict__ partial, int nparts, int npairs,
+                                                        double p_werner, double *__restrict__ out) {
+  __shared__ double sl[16][16], s[16];
+  __shared__ zd R[16], A[16], U[16], S[16], Rt[16], Tm[16], A1[16], U1[16];
+  __shared__ double w[4], w1[4];
+  const int q = blockIdx.x, t = threadIdx.x, lane = t & 31;
+  {   // slices of the parts, then the slices
+    double v = 0.0;
+    for (int b = t >> 4; b < nparts; b += 16) v += partial[((size_t)q * nparts + b) * 16 + (t & 15)];
+    sl[t >> 4][t & 15] = v;
   }
-  // concurrence: C = max(0, s1 - s2 - s3 - s4), s_i the decreasing square roots of the eigenvalues
-  // of R Rt, Rt = (Y x Y) conj(R) (Y x Y), which are those of the Hermitian sqrt(R) Rt sqrt(R)
-  zd A[16], U[16], S[16], Rt[16], Tm[16];
-  double w[4];
-  for (int i = 0; i < 16; ++i) A[i] = R[i];
-  herm4_eig(A, U, w);
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      zd v = mk<double>(0, 0);
-      for (int m = 0; m < 4; ++m) v = v + sqrt(fmax(w[m], 0.0)) * (U[m * 4 + i] * conj(U[m * 4 + j]));
-      S[j * 4 + i] = v;
+  __syncthreads();
+  if (t < 16) {
+    double v = 0.0;
+    for (int b = 0; b < 16; ++b) v += sl[b][t];
+    s[t] = (1.0 - p_werner) * v;
+  }
+  __syncthreads();
+  double *o = out + (size_t)q * 34;
+  if (t < 16) {
+    const int i = t % 4, j = t / 4, lo = min(i, j), hi = max(i, j);
+    zd v;
+    if (i == j) {
+      v = mk<double>(s[i] + 0.25 * p_werner, 0.0);
+    } else {
+      const int e = 4 + 2 * (lo == 0 ? hi - 1 : (lo == 1 ? hi + 1 : 5));   // (0,1) (0,2) (0,3) (1,2) (1,3) (2,3)
+      v = mk<double>(s[e], i < j ? s[e + 1] : -s[e + 1]);
     }
-  // (Y x Y)_{ab} = -1 for (a, b) in {(0,3), (3,0)}, +1 for {(1,2), (2,1)}, 0 otherwise
-  const int yy_col[4] = {3, 2, 1, 0};
-  const double yy_val[4] = {-1.0, 1.0, 1.0, -1.0};
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      // Rt_ij = sum yy_i,a conj(R_ab) yy_b,j with a = yy_col[i], b = yy_col[j]
-      Rt[j * 4 + i] = (yy_val[i] * yy_val[j]) * conj(R[yy_col[j] * 4 + yy_col[i]]);
+    R[t] = v;
+    o[2 * t] = v.re;
+    o[2 * t + 1] = v.im;
+  }
+  __syncthreads();
+  if (t < 32) {
+    // concurrence: C = max(0, s1 - s2 - s3 - s4), s_i the decreasing square roots of the eigenvalues
+    // of R Rt, Rt = (Y x Y) conj(R) (Y x Y), which are those of the Hermitian sqrt(R) Rt sqrt(R)
+    herm4_eig(R, U, w);
+    if (lane < 16) {
+      const int i = lane % 4, j = lane / 4;
+      // (Y x Y)_{ab} = -1 for (a, b) in {(0,3), (3,0)}, +1 for {(1,2), (2,1)}, 0 otherwise:
+      // Rt_ij = sum yy_i,a conj(R_ab) yy_b,j with a = 3 - i, b = 3 - j
+      const bool neg = (i == 0 || i == 3) != (j == 0 || j == 3);
+      Rt[lane] = (neg ? -1.0 : 1.0) * conj(R[(3 - j) * 4 + 3 - i]);
+      Tm[lane] = sqrt(fmax(w[j], 0.0)) * U[lane];
     }
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      zd v = mk<double>(0, 0);
-      for (int m = 0; m < 4; ++m) v = v + Rt[m * 4 + i] * S[j * 4 + m];
-      Tm[j * 4 + i] = v;   // Rt S
+    __syncwarp();
+    mul4(Tm, U, true, S);
+    mul4(Rt, S, false, Tm);
+    mul4(S, Tm, false, A);
+    if (lane < 16) {
+      const int i = lane % 4, j = lane / 4;
+      const zd x = A[lane], y = A[i * 4 + j];
+      Tm[lane] = mk<double>(0.5 * (x.re + y.re), i == j ? 0.0 : 0.5 * (x.im - y.im));
     }
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      zd v = mk<double>(0, 0);
-      for (int m = 0; m < 4; ++m) v = v + S[m * 4 + i] * Tm[j * 4 + m];
-      A[j * 4 + i] = v;    // S Rt S
+    __syncwarp();
+    herm4_eig(Tm, U, w);
+    const double v = sqrt(fmax(w[lane & 3], 0.0));
+    double big = v, sum = v;
+#pragma unroll
+    for (int x = 1; x <= 2; x <<= 1) {
+      big = fmax(big, __shfl_xor_sync(0xffffffffu, big, x));
+      sum += __shfl_xor_sync(0xffffffffu, sum, x);
     }
-  for (int i = 0; i < 4; ++i)
-    for (int j = i + 1; j < 4; ++j) {
-      const zd h = mk<double>(0.5 * (A[j * 4 + i].re + A[i * 4 + j].re), 0.5 * (A[j * 4 + i].im - A[i * 4 + j].im));
-      A[j * 4 + i] = h;
-      A[i * 4 + j] = conj(h);
+    if (lane == 0) o[32] = fmax(0.0, 2.0 * big - sum);
+  } else if (t < 64) {
+    // negativity: minus the sum of the negative eigenvalues of the partial transpose on spin l:
+    // T[(a0 a1), (b0 b1)] = R[(a0 b1), (b0 a1)]
+    if (lane < 16) {
+      const int a0 = lane & 1, a1 = (lane >> 1) & 1, b0 = (lane >> 2) & 1, b1 = lane >> 3;
+      A1[(2 * b0 + b1) * 4 + (2 * a0 + a1)] = R[(2 * b0 + a1) * 4 + (2 * a0 + b1)];
     }
-  for (int i = 0; i < 4; ++i) A[i * 5].im = 0.0;
-  herm4_eig(A, U, w);
-  const double c = sqrt(fmax(w[0], 0.0)) - sqrt(fmax(w[1], 0.0)) - sqrt(fmax(w[2], 0.0)) - sqrt(fmax(w[3], 0.0));
-  o[32] = fmax(0.0, c);
-  // negativity: minus the sum of the negative eigenvalues of the partial transpose on spin l:
-  // T[(a0 a1), (b0 b1)] = R[(a0 b1), (b0 a1)]
-  for (int a0 = 0; a0 < 2; ++a0)
-    for (int a1 = 0; a1 < 2; ++a1)
-      for (int b0 = 0; b0 < 2; ++b0)
-        for (int b1 = 0; b1 < 2; ++b1) A[(2 * b0 + b1) * 4 + (2 * a0 + a1)] = R[(2 * b0 + a1) * 4 + (2 * a0 + b1)];
-  herm4_eig(A, U, w);
-  double neg = 0.0;
-  for (int i = 0; i < 4; ++i)
-    if (w[i] < 0.0) neg -= w[i];
-  o[33] = neg;
+    __syncwarp();
+    herm4_eig(A1, U1, w1);
+    if (lane == 0) {
+      double neg = 0.0;
+      for (int i = 0; i < 4; ++i)
+        if (w1[i] < 0.0) neg -= w1[i];
+      o[33] = neg;
+    }
+  }
 }
 
 int launch_rdm(bool fp64, const void *V, long long N, int r, const double *lam, const int *pairs, int npairs,
@@ -252,7 +276,7 @@ int launch_rdm(bool fp64, const void *V, long long N, int r, const double *lam, 
 
 void launch_rdm_final(const double *partial, int nparts, int npairs, double p_werner, double *out, cudaStream_t st) {
   ::lrei::count_launch();
-  rdm_final_kernel<<<(npairs + 63) / 64, 64, 0, st>>>(partial, nparts, npairs, p_werner, out);
+  rdm_final_kernel<<<npairs, 256, 0, st>>>(partial, nparts, npairs, p_werner, out);
 }
 
 }  // namespace lrei

@@ -8,6 +8,7 @@
 // is solved in FP32 and then corrected to FP64 accuracy on its top-r
 // invariant subspace (sm_eig_topr), so only r x r Jacobi runs in FP64.
 #include "small.cuh"
+#include "small_dev.cuh"
 
 #include <algorithm>
 
@@ -201,10 +202,8 @@ void sm_trsv(char op, const zd *L, int ldl, int k, zd *B, int ldb, int ncols, cu
 }
 
 // ------------------------------------------------------------- Cholesky
-// Cholesky A = L L^H of a Hermitian k x k matrix (k <= 64) and the inverse of L, in one CTA.  Gaussian elimination on
-// [A | I]: step j takes the multiple A_ij / A_jj of row j off every row i > j, one entry per thread (the entries of
-// the trailing lower triangle and of the inverse's columns c <= j), and the columns are scaled by A_jj^{-1/2} at the
-// end.  An FP64 instruction takes 64 cycles in a dependent chain (a division 445, a square root 690), so the chain of a
+// Cholesky A = L L^H of a Hermitian k x k matrix (k <= 64) and the inverse of L, in one CTA: Gaussian elimination on
+// [A | I] (elim_step), and the columns are scaled by A_jj^{-1/2} at the end.  An FP64 instruction takes 64 cycles in a dependent chain (a division 445, a square root 690), so the chain of a
 // step is one division and one multiply-add group, with the square roots taken together at the end, and the inverse
 // rides along: k = 16 took 33 us with the square root in the chain, and 24 us more for each triangular solve.
 // Column j is dead when its pivot is below tol times a reference: the j-th diagonal entry of `ref` when given (the
@@ -239,33 +238,7 @@ __global__ void __launch_bounds__(256) chol_kernel(const zd *__restrict__ A, int
       deads[j] = dj;
       if (dj) ndead++;
     }
-    const int nrem = k - j - 1, ntri = nrem * (nrem + 1) / 2;
-    if (!dj) {
-      const double inv = 1.0 / piv;
-      // entries 0 .. ntri - 1: the trailing triangle by rows (row a has a + 1 entries); then nrem x (j + 1) of X
-      for (int e = t; e < ntri + nrem * (j + 1); e += nt) {
-        int i, c;
-        zd *dst;
-        zd f;
-        if (e < ntri) {
-          int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-          while ((a + 1) * (a + 2) / 2 <= e) ++a;
-          while (a * (a + 1) / 2 > e) --a;
-          i = j + 1 + a;
-          c = j + 1 + e - a * (a + 1) / 2;
-          dst = Ls + c * k + i;
-          f = conj(Ls[j * k + c]);
-        } else {
-          const int x = e - ntri;
-          i = j + 1 + x % nrem;
-          c = x / nrem;
-          dst = X + c * k + i;
-          f = X[c * k + j];
-        }
-        const zd l = Ls[j * k + i];
-        *dst = *dst - mk<double>(l.re * inv, l.im * inv) * f;
-      }
-    }
+    if (!dj) elim_step(Ls, X, k, j, 1.0 / piv);
     __syncthreads();
   }
   for (int j = t; j < k; j += nt) rs[j] = deads[j] ? 1.0 : 1.0 / sqrt(Ls[j * k + j].re);
