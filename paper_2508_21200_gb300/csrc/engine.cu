@@ -830,9 +830,10 @@ int ts_pass(lrei_ctx *c, TSArgs a, int nsm = 0) {
   a.partial = c->partial;
   a.coef_scratch = c->coef_scratch;
   a.status = c->status_dev;
+  a.red = c->red;
   int g = launch_ts(c->fp64, c->M, a, nsm > 0 ? nsm : c->nsm_use, c->st);
   if (g < 0) return LREI_ERR_ARG;
-  launch_reduce(c->partial, g, (int)ts_partial_doubles(a.gram_left, c->r), c->red, c->st);
+  if (g > 0) launch_reduce(c->partial, g, (int)ts_partial_doubles(a.gram_left, c->r), c->red, c->st);
   return LREI_OK;
 }
 

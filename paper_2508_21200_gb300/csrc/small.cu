@@ -230,6 +230,8 @@ __global__ void __launch_bounds__(256) chol_kernel(const zd *__restrict__ A, int
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (t == 0) { maxdiag = m; ndead = 0; }
   }
+  int ic[ELIM_OWN];
+  elim_own(k, ic);
   __syncthreads();
   for (int j = 0; j < k; ++j) {
     const double piv = Ls[j * k + j].re, refj = ref ? refs[j] : maxdiag;
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(256) chol_kernel(const zd *__restrict__ A, int
       deads[j] = dj;
       if (dj) ndead++;
     }
-    if (!dj) elim_step(Ls, X, k, j, 1.0 / piv);
+    if (!dj) elim_step(Ls, X, k, j, 1.0 / piv, ic);
     __syncthreads();
   }
   for (int j = t; j < k; j += nt) rs[j] = deads[j] ? 1.0 : 1.0 / sqrt(Ls[j * k + j].re);

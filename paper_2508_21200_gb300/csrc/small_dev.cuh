@@ -5,33 +5,31 @@
 namespace lrei {
 
 // Step j of the Gaussian elimination of [A | I] (A Hermitian, its lower triangle in Ls, the identity in X, k x k
-// column-major): the multiple A_ij / A_jj (inv = 1 / A_jj) of row j off every row i > j, one entry per thread: the
-// trailing lower triangle of A and columns c <= j of X.  No barrier.
-__device__ __forceinline__ void elim_step(zd *Ls, zd *X, int k, int j, double inv) {
-  const int nrem = k - j - 1, ntri = nrem * (nrem + 1) / 2;
-  // entries 0 .. ntri - 1: the trailing triangle by rows (row a has a + 1 entries); then nrem x (j + 1) of X
-  for (int e = threadIdx.x; e < ntri + nrem * (j + 1); e += blockDim.x) {
-    int i, c;
-    zd *dst;
-    zd f;
-    if (e < ntri) {
-      int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-      while ((a + 1) * (a + 2) / 2 <= e) ++a;
-      while (a * (a + 1) / 2 > e) --a;
-      i = j + 1 + a;
-      c = j + 1 + e - a * (a + 1) / 2;
-      dst = Ls + c * k + i;
-      f = conj(Ls[j * k + c]);
-    } else {
-      const int x = e - ntri;
-      i = j + 1 + x % nrem;
-      c = x / nrem;
-      dst = X + c * k + i;
-      f = X[c * k + j];
-    }
-    const zd l = Ls[j * k + i];
+// column-major): the multiple A_ij / A_jj (inv = 1 / A_jj) of row j off every row i > j: entry (i, c), c <= i, of A
+// where c > j and of X where c <= j.  Thread t owns the entries t, t + blockDim, ... of the lower triangle by rows in
+// every step, ic[] holds the first ELIM_OWN of them (i << 16 | c).  No barrier.
+constexpr int ELIM_OWN = 3;
+__device__ __forceinline__ int tri_entry(int e) {   // row i has the entries i (i + 1) / 2 + c
+  int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+  while ((i + 1) * (i + 2) / 2 <= e) ++i;
+  while (i * (i + 1) / 2 > e) --i;
+  return i << 16 | (e - i * (i + 1) / 2);
+}
+__device__ __forceinline__ void elim_own(int k, int *ic) {
+#pragma unroll
+  for (int x = 0; x < ELIM_OWN; ++x) ic[x] = tri_entry(threadIdx.x + x * blockDim.x);   // rows >= k: none
+}
+__device__ __forceinline__ void elim_step(zd *Ls, zd *X, int k, int j, double inv, const int *ic) {
+  auto entry = [&](int v) {
+    const int i = v >> 16, c = v & 0xffff;
+    if (i <= j || i >= k) return;
+    zd *dst = (c > j ? Ls : X) + c * k + i;
+    const zd f = c > j ? conj(Ls[j * k + c]) : X[c * k + j], l = Ls[j * k + i];
     *dst = *dst - mk<double>(l.re * inv, l.im * inv) * f;
-  }
+  };
+#pragma unroll
+  for (int x = 0; x < ELIM_OWN; ++x) entry(ic[x]);
+  for (int e = threadIdx.x + ELIM_OWN * blockDim.x; e < k * (k + 1) / 2; e += blockDim.x) entry(tri_entry(e));
 }
 
 // X = L^{-1} for A = L L^H (k x k, leading dimension lda, positive definite: a pivot counts as at least 1e-300), by the
@@ -41,9 +39,11 @@ __device__ __forceinline__ void chol_inv_cta(const zd *A, int lda, int k, zd *Ls
     Ls[e] = A[(size_t)(e / k) * lda + e % k];
     X[e] = mk<double>(e % k == e / k ? 1.0 : 0.0, 0);
   }
+  int ic[ELIM_OWN];
+  elim_own(k, ic);
   __syncthreads();
   for (int j = 0; j < k; ++j) {
-    elim_step(Ls, X, k, j, 1.0 / fmax(Ls[j * k + j].re, 1e-300));
+    elim_step(Ls, X, k, j, 1.0 / fmax(Ls[j * k + j].re, 1e-300), ic);
     __syncthreads();
   }
   // row i of X by A_ii^{-1/2}: all rows' roots in parallel, in the imaginary parts of the pivots

@@ -817,15 +817,27 @@ __global__ void coef_convert_kernel(const zd *coefQ, const zd *coefS, int nq, in
   }
 }
 
-__global__ void reduce_kernel(const double *__restrict__ part, int nparts, int len, double *__restrict__ out) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < len; e += gridDim.x * blockDim.x) {
-    double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    int p = 0;
-    for (; p + 8 <= nparts; p += 8)
+// out = the sum of the parts: 16 entries per CTA, the parts in 32 slices, then the slices, in a fixed order.  Latency:
+// an FP64 addition takes a scheduler 64 cycles, so a thread adds nparts / 32 values.  (Slices by one kernel and their
+// sum by another, 16 slices: 9.2 + 5.8 us with 148 parts at r = 8.)
+__global__ void __launch_bounds__(512) reduce_kernel(const double *__restrict__ part, int nparts, int len,
+                                                     double *__restrict__ out) {
+  __shared__ double red[32][17];
+  const int t = threadIdx.x, e = blockIdx.x * 16 + (t & 15);
+  double v = 0.0;
+  if (e < len) {
+#pragma unroll 4
+    for (int p = t >> 4; p < nparts; p += 32) v += part[(size_t)p * len + e];
+  }
+  red[t >> 4][t & 15] = v;
+  __syncthreads();
+  if (t < 64) {
+    v = 0.0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) s[u] += part[(size_t)(p + u) * len + e];
-    for (; p < nparts; ++p) s[0] += part[(size_t)p * len + e];
-    out[e] = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+    for (int x = 0; x < 8; ++x) v += red[(t & 3) * 8 + x][t >> 2];
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if ((t & 3) == 0 && blockIdx.x * 16 + (t >> 2) < len) out[blockIdx.x * 16 + (t >> 2)] = v;
   }
 }
 
@@ -989,8 +1001,87 @@ static int launch_ts_t(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_
   return grid;
 }
 
+// ------------------------------------------- few rows
+// Passes of few rows are latency: tiles leave most SMs idle (one CTA per 256 rows in the complex128 pass) and their sums need
+// a second launch.  Here every entry of the new block is a sum over eight lanes and every Gram entry one over a warp
+// or a CTA, in FP64 for both precisions (the coefficients as they are), and the Gram goes to a.red directly.
+// The rows of a CTA are read before one is written, so the new block may replace an input.
+template <typename T>
+__global__ void __launch_bounds__(256) few_new_kernel(TSArgs a) {
+  const int r = a.r, rows = 32 / r, o = threadIdx.x >> 3, q = threadIdx.x & 7, j = o % r;
+  const long long row = (long long)blockIdx.x * rows + o / r;
+  const bool in = o < rows * r && row < a.N;
+  const int K = (a.nq + (a.mode == 1 ? 1 : 0)) * r;
+  zd s = mk<double>(0, 0);
+  if (in)
+    for (int k = q; k < K; k += 8) {
+      const int m = k / r, i = k % r;
+      const cx<T> x = reinterpret_cast<const cx<T> *>(m < a.nq ? a.q[m] : a.src)[(size_t)row * r + i];
+      const zd c = m < a.nq ? (a.coefQ ? a.coefQ[(size_t)j * a.nq * r + k] : mk<double>(0, 0))
+                            : (a.coefS ? a.coefS[(size_t)j * r + i] : mk<double>(0, 0));
+      fma_(s, cvt<double>(x), c);
+    }
+#pragma unroll
+  for (int x = 4; x > 0; x >>= 1) {
+    s.re += __shfl_xor_sync(0xffffffffu, s.re, x);
+    s.im += __shfl_xor_sync(0xffffffffu, s.im, x);
+  }
+  __syncthreads();
+  if (in && q == 0)
+    reinterpret_cast<cx<T> *>(a.out)[(size_t)row * r + j] = row < a.zero_rows ? mk<T>(0, 0) : cvt<T>(s);
+}
+
+// TPE threads per entry, 128 per CTA.
+template <typename T, int TPE>
+__global__ void __launch_bounds__(128) few_gram_kernel(TSArgs a, const cx<T> *__restrict__ G) {
+  __shared__ zd part[4];
+  const int r = a.r, ldg = (a.gram_left + 1) * r, t = threadIdx.x % TPE;
+  const int e = blockIdx.x * (128 / TPE) + threadIdx.x / TPE, j = e / ldg, row = e % ldg, m = row / r, i = row % r;
+  zd s = mk<double>(0, 0);
+  if (e < ldg * r) {
+    const cx<T> *L = m < a.gram_left ? reinterpret_cast<const cx<T> *>(a.q[m]) : G;
+#pragma unroll 4
+    for (int b = t; b < (int)a.N; b += TPE) fmac_(s, cvt<double>(L[(size_t)b * r + i]), cvt<double>(G[(size_t)b * r + j]));
+  }
+#pragma unroll
+  for (int x = 16; x > 0; x >>= 1) {
+    s.re += __shfl_xor_sync(0xffffffffu, s.re, x);
+    s.im += __shfl_xor_sync(0xffffffffu, s.im, x);
+  }
+  if (TPE > 32) {
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = (part[0] + part[1]) + (part[2] + part[3]);
+  }
+  if (t == 0 && e < ldg * r) reinterpret_cast<zd *>(a.red)[e] = s;
+}
+
+// Up to 4096 rows and 2^20 multiply-adds per Gram, where these launches take less than the tiles' shortest:
+// FP64 at n = 8, r = 4, 5 blocks: Gram 24 us as tiles and their sum, 4 here; projection and Gram 20, 8 here.
+template <typename T> static bool launch_few(const TSArgs &a, cudaStream_t st) {
+  const int g = a.gram_left + 1;
+  if (!a.red || a.apply_h || a.N > 4096 || a.N * g * a.r * a.r > (1 << 20) || a.nq + 1 > MAXB + 1) return false;
+  if (a.mode == 0 ? a.out != nullptr : a.out == nullptr) return false;
+  if (a.mode != 2 && !a.src) return false;
+  if (a.mode != 0)
+    for (int m = 0; m < a.gram_left; ++m)
+      if (a.q[m] == a.out) return false;
+  const cx<T> *G = reinterpret_cast<const cx<T> *>(a.mode == 0 ? a.src : a.out);
+  if (a.mode != 0) {
+    const int rows = 32 / a.r;
+    ::lrei::count_launch();
+    few_new_kernel<T><<<(int)((a.N + rows - 1) / rows), 256, 0, st>>>(a);
+  }
+  const int entries = g * a.r * a.r;
+  ::lrei::count_launch();
+  if (a.N <= 512) few_gram_kernel<T, 32><<<(entries + 3) / 4, 128, 0, st>>>(a, G);
+  else few_gram_kernel<T, 128><<<entries, 128, 0, st>>>(a, G);
+  return true;
+}
+
 int launch_ts(bool fp64, const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_t st) {
   if (a.nq > MAXB || a.gram_left > a.nq || a.r < 1 || a.r > MAX_R) return -1;
+  if (fp64 ? launch_few<double>(a, st) : launch_few<float>(a, st)) return 0;
   if (fp64) {
     const int n = launch_tsx(a, nsm, st);
     if (n > 0) return n;
@@ -998,39 +1089,9 @@ int launch_ts(bool fp64, const ModelArgs &M, const TSArgs &a, int nsm, cudaStrea
   return fp64 ? launch_ts_t<double>(M, a, nsm, st) : launch_ts_t<float>(M, a, nsm, st);
 }
 
-// Two-stage deterministic reduction: CTAs (entry chunk, part slice) sum a fixed slice of parts,
-// then one pass sums the slices in order.
-__global__ void reduce_slices_kernel(const double *__restrict__ part, int nparts, int len, int nslice,
-                                     double *__restrict__ tmp) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sl = blockIdx.y;
-  if (e >= len) return;
-  const int per = (nparts + nslice - 1) / nslice;
-  const int p0 = sl * per, p1 = min(nparts, p0 + per);
-  double s[4] = {0, 0, 0, 0};
-  int p = p0;
-  for (; p + 4 <= p1; p += 4)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) s[u] += part[(size_t)(p + u) * len + e];
-  for (; p < p1; ++p) s[0] += part[(size_t)p * len + e];
-  tmp[(size_t)sl * len + e] = (s[0] + s[1]) + (s[2] + s[3]);
-}
-
 void launch_reduce(const double *partial, int nparts, int len_doubles, double *out, cudaStream_t st) {
-  const int nslice = nparts >= 64 ? 16 : 1;
-  if (nslice == 1) {
-    int blocks = (len_doubles + 255) / 256;
-    ::lrei::count_launch();
-    reduce_kernel<<<blocks, 256, 0, st>>>(partial, nparts, len_doubles, out);
-    return;
-  }
-  // the slices live after the partials of the largest grid (ts_max_grid(nsm) parts), which the
-  // caller sized with room for nslice extra rows
-  double *tmp = const_cast<double *>(partial) + (size_t)nparts * len_doubles;
-  dim3 g((len_doubles + 127) / 128, nslice);
-  ::lrei::count_launch(2);
-  reduce_slices_kernel<<<g, 128, 0, st>>>(partial, nparts, len_doubles, nslice, tmp);
-  reduce_kernel<<<(len_doubles + 255) / 256, 256, 0, st>>>(tmp, nslice, len_doubles, out);
+  ::lrei::count_launch();
+  reduce_kernel<<<(len_doubles + 15) / 16, 512, 0, st>>>(partial, nparts, len_doubles, out);
 }
 
 void launch_hv(bool fp64, const ModelArgs &M, const void *X, void *Y, long long N, int r, int nsm, cudaStream_t st,

@@ -29,9 +29,10 @@ struct TSArgs {
   void *coef_scratch;   // device, >= (MAXB+1)*MAX_R*MAX_R*16 bytes (converted coefficients)
   long long zero_rows;  // modes 1, 2: rows < zero_rows of the new block are set to zero
   int *status;          // device status word (may be NULL)
+  double *red = nullptr;   // where the sum of the partials goes (may be NULL)
 };
 
-// Returns the grid size used (number of partials written), or -1 on error.
+// Returns the grid size used (number of partials written), 0 when the sums already are in a.red, or -1 on error.
 int launch_ts(bool fp64, const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_t st);
 int ts_max_grid(int nsm);
 int ts_init();
