@@ -127,21 +127,33 @@ __global__ void stage_xwz_kernel(const zd *__restrict__ G, int r, const double *
     if (i == j) g.im = 0.0;
     gcol[i] = g;
     xcol[i] = x11_factor(lam[i], lam[j], kappa, model) * g;
+    if (blockIdx.y) continue;
     X11[(size_t)j * r + i] = xcol[i];
     if (Gh) Gh[(size_t)j * r + i] = g;
   }
   __syncthreads();
   const zd cc = conj(c_factor(lam[j], kappa, model));
-  for (int row = threadIdx.x; row < K; row += blockDim.x) {
-    zd yg = mk<double>(0, 0), yx = mk<double>(0, 0);
-    for (int i = 0; i < r; ++i) {
-      const zd y = Y[(size_t)i * ld + row];
-      fma_(yg, y, gcol[i]);
-      fma_(yx, y, xcol[i]);
+  // eight lanes (4 parts x re, im) per row, 32 rows per CTA: the sums are chains of FP64 instructions of 64 cycles
+  const int row = blockIdx.y * 32 + (threadIdx.x >> 3), cm = threadIdx.x & 1, q = (threadIdx.x >> 1) & 3;
+  double yg = 0.0, yx = 0.0;
+  if (row < K)
+    for (int i = q; i < r; i += 4) {
+      const zd y = Y[(size_t)i * ld + row], g = gcol[i], x = xcol[i];
+      yg = fma(y.re, cm ? g.im : g.re, fma(cm ? y.im : -y.im, cm ? g.re : g.im, yg));
+      yx = fma(y.re, cm ? x.im : x.re, fma(cm ? y.im : -y.im, cm ? x.re : x.im, yx));
     }
-    const zd w = (T[(size_t)j * ld + row] - yg) * cc;
-    W[(size_t)j * ld + row] = w;
-    Z[(size_t)j * ld + row] = yx + w;
+#pragma unroll
+  for (int o = 2; o <= 4; o <<= 1) {
+    yg += __shfl_xor_sync(0xffffffffu, yg, o);
+    yx += __shfl_xor_sync(0xffffffffu, yx, o);
+  }
+  double d = 0.0;
+  if (row < K) d = reinterpret_cast<const double *>(T + (size_t)j * ld + row)[cm] - yg;
+  const double od = __shfl_xor_sync(0xffffffffu, d, 1);   // the other component
+  if (row < K && q == 0) {
+    const double w = cm ? fma(od, cc.im, d * cc.re) : fma(d, cc.re, -od * cc.im);
+    reinterpret_cast<double *>(W + (size_t)j * ld + row)[cm] = w;
+    reinterpret_cast<double *>(Z + (size_t)j * ld + row)[cm] = yx + w;
   }
 }
 
@@ -376,8 +388,7 @@ __global__ void __launch_bounds__(512) obs_final_kernel(const double *__restrict
       out[48 + i] = p * inv_n + (1.0 - p) * lams[i];
     }
 }
-// Threads: an entry each in the elementwise part.
-static int obs_final_threads(int r) { return r * r >= 512 ? 512 : (r * r < 64 ? 64 : (r * r + 31) / 32 * 32); }
+static int obs_final_threads(int r) { return std::max(64, eliminate_threads(r)); }
 
 // ----------------------------------------------------------- controller features
 // ||[rho, H]||_F^2 = 2 Tr(Lambda^2 V^*H^2V) - 2 Tr(Lambda G Lambda G); in the Krylov frame H V_1 has
@@ -889,8 +900,8 @@ void enqueue_stage(lrei_ctx *c, const Tableau &tb, int j, cudaStream_t st2) {
   sm_gemm('N', 'N', K, r, b, ONE, c->Tbar, KM, c->ys[j], KM, ZERO, c->ts, KM, st2);
   sm_gemm('C', 'N', r, r, b, ONE, c->ys[j], KM, c->ts, KM, ZERO, c->G, r, st2);
   ::lrei::count_launch();
-  stage_xwz_kernel<<<r, 128, 2 * r * sizeof(zd), st2>>>(c->G, r, c->lam0_dev, c->kappa, c->model, c->ys[j], c->ts, K,
-                                                        KM, c->X11, c->zs[j], c->wsv[j], j == 0 ? c->Gh : nullptr);
+  stage_xwz_kernel<<<dim3(r, (K + 31) / 32), 256, 2 * r * sizeof(zd), st2>>>(
+      c->G, r, c->lam0_dev, c->kappa, c->model, c->ys[j], c->ts, K, KM, c->X11, c->zs[j], c->wsv[j], j == 0 ? c->Gh : nullptr);
   if (j == 0) {
     ::lrei::count_launch();
     feat_comm_kernel<<<1, 256, 0, st2>>>(c->ts, K, KM, c->Gh, r, c->lam0_dev, c->feat_dev);
@@ -1183,7 +1194,7 @@ int enqueue_ab_step(lrei_ctx *c, int m) {
     sm_gemm('N', 'N', K, r, r, ONE, vb, KM, c->Ainv, r, ZERO, c->ys[l], KM, st);
     sm_gemm('N', 'N', K, r, r, ONE, yb, KM, c->Ainv, r, ZERO, c->tys[l], KM, st);
     sm_gemm('C', 'N', r, r, K, ONE, c->ys[l], KM, c->tys[l], KM, ZERO, c->G, r, st);
-    ::lrei::count_launch(); stage_xwz_kernel<<<r, 128, 2 * r * sizeof(zd), st>>>(c->G, r, c->lam0_dev, c->kappa, c->model, c->ys[l],
+    ::lrei::count_launch(); stage_xwz_kernel<<<dim3(r, (K + 31) / 32), 256, 2 * r * sizeof(zd), st>>>(c->G, r, c->lam0_dev, c->kappa, c->model, c->ys[l],
                                                          c->tys[l], K, KM, c->X11, c->zs[l], c->wsv[l],
                                                          l == 0 ? c->Gh : nullptr);
   }

@@ -203,47 +203,42 @@ void sm_trsv(char op, const zd *L, int ldl, int k, zd *B, int ldb, int ncols, cu
 
 // ------------------------------------------------------------- Cholesky
 // Cholesky A = L L^H of a Hermitian k x k matrix (k <= 64) and the inverse of L, in one CTA: Gaussian elimination on
-// [A | I] (elim_step), and the columns are scaled by A_jj^{-1/2} at the end.  An FP64 instruction takes 64 cycles in a dependent chain (a division 445, a square root 690), so the chain of a
-// step is one division and one multiply-add group, with the square roots taken together at the end, and the inverse
-// rides along: k = 16 took 33 us with the square root in the chain, and 24 us more for each triangular solve.
-// Column j is dead when its pivot is below tol times a reference: the j-th diagonal entry of `ref` when given (the
+// [A | I] (eliminate), and the columns are scaled by A_jj^{-1/2} at the end.  The inverse rides along in the chain of the
+// steps (a triangular solve of its own took 24 us at k = 16).
+// Column j is dead when its pivot is not above tol times a reference: the j-th diagonal entry of `ref` when given (the
 // squared norm of the raw column), else the largest diagonal entry of A.  A dead column gets L[j][j] = 1 and a zero
 // sub-column (and, with zero_row, a zero row).
-__global__ void __launch_bounds__(256) chol_kernel(const zd *__restrict__ A, int lda, int k, zd *__restrict__ Lout, int ldl,
+__global__ void __launch_bounds__(512) chol_kernel(const zd *__restrict__ A, int lda, int k, zd *__restrict__ Lout, int ldl,
                                                    zd *__restrict__ Iout, int ldi, int inv_h, zd *__restrict__ Rc, int ldrc, double tol,
                                                    int zero_row, int *dead, int *status, int flag_rank,
                                                    const zd *__restrict__ ref, int ldref) {
   extern __shared__ zd Ls[];   // k x k: A's lower triangle, then L before scaling; and k x k: the inverse before scaling
   zd *X = Ls + (size_t)k * k;
-  __shared__ double maxdiag, rs[64], refs[64];
-  __shared__ int deads[64], ndead;
+  __shared__ double rs[64], tolref[64], inv[64];
+  __shared__ int deads[64];
   const int t = threadIdx.x, nt = blockDim.x;
   for (int e = t; e < k * k; e += nt) {
     const int i = e % k, j = e / k;
     Ls[e] = (i >= j) ? A[(size_t)j * lda + i] : mk<double>(0, 0);
     X[e] = mk<double>(i == j ? 1.0 : 0.0, 0);
   }
-  for (int i = t; i < k; i += nt) refs[i] = ref ? ref[(size_t)i * ldref + i].re : 0.0;
   if (t < 32) {
     double m = 0.0;
-    for (int i = t; i < k; i += 32) m = fmax(m, A[(size_t)i * lda + i].re);
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (t == 0) { maxdiag = m; ndead = 0; }
-  }
-  int ic[ELIM_OWN];
-  elim_own(k, ic);
-  __syncthreads();
-  for (int j = 0; j < k; ++j) {
-    const double piv = Ls[j * k + j].re, refj = ref ? refs[j] : maxdiag;
-    const bool dj = !(piv > tol * refj) || !isfinite(piv) || !(refj > 0.0);
-    if (t == 0) {
-      deads[j] = dj;
-      if (dj) ndead++;
+    if (!ref) {
+      for (int i = t; i < k; i += 32) m = fmax(m, A[(size_t)i * lda + i].re);
+      // not negative: ordered as integers, which run at full rate
+      unsigned long long b = __double_as_longlong(m);
+      for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+      m = __longlong_as_double(b);
     }
-    if (!dj) elim_step(Ls, X, k, j, 1.0 / piv, ic);
-    __syncthreads();
+    for (int i = t; i < k; i += 32) {
+      const double r = ref ? ref[(size_t)i * ldref + i].re : m;
+      tolref[i] = r > 0.0 ? tol * r : __longlong_as_double(0x7ff0000000000000ll);   // no positive reference: dead
+    }
   }
-  for (int j = t; j < k; j += nt) rs[j] = deads[j] ? 1.0 : 1.0 / sqrt(Ls[j * k + j].re);
+  __syncthreads();
+  eliminate(Ls, X, k, tolref, inv, deads);
+  for (int j = t; j < k; j += nt) rs[j] = deads[j] ? 1.0 : newton_rsqrt(Ls[j * k + j].re);
   __syncthreads();
   for (int e = t; e < k * k; e += nt) {
     const int i = e % k, j = e / k;
@@ -267,13 +262,15 @@ __global__ void __launch_bounds__(256) chol_kernel(const zd *__restrict__ A, int
   }
   if (dead)
     for (int j = t; j < k; j += nt) dead[j] = deads[j];
-  if (t == 0 && ndead > 0 && flag_rank && status) atomicOr(status, ST_RANK);
+  if (flag_rank && status)
+    for (int j = t; j < k; j += nt)
+      if (deads[j]) atomicOr(status, ST_RANK);
 }
 
 void sm_chol(const zd *A, int lda, int k, zd *L, int ldl, double tol, int zero_row, int *dead, int *status,
              int flag_rank, cudaStream_t st, const zd *ref, int ldref, zd *Linv, int ldi, int inv_h, zd *Rc, int ldrc) {
   ::lrei::count_launch();
-  chol_kernel<<<1, 256, 2 * (size_t)k * k * sizeof(zd), st>>>(A, lda, k, L, ldl, Linv, ldi, inv_h, Rc, ldrc, tol, zero_row, dead,
+  chol_kernel<<<1, eliminate_threads(k), 2 * (size_t)k * k * sizeof(zd), st>>>(A, lda, k, L, ldl, Linv, ldi, inv_h, Rc, ldrc, tol, zero_row, dead,
                                                               status, flag_rank, ref, ldref);
 }
 
