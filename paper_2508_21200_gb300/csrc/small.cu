@@ -290,13 +290,6 @@ __device__ __forceinline__ void round_pair(int pos, int round, int kp, int *p, i
   *p = min(a, b);
   *q = max(a, b);
 }
-template <typename T> __device__ __forceinline__ cx<T> tri_get(const cx<T> *A, int ld, int i, int j) {
-  return i <= j ? A[j * ld + i] : conj(A[i * ld + j]);
-}
-template <typename T> __device__ __forceinline__ void tri_put(cx<T> *A, int ld, int i, int j, cx<T> v) {
-  if (i <= j) A[j * ld + i] = v;
-  else A[i * ld + j] = conj(v);
-}
 // item e of the pairs of positions a < b, e = b (b - 1) / 2 + a; with diag = 1 of a <= b, e = b (b + 1) / 2 + a
 __device__ __forceinline__ void tri_item(int e, int *a, int *b, int diag = 0) {
   int y = (int)((sqrtf(8.f * (float)e + 1.f) + 1.f) * 0.5f);
@@ -306,49 +299,77 @@ __device__ __forceinline__ void tri_item(int e, int *a, int *b, int diag = 0) {
   *a = e - y * (y - 1) / 2;
 }
 
-constexpr int J32_ITEMS = 8;        // pairs of pairs per thread: enough for k = 162, where A fills the shared memory
 constexpr int J32_SWEEPS = 12;
 constexpr int J32_KMAX = 162;
 
-// FP32.  A round is latency: the angle, the blocks, two barriers.  The eigenvectors are not accumulated here: the
-// rotations (c, s, p | q << 16) of every round go to rots, and replay_kernel applies them to the rows of U on many SMs.
-// The odd leading dimension keeps mirrored (row-wise) accesses free of bank conflicts.
-// order[i]: rank of diagonal entry i in decreasing order.
+// The storage is by position in the tournament, not by row: pair a of every round is the positions (a, kp - 1 - a), and a
+// round writes its results where the next one reads them: position x moves to x - 1 (1 to kp - 1, 0 stays), so
+// all addresses are the same in every round, and after a sweep (kp - 1 rounds) every row is back in its place.
+__device__ __forceinline__ int next_pos(int x, int kp) { return x == 0 ? 0 : (x == 1 ? kp - 1 : x - 1); }
+__device__ __forceinline__ int tri_at(int x, int y) { return (y * (y + 1) >> 1) + x; }   // x <= y
+
+// FP32.  A round is a chain of instructions in few warps: the pairs' angles, a barrier, the 2 x 2 blocks of pairs a <= b
+// (one thread each, the addresses of its first J32_OWN blocks in registers), a barrier.  The matrix is read from one
+// buffer and written to the other.  The eigenvectors are not accumulated here: the rotations (c, s) of every round go
+// to rots, and replay_kernel applies them to the rows of U on many SMs.  order[i]: rank of diagonal entry i in decreasing order.
+// A round takes 0.35 us at k = 16, 0.53 at k = 40, 0.92 at k = 80, 4.0 at k = 160; by row indices and in place 0.65 at k = 40.
+// (Four threads per block, an entry each: 0.38, 0.53 at k = 40, 0.97 at k = 64 against 0.77; the angles by every block's
+// thread, without the first barrier: 0.9 at k = 16.)
+constexpr int J32_OWN = 2;
 __global__ void __launch_bounds__(512) jacobi32_kernel(const zd *__restrict__ Ain, int lda, int k, double *__restrict__ wout,
                                                        int *__restrict__ order, float4 *__restrict__ rots,
                                                        int *__restrict__ meta, float tol) {
   extern __shared__ __align__(16) unsigned char sm[];
-  const int kp = k + (k & 1), ld = kp + 1, np = kp / 2, nitem = np * (np - 1) / 2;
-  float4 *rot = reinterpret_cast<float4 *>(sm);
-  cx<float> *A = reinterpret_cast<cx<float> *>(rot + np);    // upper triangle
-  __shared__ float red[2][16];
+  const int kp = k + (k & 1), np = kp / 2, nitem = np * (np + 1) / 2, ntri = kp * (kp + 1) / 2;
+  cx<float> *A = reinterpret_cast<cx<float> *>(sm), *B = A + ntri;    // upper triangles: read, written
+  __shared__ float red[2][32];
+  __shared__ float4 rot[J32_KMAX / 2];
   const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wp = t >> 5;
-  for (int e = t; e < kp * kp; e += nt) {
-    const int i = e % kp, j = e / kp;
-    cx<float> v = mk<float>(0.f, 0.f);
-    if (i < k && j < k && i <= j) v = cvt<float>(Ain[(size_t)j * lda + i]);
-    A[j * ld + i] = v;
-  }
-  int item[J32_ITEMS];
+  for (int j = wp; j < kp; j += nt / 32)
+    for (int i = lane; i <= j; i += 32) A[tri_at(i, j)] = j < k ? cvt<float>(Ain[(size_t)j * lda + i]) : mk<float>(0.f, 0.f);
+  // where entry (x, y), x <= y, goes; the sign bit: conjugated
+  auto dst = [&](int x, int y) {
+    const int u = next_pos(x, kp), v = next_pos(y, kp);
+    return u <= v ? tri_at(u, v) : (int)(tri_at(v, u) | 0x80000000);
+  };
+  struct Block {
+    int a, b, w[4];   // where the entries (pa, pb), (pa, qb), (pb, qa), (qb, qa) go
+  };
+  auto make_block = [&](int e) {
+    Block I;
+    tri_item(e < nitem ? e : 0, &I.a, &I.b, 1);
+    const int qa = kp - 1 - I.a, qb = kp - 1 - I.b;
+    I.w[0] = dst(I.a, I.b);
+    I.w[1] = dst(I.a, qb);
+    I.w[2] = dst(I.b, qa);
+    I.w[3] = dst(qb, qa);
+    return I;
+  };
+  Block own[J32_OWN];
 #pragma unroll
-  for (int x = 0; x < J32_ITEMS; ++x) {
-    int a = 0, b = 0;
-    if (t + x * nt < nitem) tri_item(t + x * nt, &a, &b);
-    item[x] = a | b << 16;
+  for (int x = 0; x < J32_OWN; ++x) own[x] = make_block(t + x * nt);
+  int p1 = 0, p2 = 0, p3 = 0;      // pair t: A_pp, A_qq, A_pq
+  if (t < np) {
+    p1 = tri_at(t, t);
+    p2 = tri_at(kp - 1 - t, kp - 1 - t);
+    p3 = tri_at(t, kp - 1 - t);
   }
   if (t < META_INTS) meta[t] = 0;
   __syncthreads();
+  auto put = [&](int i, cx<float> v) {
+    if (i < 0) v.im = -v.im;
+    B[i & 0x7fffffff] = v;
+  };
   int rounds = 0, sweeps = 0;
   for (; sweeps < J32_SWEEPS; ++sweeps) {
     // convergence test: off-diagonal vs total Frobenius norm
     float off = 0.f, tot = 0.f;
-    for (int e = t; e < kp * kp; e += nt) {
-      const int i = e % kp, j = e / kp;
-      if (i > j) continue;
-      const float v = norm2(A[j * ld + i]);
-      if (i == j) tot += v;
-      else off += 2.f * v;
-    }
+    for (int j = wp; j < kp; j += nt / 32)
+      for (int i = lane; i <= j; i += 32) {
+        const float v = norm2(A[tri_at(i, j)]);
+        if (i == j) tot += v;
+        else off += 2.f * v;
+      }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       off += __shfl_xor_sync(0xffffffffu, off, o);
@@ -356,55 +377,60 @@ __global__ void __launch_bounds__(512) jacobi32_kernel(const zd *__restrict__ Ai
     }
     if (lane == 0) { red[0][wp] = off; red[1][wp] = tot; }
     __syncthreads();
-    off = tot = 0.f;
-    for (int w = 0; w < nt / 32; ++w) { off += red[0][w]; tot += red[1][w]; }
+    off = lane < nt / 32 ? red[0][lane] : 0.f;
+    tot = lane < nt / 32 ? red[1][lane] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    }
     tot += off;
     if (off <= tol * tol * tot || !(tot == tot)) break;
     for (int round = 0; round < kp - 1; ++round, ++rounds) {
-      for (int pi = t; pi < np; pi += nt) {
-        int p, q;
-        round_pair(pi, round, kp, &p, &q);
-        const cx<float> b = A[q * ld + p];
-        const float n2 = norm2(b), a = A[p * ld + p].re, d = A[q * ld + q].re;
-        float c = 1.f, f = 0.f;
-        if (n2 > 1e-37f) {   // tan = f |b| with f = sign(d - a) / (|h| + sqrt(h^2 + |b|^2)), h = (d - a) / 2
-          const float h = 0.5f * (d - a), g = fmaf(h, h, n2);
-          f = copysignf(__fdividef(1.f, fabsf(h) + g * rsqrtf(g)), h);
-          c = rsqrtf(fmaf(n2 * f, f, 1.f));
-          A[p * ld + p] = mk<float>(fmaf(-f, n2, a), 0.f);   // the pair's own block: A_pp - tan |b|, A_qq + tan |b|, 0
-          A[q * ld + q] = mk<float>(fmaf(f, n2, d), 0.f);
-          A[q * ld + p] = mk<float>(0.f, 0.f);
-        }
-        const float4 R = make_float4(c, c * f * b.re, c * f * b.im, __int_as_float(p | q << 16));
-        rot[pi] = R;
-        rots[(size_t)rounds * np + pi] = R;
+      if (t < np) {   // tan = f |b|, f = sign(d - a) / (|h| + sqrt(h^2 + |b|^2)), h = (d - a) / 2
+        const cx<float> b = A[p3];
+        const float n2 = norm2(b), h = 0.5f * (A[p2].re - A[p1].re), g = fmaxf(fmaf(h, h, n2), 1e-37f);
+        const float f = n2 > 1e-37f ? copysignf(__fdividef(1.f, fabsf(h) + g * rsqrtf(g)), h) : 0.f;
+        const float c = rsqrtf(fmaf(n2 * f, f, 1.f)), cf = c * f;
+        const float4 R = make_float4(c, cf * b.re, cf * b.im, f * n2);
+        rot[t] = R;
+        rots[(size_t)rounds * np + t] = R;
       }
       __syncthreads();
-#pragma unroll
-      for (int x = 0; x < J32_ITEMS; ++x)
-        if (t + x * nt < nitem) {
-          const float4 Ra = rot[item[x] & 0xffff], Rb = rot[item[x] >> 16];
-          const int pa = __float_as_int(Ra.w) & 0xffff, qa = __float_as_int(Ra.w) >> 16;
-          const int pb = __float_as_int(Rb.w) & 0xffff, qb = __float_as_int(Rb.w) >> 16;
-          const cx<float> sa = mk<float>(Ra.y, Ra.z), sb = mk<float>(Rb.y, Rb.z);
-          const cx<float> x00 = tri_get(A, ld, pa, pb), x10 = tri_get(A, ld, qa, pb), x01 = tri_get(A, ld, pa, qb),
-                          x11 = tri_get(A, ld, qa, qb);
-          const cx<float> y00 = Rb.x * x00 - conj(sb) * x01, y01 = sb * x00 + Rb.x * x01;    // Y = X J_b
-          const cx<float> y10 = Rb.x * x10 - conj(sb) * x11, y11 = sb * x10 + Rb.x * x11;
-          tri_put(A, ld, pa, pb, Ra.x * y00 - sa * y10);                                     // X' = J_a^H Y
-          tri_put(A, ld, pa, qb, Ra.x * y01 - sa * y11);
-          tri_put(A, ld, qa, pb, conj(sa) * y00 + Ra.x * y10);
-          tri_put(A, ld, qa, qb, conj(sa) * y01 + Ra.x * y11);
+      auto block = [&](const Block &I) {
+        const int pa = I.a, qa = kp - 1 - I.a, pb = I.b, qb = kp - 1 - I.b;
+        const float4 Ra = rot[pa], Rb = rot[pb];
+        if (pa == pb) {
+          put(I.w[0], mk<float>(A[tri_at(pa, pa)].re - Ra.w, 0.f));
+          put(I.w[1], mk<float>(0.f, 0.f));
+          put(I.w[3], mk<float>(A[tri_at(qa, qa)].re + Ra.w, 0.f));
+          return;
         }
+        const cx<float> x00 = A[tri_at(pa, pb)], x01 = A[tri_at(pa, qb)], x10 = conj(A[tri_at(pb, qa)]), x11 = conj(A[tri_at(qb, qa)]);
+        const cx<float> sa = mk<float>(Ra.y, Ra.z), sb = mk<float>(Rb.y, Rb.z);
+        const cx<float> y00 = Rb.x * x00 - conj(sb) * x01, y01 = sb * x00 + Rb.x * x01;    // Y = X J_b
+        const cx<float> y10 = Rb.x * x10 - conj(sb) * x11, y11 = sb * x10 + Rb.x * x11;
+        put(I.w[0], Ra.x * y00 - sa * y10);                                                // X' = J_a^H Y
+        put(I.w[1], Ra.x * y01 - sa * y11);
+        put(I.w[2], conj(conj(sa) * y00 + Ra.x * y10));
+        put(I.w[3], conj(conj(sa) * y01 + Ra.x * y11));
+      };
+#pragma unroll
+      for (int x = 0; x < J32_OWN; ++x)
+        if (t + x * nt < nitem) block(own[x]);
+      for (int e = t + J32_OWN * nt; e < nitem; e += nt) block(make_block(e));
       __syncthreads();
+      cx<float> *x = A;
+      A = B;
+      B = x;
     }
   }
   // eigenvalues and their order (decreasing, ties by index)
   for (int i = t; i < k; i += nt) {
-    const float wi = A[i * ld + i].re;
+    const float wi = A[tri_at(i, i)].re;
     int rank = 0;
     for (int j = 0; j < k; ++j) {
-      const float wj = A[j * ld + j].re;
+      const float wj = A[tri_at(j, j)].re;
       rank += (wj > wi) || (wj == wi && j < i);
     }
     wout[rank] = (double)wi;
@@ -417,52 +443,71 @@ __global__ void __launch_bounds__(512) jacobi32_kernel(const zd *__restrict__ Ai
   }
 }
 
-// U = J_1 J_2 ... applied to the rows of the identity (a row sees every rotation, and no other row): one warp per row,
-// eight rows per CTA, the rotations of REPLAY rounds at a time through shared memory.  Writes U with its columns in
-// decreasing order of eigenvalue: all of them in FP32, the first nout also in FP64.
+// U = J_1 J_2 ... applied to the rows of the identity (a row sees every rotation, and no other row): one warp per row, eight
+// rows per CTA, the rotations of REPLAY rounds at a time through shared memory.  The row is in registers by position
+// as above: lane holds the pairs a = PPL lane + 0 .. PPL - 1, i.e. positions a and kp - 1 - a, and a round ends with the
+// move of every position by one.  Writes U with its columns in decreasing order of eigenvalue: all of them in FP32, the
+// first nout also in FP64.  (Row in shared memory: 0.28 us a round at k = 80.)
 constexpr int REPLAY = 16;
+template <int PPL>
 __global__ void __launch_bounds__(256) replay_kernel(int k, const float4 *__restrict__ rots, const int *__restrict__ meta,
                                                      const int *__restrict__ order, cx<float> *__restrict__ Uf,
                                                      zd *__restrict__ Uout, int ldu, int nout) {
   extern __shared__ __align__(16) unsigned char sm[];
   const int kp = k + (k & 1), np = kp / 2;
   float4 *R = reinterpret_cast<float4 *>(sm);                       // [REPLAY][np]
-  const int t = threadIdx.x, lane = t & 31, wp = t >> 5, row = blockIdx.x * 8 + wp;
-  cx<float> *u = reinterpret_cast<cx<float> *>(R + REPLAY * np) + wp * kp;
-  for (int i = lane; i < kp; i += 32) u[i] = mk<float>(i == row ? 1.f : 0.f, 0.f);
-  const int rounds = meta[0];
+  const int t = threadIdx.x, lane = t & 31, wp = t >> 5, row = blockIdx.x * 8 + wp, a0 = lane * PPL;
+  cx<float> x[PPL], y[PPL];
+#pragma unroll
+  for (int p = 0; p < PPL; ++p) {
+    x[p] = mk<float>(a0 + p == row ? 1.f : 0.f, 0.f);
+    y[p] = mk<float>(kp - 1 - a0 - p == row ? 1.f : 0.f, 0.f);
+  }
+  const int rounds = meta[META_ROUNDS];
   for (int r0 = 0; r0 < rounds; r0 += REPLAY) {
     const int nr = min(REPLAY, rounds - r0);
     __syncthreads();
     for (int e = t; e < nr * np; e += 256) R[e] = rots[(size_t)r0 * np + e];
     __syncthreads();
+#pragma unroll 2
     for (int rd = 0; rd < nr; ++rd) {
-      for (int pi = lane; pi < np; pi += 32) {
-        const float4 r = R[rd * np + pi];
-        const int p = __float_as_int(r.w) & 0xffff, q = __float_as_int(r.w) >> 16;
-        const cx<float> s = mk<float>(r.y, r.z), x = u[p], y = u[q];
-        u[p] = r.x * x - conj(s) * y;
-        u[q] = s * x + r.x * y;
+      cx<float> x1[PPL], y1[PPL];
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        const float4 r = R[rd * np + min(a0 + p, np - 1)];
+        const cx<float> s = mk<float>(r.y, r.z);
+        x1[p] = r.x * x[p] - conj(s) * y[p];
+        y1[p] = s * x[p] + r.x * y[p];
       }
-      __syncwarp();
+      const cx<float> dn = mk<float>(__shfl_down_sync(0xffffffffu, x1[0].re, 1), __shfl_down_sync(0xffffffffu, x1[0].im, 1));
+      const cx<float> up = mk<float>(__shfl_up_sync(0xffffffffu, y1[PPL - 1].re, 1), __shfl_up_sync(0xffffffffu, y1[PPL - 1].im, 1));
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        const cx<float> next = p + 1 < PPL ? x1[p + 1 < PPL ? p + 1 : 0] : dn, prev = p > 0 ? y1[p > 0 ? p - 1 : 0] : up;
+        x[p] = a0 + p == 0 ? x1[p] : (a0 + p == np - 1 ? y1[p] : next);
+        y[p] = a0 + p == 0 ? (np == 1 ? y1[p] : next) : prev;
+      }
     }
   }
   if (row < k)
-    for (int i = lane; i < k; i += 32) {
-      const int rk = order[i];
-      Uf[(size_t)rk * k + row] = u[i];
-      if (rk < nout) Uout[(size_t)rk * ldu + row] = cvt<double>(u[i]);
-    }
+#pragma unroll
+    for (int p = 0; p < PPL; ++p)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = h ? kp - 1 - a0 - p : a0 + p;
+        if (a0 + p >= np || i >= k) continue;
+        const cx<float> u = h ? y[p] : x[p];
+        const int rk = order[i];
+        Uf[(size_t)rk * k + row] = u;
+        if (rk < nout) Uout[(size_t)rk * ldu + row] = cvt<double>(u);
+      }
 }
 
 static size_t j32_smem(int k) {
   const int kp = k + (k & 1);
-  return (size_t)kp * (kp + 1) * sizeof(cx<float>) + (size_t)(kp / 2) * sizeof(float4);
+  return (size_t)kp * (kp + 1) * sizeof(cx<float>);
 }
-static size_t replay_smem(int k) {
-  const int kp = k + (k & 1);
-  return (size_t)REPLAY * (kp / 2) * sizeof(float4) + (size_t)8 * kp * sizeof(cx<float>);
-}
+static size_t replay_smem(int k) { return (size_t)REPLAY * ((k + 1) / 2) * sizeof(float4); }
 
 // Conversions by their bits (a conversion instruction runs at the FP64 rate): x truncated to FP32 (zero below
 // 2^-126; x is finite and below 2^128), and back (normal numbers and zero).
@@ -849,12 +894,15 @@ void sm_eig_topr(const zd *M, int ldm, int k, int r, zd *Y, int ldy, double *mu,
   float4 *rots = (float4 *)take(rots_bytes(k));
   const zd one = mk<double>(1, 0), zero = mk<double>(0, 0);
   // 1. FP32 eigendecomposition of the whole k x k matrix: all eigenvectors in FP32 (U32), the
-  //    top r also in FP64 (E1), eigenvalues in FP64 (w).  Threads: one item each while the CTA has them.
-  const int np = (k + 1) / 2, nt = std::min(512, std::max(64, (np * (np - 1) / 2 + 31) / 32 * 32));
+  //    top r also in FP64 (E1), eigenvalues in FP64 (w).  Threads: a block each while the CTA has them.
+  const int np = (k + 1) / 2, nt = std::min(512, std::max(64, (np * (np + 1) / 2 + 31) / 32 * 32));
   ::lrei::count_launch();
   jacobi32_kernel<<<1, nt, j32_smem(k), st>>>(M, ldm, k, w, order, rots, meta, 1e-5f);
   ::lrei::count_launch();
-  replay_kernel<<<(k + 7) / 8, 256, replay_smem(k), st>>>(k, rots, meta, order, U32, E1, k, r);
+  auto replay = [&](auto kern) { kern<<<(k + 7) / 8, 256, replay_smem(k), st>>>(k, rots, meta, order, U32, E1, k, r); };
+  if (np <= 32) replay(replay_kernel<1>);
+  else if (np <= 64) replay(replay_kernel<2>);
+  else replay(replay_kernel<3>);
   // 2.-3. block-Newton corrections of the top-r invariant subspace and polar re-orthonormalisations, each pass
   //       returning at once when the ones before it have converged
   const dim3 rows(r, (k + 31) / 32);
