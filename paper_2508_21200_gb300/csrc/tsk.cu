@@ -1,8 +1,7 @@
 // Tall-skinny (N-length) kernels of the LREI hot path.
 //
 //  * The per-row matrix-free H.V gather (hv_group; paper Sec. 3.3 "sparsity of H",
-//    Hamiltonian eq. H1), used inside the fused passes and as the fallback of the
-//    full-row H.V kernel of hv.cu for rows that are not a multiple of 16 bytes:
+//    Hamiltonian eq. H1), the fallback of the full-row H.V kernel of hv.cu for rows that are not a multiple of 16 bytes:
 //    a thread owns CPT consecutive columns of one row; partner rows are read
 //    through the read-only cache (rows of one N x r block are contiguous).
 //  * Fused tile passes (apply / extend / combine, see tsk.cuh) compute the
@@ -173,8 +172,7 @@ __host__ __device__ inline size_t ts_bytes(int nq, int gram_left, int r, int tr,
 }
 
 template <typename T, int CPT>
-__global__ void __launch_bounds__(TS_THREADS) ts_kernel(const __grid_constant__ ModelArgs M,
-                                                       const __grid_constant__ TSArgs a, int tr, int coef_smem,
+__global__ void __launch_bounds__(TS_THREADS) ts_kernel(const __grid_constant__ TSArgs a, int tr, int coef_smem,
                                                        const cx<T> *__restrict__ coefg) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int r = a.r, nq = a.nq, gl = a.gram_left;
@@ -208,11 +206,7 @@ __global__ void __launch_bounds__(TS_THREADS) ts_kernel(const __grid_constant__ 
         const int lr = e / gpr, c0 = (e % gpr) * CPT;
         cx<T> v[CPT];
         if (lr < rows) {
-          if (a.apply_h) {
-            hv_group<T, CPT>(M, src, r, (uint32_t)(row0 + lr), c0, v);
-          } else {
-            Group<T, CPT>::load(src + (size_t)(row0 + lr) * r + c0, v);
-          }
+          Group<T, CPT>::load(src + (size_t)(row0 + lr) * r + c0, v);
         } else {
 #pragma unroll
           for (int c = 0; c < CPT; ++c) v[c] = mk<T>(0, 0);
@@ -310,8 +304,7 @@ __host__ __device__ inline size_t ts2_bytes(int nq, int gl, int r, int tr, int m
 }
 
 template <typename T, int CPT, int MT>
-__global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__ ModelArgs M,
-                                                        const __grid_constant__ TSArgs a, int tr,
+__global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__ TSArgs a, int tr,
                                                         const cx<T> *__restrict__ coefg) {
   constexpr int MI = TS2<T>::MI, MJ = TS2<T>::MJ;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -380,8 +373,7 @@ __global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__
         const int lr = e / gpr, c0 = (e % gpr) * CPT;
         cx<T> v[CPT];
         if (lr < rows) {
-          if (a.apply_h) hv_group<T, CPT>(M, src, r, (uint32_t)(row0 + lr), c0, v);
-          else Group<T, CPT>::load(src + (size_t)(row0 + lr) * r + c0, v);
+          Group<T, CPT>::load(src + (size_t)(row0 + lr) * r + c0, v);
         } else {
 #pragma unroll
           for (int c = 0; c < CPT; ++c) v[c] = mk<T>(0, 0);
@@ -491,7 +483,8 @@ __global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__
 }
 
 // ------------------------------------------- fused tile pass, pipelined (complex64 bulk)
-// Same contract as ts_kernel for T = float, split H.V (apply_h == 0) and r in {8, 16, 32}.
+// Same contract as ts_kernel for T = float: R = 8, 16 or 32 is the next width from r up; with PAD
+// (r < R) the columns r .. R - 1 of the tiles are zero, and rows are copied by elements.
 // Each CTA walks its tiles of TR rows with the next tiles' blocks already in flight: cp.async copies the rows of every
 // input block into a ring of nst buffers (padded rows of RS complex) while the current tile is computed.
 // What bounds it is the FP32 pipe (at r = 16, 5 blocks: 150 us of multiply-adds against 99 us of bytes), next to it the
@@ -516,7 +509,7 @@ template <int R> struct TS3 {
 constexpr int TS3_STAGES = 6;
 
 // GMAX: Gram blocks this instance handles (gl + 1 <= GMAX; with EXACT gl + 1 == GMAX)
-template <int R, int TR, int GMAX, bool EXACT, int A, int MINB>
+template <int R, int TR, int GMAX, bool EXACT, int A, int MINB, bool PAD = false>
 __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ TSArgs a, const cx<float> *__restrict__ coefg,
                                                        int nst) {
   constexpr int RS = TS3<R>::RS, KW = TS3<R>::KW, KX = 128 / TR;   // KX: warps of one projection sum
@@ -542,11 +535,16 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
   const int c0 = mt / NJ * A, jg = mt % NJ;
   const long long N = a.N;
   const long long ntiles = (N + TR - 1) / TR;
-  const int ldg = g * R;
-  double2 *outp = reinterpret_cast<double2 *>(a.partial + (size_t)blockIdx.x * ldg * R * 2);
+  const int r = PAD ? a.r : R;
+  const int ldg = g * r;
+  double2 *outp = reinterpret_cast<double2 *>(a.partial + (size_t)blockIdx.x * ldg * r * 2);
 
   if (mode != 0)
     for (int e = tid; e < (nq + 1) * R * R; e += 256) cs[e] = coefg[e];
+  if (PAD) {
+    for (int e = tid; e < nst * nb * bstride; e += 256) buf[e] = mk<float>(0.f, 0.f);
+    __syncthreads();
+  }
 
   // A tile's rows are contiguous: chunk tid + 256 x of a block.  Rows beyond N (in the last tile only) become zero.
   const int lr_t = tid / CH;
@@ -556,14 +554,28 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
     const size_t off = (size_t)row0 * (R * sizeof(cx<float>)) + tid * 16;
     uint32_t sa = sm_t + sb * nb * (bstride * 8);
     const bool full = row0 + TR <= N;
+    if constexpr (PAD) {
+      const uint32_t inv = 65536 / r + 1;   // e / r = e inv >> 16 for e < 2048
+      sa = (uint32_t)__cvta_generic_to_shared(buf) + sb * nb * (bstride * 8);
+      for (int e = tid; e < TR * r; e += 256) {
+        const int lr = (int)(e * inv >> 16), c = e - lr * r;
+        const bool ok = row0 + lr < N;
+        for (int m = 0; m < nb; ++m) {
+          const char *base = reinterpret_cast<const char *>(m < nq ? a.q[m] : a.src);
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa + (m * bstride + lr * RS + c) * 8),
+                       "l"(ok ? base + ((size_t)row0 * r + e) * 8 : base), "r"(ok ? 8 : 0));
+        }
+      }
+    } else {
 #pragma unroll 1
-    for (int m = 0; m < nb; ++m, sa += bstride * 8) {
-      const char *gp = reinterpret_cast<const char *>(m < nq ? a.q[m] : a.src) + off;
+      for (int m = 0; m < nb; ++m, sa += bstride * 8) {
+        const char *gp = reinterpret_cast<const char *>(m < nq ? a.q[m] : a.src) + off;
 #pragma unroll
-      for (int x = 0; x < TR * CH / 256; ++x) {
-        const bool ok = full || row0 + lr_t + x * (256 / CH) < N;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa + x * (256 / CH) * RS * 8),
-                     "l"(ok ? gp + x * 4096 : gp - off), "r"(ok ? 16 : 0));
+        for (int x = 0; x < TR * CH / 256; ++x) {
+          const bool ok = full || row0 + lr_t + x * (256 / CH) < N;
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa + x * (256 / CH) * RS * 8),
+                       "l"(ok ? gp + x * 4096 : gp - off), "r"(ok ? 16 : 0));
+        }
       }
     }
   };
@@ -615,7 +627,8 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
 #pragma unroll
             for (int y = 0; y < LEFT; ++y) {
               const int yy = y0 + y, col = 2 * (jg + (yy >> 1) * NJ) + (yy & 1);
-              double2 *slot = outp + (size_t)col * ldg + m * R + c0 + x;
+              if (PAD && (col >= r || c0 + x >= r)) continue;
+              double2 *slot = outp + (size_t)col * ldg + m * r + c0 + x;
               float4 s = first ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<float4 *>(slot);
               two_sum_acc(s.x, s.y, f[y].x);
               two_sum_acc(s.z, s.w, f[y].y);
@@ -731,7 +744,15 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
         }
         if (!(lr < rows && row0 + lr >= a.zero_rows)) w = make_float4(0.f, 0.f, 0.f, 0.f);
         *nd = w;
-        if (out && lr < rows) *reinterpret_cast<float4 *>(out + (size_t)(row0 + lr) * R + ch * 2) = w;
+        if (out && lr < rows) {
+          cx<float> *o = out + (size_t)(row0 + lr) * r + ch * 2;
+          if (!PAD) {
+            *reinterpret_cast<float4 *>(o) = w;
+          } else {
+            if (ch * 2 < r) o[0] = mk<float>(w.x, w.y);
+            if (ch * 2 + 1 < r) o[1] = mk<float>(w.z, w.w);
+          }
+        }
       }
       __syncthreads();
       G = ns;
@@ -785,10 +806,9 @@ static size_t ts3_bytes(int r, int nq, int mode, int tr, int nst) {
   return b;
 }
 
-// Coefficients in the padded row-major layout of ts2_kernel: row m*rp + i, column j.
+// Coefficients in a padded row-major layout (rp columns): row m*rp + i, column j.
 template <typename T>
-__global__ void coef_convert2_kernel(const zd *coefQ, const zd *coefS, int nq, int r, int mode, cx<T> *out) {
-  const int rp = ts2_rp(r);
+__global__ void coef_convert2_kernel(const zd *coefQ, const zd *coefS, int nq, int r, int rp, int mode, cx<T> *out) {
   const int rows = (nq + 1) * rp;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * rp; e += gridDim.x * blockDim.x) {
     const int row = e / rp, j = e % rp, m = row / rp, i = row % rp;
@@ -845,7 +865,7 @@ int ts_max_grid(int nsm) { return 2 * nsm; }
 size_t ts_partial_doubles(int gram_left, int r) { return (size_t)(gram_left + 1) * r * r * 2; }
 
 template <typename T>
-static int launch_ts_v1(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_t st) {
+static int launch_ts_v1(const TSArgs &a, int nsm, cudaStream_t st) {
   const int r = a.r;
   // choose tile rows / coefficient placement so the CTA fits in shared memory
   const size_t budget = 200 * 1024;
@@ -873,7 +893,7 @@ static int launch_ts_v1(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream
   int cpt = 1;
   if (r % cpt_max == 0) cpt = cpt_max;
   else if (r % 2 == 0) cpt = 2;
-  auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(M, a, tr, coef_smem ? 1 : 0, coefg); };
+  auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(a, tr, coef_smem ? 1 : 0, coefg); };
   if (cpt == 4) go(ts_kernel<T, (sizeof(T) == 4 ? 4 : 2)>);
   else if (cpt == 2) go(ts_kernel<T, 2>);
   else go(ts_kernel<T, 1>);
@@ -886,15 +906,18 @@ static int launch_ts_v1(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream
 // micro-tile up to 4 Gram blocks at r = 16 (4: 206 against 256 us at n = 20) and 3 at r = 32 (3: 2.4 against 2.6 ms at
 // n = 22; 4: 3.3 against 3.15); 64-row tiles halve the barriers of 32-row ones (r = 16, one block: 79 -> 71 us) and are
 // taken where two stages of them fit.
+// Ranks that are no width are padded: Grams of 2 and 5 blocks at n = 18 took, by ts2_kernel and here, 84 and 44 us (5 blocks) at
+// r = 1, 74 / 102 and 38 / 54 at r = 5, 91 / 158 and 64 / 105 at r = 9, 82 / 169 and 67 / 111 at r = 12; from 17 on the width 32 costs more than
+// ts2_kernel (133 / 294 against 187 / 333 at r = 17, 166 against 195 for two blocks at r = 24) except for many blocks of
+// a rank near it (534 against 348 us for five at r = 24).
 struct TS3Plan {
-  int tr, two, nst;
+  int R, tr, two, nst;
   size_t bytes;
 };
 static TS3Plan ts3_plan(const TSArgs &a) {
-  TS3Plan p{0, 0, 0, 0};
-  if (a.apply_h) return p;
+  TS3Plan p{0, 0, 0, 0, 0};
   if (a.mode == 0 && a.out) return p;
-  const int r = a.r, nq = a.nq, gl = a.gram_left, mode = a.mode;
+  const int nq = a.nq, gl = a.gram_left, mode = a.mode;
   const int nb = nq + (mode != 2 ? 1 : 0);
   if (nb < 1 || nb > 8 || gl + 1 > 8 || gl > nq || (mode == 2 && nq < 1)) return p;
   auto al = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
@@ -902,8 +925,9 @@ static TS3Plan ts3_plan(const TSArgs &a) {
     if (!al(a.q[m])) return p;
   if (mode != 2 && !al(a.src)) return p;
   if (a.out && !al(a.out)) return p;
-  if (r != 8 && r != 16 && r != 32) return p;
-  const int two = r == 16 ? gl + 1 <= 4 : (r == 32 ? gl + 1 <= 3 : 0);
+  const int r = p.R = a.r <= 8 ? 8 : (a.r <= 16 ? 16 : 32);
+  if (r == 32 && a.r < 32 && (a.r < 24 || gl + 1 < 4)) return p;
+  const int two = r != a.r ? 0 : (r == 16 ? gl + 1 <= 4 : (r == 32 ? gl + 1 <= 3 : 0));
   for (int t = two; t >= 0; --t)
     for (int tr = 64; tr >= (r == 8 ? 64 : 32); tr /= 2) {
       const size_t lim = (t ? 113 : 227) * 1024;
@@ -919,7 +943,13 @@ static TS3Plan ts3_plan(const TSArgs &a) {
 }
 
 using TS3Kernel = void (*)(TSArgs, const cx<float> *, int);
-template <int R, int TR> static TS3Kernel ts3_instance(int g, bool two) {
+template <int R, int TR> static TS3Kernel ts3_padded(int g) {
+  if constexpr (R < 32)
+    if (g <= 3) return ts3_kernel<R, TR, 3, false, 1, 1, true>;
+  return g <= 5 ? ts3_kernel<R, TR, 5, false, 1, 1, true> : ts3_kernel<R, TR, 8, false, 1, 1, true>;
+}
+template <int R, int TR> static TS3Kernel ts3_instance(int g, bool two, bool pad) {
+  if (pad) return ts3_padded<R, TR>(g);
   if (g > 5) return ts3_kernel<R, TR, 8, false, 1, 1>;
   if (two) {
     if (g == 1) return ts3_kernel<R, TR, 1, true, 2, 2>;
@@ -932,9 +962,10 @@ template <int R, int TR> static TS3Kernel ts3_instance(int g, bool two) {
   if (g == 4) return ts3_kernel<R, TR, 4, true, 2, 1>;
   return ts3_kernel<R, TR, 5, true, 2, 1>;
 }
-static TS3Kernel ts3_pick(int r, int tr, int g, bool two) {
-  if (r == 16) return tr == 64 ? ts3_instance<16, 64>(g, two) : ts3_instance<16, 32>(g, two);
-  if (r == 32) return tr == 64 ? ts3_instance<32, 64>(g, two) : ts3_instance<32, 32>(g, two);
+static TS3Kernel ts3_pick(int R, int tr, int g, bool two, bool pad) {
+  if (R == 16) return tr == 64 ? ts3_instance<16, 64>(g, two, pad) : ts3_instance<16, 32>(g, two, pad);
+  if (R == 32) return tr == 64 ? ts3_instance<32, 64>(g, two, pad) : ts3_instance<32, 32>(g, two, pad);
+  if (pad) return ts3_padded<8, 64>(g);
   if (g <= 2) return ts3_kernel<8, 64, 2, false, 1, 1>;
   return g <= 5 ? ts3_kernel<8, 64, 5, false, 1, 1> : ts3_kernel<8, 64, 8, false, 1, 1>;
 }
@@ -945,7 +976,7 @@ static int launch_ts3(const TSArgs &a, int nsm, cudaStream_t st, const TS3Plan &
     if (!a.coef_scratch) return -1;
     coefg = reinterpret_cast<const cx<float> *>(a.coef_scratch);
     ::lrei::count_launch();
-    coef_convert2_kernel<float><<<8, 256, 0, st>>>(a.coefQ, a.coefS, a.nq, a.r, a.mode,
+    coef_convert2_kernel<float><<<8, 256, 0, st>>>(a.coefQ, a.coefS, a.nq, a.r, p.R, a.mode,
                                                   reinterpret_cast<cx<float> *>(a.coef_scratch));
   }
   // persistent, each CTA walking tiles blockIdx.x, + gridDim.x, ...: one or two CTAs per SM (ts3_plan)
@@ -954,12 +985,12 @@ static int launch_ts3(const TSArgs &a, int nsm, cudaStream_t st, const TS3Plan &
   int grid = (int)(ntiles < cap ? ntiles : cap);
   if (grid < 1) grid = 1;
   ::lrei::count_launch();
-  ts3_pick(a.r, p.tr, a.gram_left + 1, p.two)<<<grid, 256, p.bytes, st>>>(a, coefg, p.nst);
+  ts3_pick(p.R, p.tr, a.gram_left + 1, p.two, a.r != p.R)<<<grid, 256, p.bytes, st>>>(a, coefg, p.nst);
   return grid;
 }
 
 template <typename T>
-static int launch_ts_t(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_t st) {
+static int launch_ts_t(const TSArgs &a, int nsm, cudaStream_t st) {
   if (sizeof(T) == 4) {
     const TS3Plan p = ts3_plan(a);
     if (p.bytes) return launch_ts3(a, nsm, st, p);
@@ -972,14 +1003,14 @@ static int launch_ts_t(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_
   if (mt > 0)
     while (tr > 8 && ts2_bytes<T>(a.nq, a.gram_left, r, tr, a.mode, mt) > budget) tr /= 2;
   if (mt == 0 || ts2_bytes<T>(a.nq, a.gram_left, r, tr, a.mode, mt) > budget)
-    return launch_ts_v1<T>(M, a, nsm, st);
+    return launch_ts_v1<T>(a, nsm, st);
   const size_t bytes = ts2_bytes<T>(a.nq, a.gram_left, r, tr, a.mode, mt);
   cx<T> *coefg = nullptr;
   if (a.mode != 0) {
     if (!a.coef_scratch) return -1;
     coefg = reinterpret_cast<cx<T> *>(a.coef_scratch);
     ::lrei::count_launch();
-    coef_convert2_kernel<T><<<8, 256, 0, st>>>(a.coefQ, a.coefS, a.nq, r, a.mode, coefg);
+    coef_convert2_kernel<T><<<8, 256, 0, st>>>(a.coefQ, a.coefS, a.nq, r, rp, a.mode, coefg);
   }
   const long long ntiles = (a.N + tr - 1) / tr;
   int grid = (int)(ntiles < (long long)ts_max_grid(nsm) ? ntiles : ts_max_grid(nsm));
@@ -988,7 +1019,7 @@ static int launch_ts_t(const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_
   int cpt = 1;
   if (r % cpt_max == 0) cpt = cpt_max;
   else if (r % 2 == 0) cpt = 2;
-  auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(M, a, tr, coefg); };
+  auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(a, tr, coefg); };
   if (mt == 1) {
     if (cpt == cpt_max && cpt_max == 4) go(ts2_kernel<T, (sizeof(T) == 4 ? 4 : 2), 1>);
     else if (cpt == 2) go(ts2_kernel<T, 2, 1>);
@@ -1060,7 +1091,7 @@ __global__ void __launch_bounds__(128) few_gram_kernel(TSArgs a, const cx<T> *__
 // FP64 at n = 8, r = 4, 5 blocks: Gram 24 us as tiles and their sum, 4 here; projection and Gram 20, 8 here.
 template <typename T> static bool launch_few(const TSArgs &a, cudaStream_t st) {
   const int g = a.gram_left + 1;
-  if (!a.red || a.apply_h || a.N > 4096 || a.N * g * a.r * a.r > (1 << 20) || a.nq + 1 > MAXB + 1) return false;
+  if (!a.red || a.N > 4096 || a.N * g * a.r * a.r > (1 << 20) || a.nq + 1 > MAXB + 1) return false;
   if (a.mode == 0 ? a.out != nullptr : a.out == nullptr) return false;
   if (a.mode != 2 && !a.src) return false;
   if (a.mode != 0)
@@ -1081,12 +1112,21 @@ template <typename T> static bool launch_few(const TSArgs &a, cudaStream_t st) {
 
 int launch_ts(bool fp64, const ModelArgs &M, const TSArgs &a, int nsm, cudaStream_t st) {
   if (a.nq > MAXB || a.gram_left > a.nq || a.r < 1 || a.r > MAX_R) return -1;
+  if (a.apply_h) {   // H.V by its own kernel, then a pass that only reads
+    if (a.mode != 0 || !a.out || a.out == a.src) return -1;
+    launch_hv(fp64, M, a.src, a.out, a.N, a.r, nsm, st, a.status);
+    TSArgs b = a;
+    b.src = a.out;
+    b.out = nullptr;
+    b.apply_h = 0;
+    return launch_ts(fp64, M, b, nsm, st);
+  }
   if (fp64 ? launch_few<double>(a, st) : launch_few<float>(a, st)) return 0;
   if (fp64) {
     const int n = launch_tsx(a, nsm, st);
     if (n > 0) return n;
   }
-  return fp64 ? launch_ts_t<double>(M, a, nsm, st) : launch_ts_t<float>(M, a, nsm, st);
+  return fp64 ? launch_ts_t<double>(a, nsm, st) : launch_ts_t<float>(a, nsm, st);
 }
 
 void launch_reduce(const double *partial, int nparts, int len_doubles, double *out, cudaStream_t st) {
@@ -1278,13 +1318,9 @@ int ts_init() {
     if (x != cudaSuccess) e = x;
   };
   for (int g = 1; g <= 8; ++g)
-    for (int two = 0; two < 2; ++two) {
-      set3((const void *)ts3_pick(8, 64, g, two));
-      set3((const void *)ts3_pick(16, 64, g, two));
-      set3((const void *)ts3_pick(16, 32, g, two));
-      set3((const void *)ts3_pick(32, 64, g, two));
-      set3((const void *)ts3_pick(32, 32, g, two));
-    }
+    for (int v = 0; v < 4; ++v)
+      for (int R = 8; R <= 32; R *= 2)
+        for (int tr = R == 8 ? 64 : 32; tr <= 64; tr *= 2) set3((const void *)ts3_pick(R, tr, g, v & 1, v & 2));
   set((const void *)ts_kernel<double, 2>);
   set((const void *)ts_kernel<double, 1>);
   set((const void *)ts_kernel<float, 4>);

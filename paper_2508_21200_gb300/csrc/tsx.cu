@@ -727,7 +727,7 @@ int tsx_run(const TSArgs &a, bool proj, const XPlan &p, int nsm, cudaStream_t st
 // 10.96 ms there and 0.26 / 0.49 / 0.67 / 0.99 ms here (the five blocks' tensor work alone is 0.47 ms), the projection of
 // five blocks onto one 2.2 ms, an RK4 step 96.0 and 22.2 ms; at n = 8, r = 4 the Gram of four 22.8 and 19.5 us.
 int launch_tsx(const TSArgs &a, int nsm, cudaStream_t st) {
-  if (a.apply_h || (a.mode == 0 && a.out) || (a.mode != 0 && !a.out) || a.r > MAX_R || a.N < 256) return 0;
+  if ((a.mode == 0 && a.out) || (a.mode != 0 && !a.out) || a.r > MAX_R || a.N < 256) return 0;
   auto off = [](const void *x) { return (reinterpret_cast<uintptr_t>(x) & 15) != 0; };
   for (int m = 0; m < a.nq; ++m)
     if (off(a.q[m])) return 0;
