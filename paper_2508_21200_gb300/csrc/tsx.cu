@@ -459,7 +459,8 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
       bar_sync(BAR_FULL + (i & 1), all);
       const bool changed = G.flags[4 + 2 * (i & 3)] != 0;
       bool direct = G.flags[5 + 2 * (i & 3)] != 0 || G.flags[0] != 0;
-      if (!direct && (!sliced || changed)) {
+      if (changed) sliced = false;   // also when this tile is direct: the next one that is cut has the new exponents
+      if (!direct && !sliced) {
         slice_coefs(a, p, G, el);
         sliced = true;
         direct = G.flags[0] != 0;
