@@ -8,9 +8,9 @@
 // with one exponent e per column (55 bits below 2^e, so an entry of the column's top binade is exact), the
 // digits held exactly in FP16.  The product of two digit planes is an integer sum, exact in the tensor core's
 // FP32 accumulator while it stays below 2^24.  Of the 49 digit products the 28 with s + t <= 6 are formed (the
-// others are below 2^-55 of the largest); those of equal s + t share an accumulator (a "class").  Every 128 rows
-// (2 x 128 x 4 x 2^14 = 2^24 for the first four classes; a class beyond the fourth carries less than 2^-32 of the
-// result) the classes go into two 64-bit integers per entry, without rounding.
+// others are below 2^-55 of the largest); those of equal s + t share an accumulator (a "class").  Every 128 complex summands
+// (the rows of a Gram, the columns of a projection: 2 x 128 x 4 x 2^14 = 2^24 for the first four classes; a class beyond
+// the fourth carries less than 2^-32 of the result) the classes go into two 64-bit integers per entry, without rounding.
 // A column keeps its exponent from tile to tile while the tile's largest entry stays within a few bits below it;
 // when it does not, the sums so far are flushed to the CTA's FP64 partial at the old exponents and the column
 // gets a new one, so no tile loses bits to a larger one.  A tile with infinities, NaN or entries near the ends of
@@ -54,7 +54,7 @@ namespace {
 constexpr int NS = 7;                 // digits
 constexpr int CUT_UNITS = 4;          // units a cutting warp holds in registers
 constexpr int X_THREADS = 512;        // most threads of a CTA (128 registers)
-constexpr int X_DRAIN = 128;          // rows between drains
+constexpr int X_DRAIN = 128;          // complex summands between drains
 constexpr int X_SLACK = 2;            // bits a column's tile may stay below its exponent
 constexpr int X_EMIN = 530, X_EMAX = 1510;   // exponent fields that are cut; others take the direct path
 constexpr int E_UNSET = -100000;
@@ -140,9 +140,9 @@ __device__ __forceinline__ void digit_planes(unsigned long long a, unsigned long
 
 // The classes as integers (first three, last four): x = h 2^-16 + l 2^-48.
 __device__ __forceinline__ void class_ints(const float (&a)[NS], long long &h, long long &l) {
-  h = ((long long)__float2int_rn(a[0]) << 16) + (long long)(__float2int_rn(a[1]) * 256) + __float2int_rn(a[2]);
+  h = ((long long)__float2int_rn(a[0]) << 16) + ((long long)__float2int_rn(a[1]) << 8) + __float2int_rn(a[2]);
   l = ((long long)__float2int_rn(a[3]) << 24) + ((long long)__float2int_rn(a[4]) << 16) +
-      (long long)(__float2int_rn(a[5])) * 256 + __float2int_rn(a[6]);
+      ((long long)__float2int_rn(a[5]) << 8) + __float2int_rn(a[6]);
 }
 // (h 2^-16 + l 2^-48) 2^k, rounded once, by integer operations (an FP64 conversion or multiply takes a scheduler
 // 64 cycles; this is about 30 integer instructions).
@@ -476,6 +476,22 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
           for (int w = 0; w < NS; ++w)
 #pragma unroll
             for (int k = 0; k < 4; ++k) pa[w][k] = 0.f;
+          long long hh[4] = {0, 0, 0, 0}, ll[4] = {0, 0, 0, 0};
+          auto drain = [&]() {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              float c[NS];
+#pragma unroll
+              for (int w2 = 0; w2 < NS; ++w2) {
+                c[w2] = pa[w2][k];
+                pa[w2][k] = 0.f;
+              }
+              long long x, y;
+              class_ints(c, x, y);
+              hh[k] += x;
+              ll[k] += y;
+            }
+          };
           const uint32_t *w = G.coef + (size_t)n * NS * 64 + lane;
           uint32_t ad = dig_a + (uint32_t)((i & 1) * dig_words) * 4u + (uint32_t)(kc * ncg * NS) * 512u + lane * 16u;
 #pragma unroll 2
@@ -494,7 +510,9 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
 #pragma unroll
               for (int u = 0; u + s < NS; ++u) mma16816(pa[s + u], av, b0[u], b1[u]);
             }
+            if ((cg + 1) % (X_DRAIN / 8) == 0) drain();
           }
+          drain();
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             // fragment row k of a chunk is row (k & 8) + 4 (k & 1) + (k & 7) / 2
@@ -503,14 +521,7 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
             const long long row = row0 + lr;
             const int f = G.fcol[j] - 7;
             double v = 0.0;
-            if (f != E_UNSET - 7 && row >= a.zero_rows) {
-              float c[NS];
-#pragma unroll
-              for (int w2 = 0; w2 < NS; ++w2) c[w2] = pa[w2][k];
-              long long hh, ll;
-              class_ints(c, hh, ll);
-              v = ints_value(hh, ll, f);
-            }
+            if (f != E_UNSET - 7 && row >= a.zero_rows) v = ints_value(hh[k], ll[k], f);
             G.nv[lr * p.ldnv + 2 * j + h] = v;
           }
         }

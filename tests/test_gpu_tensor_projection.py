@@ -158,3 +158,34 @@ def test_non_finite(project, bad):
     assert not torch.isfinite(torch.view_as_real(out[:, 4])).any()
     cols = torch.arange(r, device="cuda") != 4
     assert float((out - ref)[:, cols].abs().max()) < 2 * r * 2.0 ** -47 * float(C.abs().max())
+
+
+def _digits(shape, rng):
+    """Integers sum_s d_s 2^(8 (6 - s)), 119 <= d_s <= 127 (the last a multiple of 4, so that 53 bits hold them): every digit
+    near the largest."""
+    d = rng.integers(119, 128, (7, *shape))
+    d[6] = 124
+    return sum(d[s].astype(object) << (8 * (6 - s)) for s in range(7))
+
+
+@pytest.mark.parametrize("r,nq", [(16, 3), (32, 4), (17, 6)])
+def test_sums_of_the_largest_digits(project, r, nq):
+    # All products of one sign and near 2^14, K = 64, 160 and 119 complex columns of them.  Exact: the inputs and the first four
+    # classes of digit products.  The fifth passes 2^24 in the last fifth of 128 columns: at most 16 instructions that may cut
+    # 2 units of 2^-46 each, 5e-13 of products near one; the sum has at least 100 of these, so 4e-15 of it leaves room for the
+    # digit products left out (2^-52) and the rounding of the result.
+    N, K = 8192, (nq + 1) * r
+    rng = np.random.default_rng(r)
+    rows = rng.integers(0, 64, N)                         # 64 different rows
+    xr, xi, cr, ci = (_digits(s, rng) for s in ((64, K), (64, K), (K, r), (K, r)))
+    x = (xr.astype(np.float64) + 1j * xi.astype(np.float64))[rows]
+    x[: N // 2] /= 2                                      # the exponents stay one above these rows' and are those of the others
+    c = cr.astype(np.float64) - 1j * ci.astype(np.float64)
+    X, C = torch.from_numpy(x).cuda(), torch.from_numpy(c).cuda()
+    blocks = [X[:, i * r:(i + 1) * r].contiguous() for i in range(nq + 1)]
+    out = project(blocks[:nq], blocks[nq], C).cpu().numpy()[N // 2:]
+    re = xr.dot(cr) + xi.dot(ci)                          # exact integers
+    got = out.real
+    err = max(abs(int(got[k, j]) - re[rows[N // 2 + k], j]) / re[rows[N // 2 + k], j] for k in range(0, N // 2, 7)
+              for j in range(r))
+    assert err < 4e-15
