@@ -498,8 +498,13 @@ __global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__
 // Every 16-byte load of a quarter-warp and 8-byte load of a half-warp falls in distinct banks: a thread's columns are
 // 16-byte chunks (2 columns) R / 8 (Gram) or R / 4 (projection) chunks apart, lanes of one sum whose
 // coefficients would share banks read their two chunks in swapped order, and RS is chosen so.
-// At a flush (128 rows per lane in plain FP32 at r = 16) the lanes of a micro-tile are combined by halving
-// shuffles, and each sum is added to its compensated FP32 pair (TwoSum), kept in the CTA's partial (L2).
+// At a flush the lanes of a micro-tile are combined by halving shuffles and each sum is added to its compensated
+// FP32 pair, kept in the CTA's partial (L2), all by TwoSum: only the rows that one lane takes between two flushes are summed
+// plainly (LROWS: 16 to 256), since the error of a Gram grows with their number (a diagonal entry at n = 18: 8e-10 of it at 16
+// rows, 5e-9 at 128).  Padded ranks take as many as keep their error at that of ts2_kernel, whose 8 to 32 rows over 16 lanes
+// (r < 16) or 64 to 128 rows (r > 16) are combined plainly, and eight blocks of width 32 likewise.  Measured at n = 18, with sums four
+// to eight times as long and now: two blocks 38 -> 42 us at r = 5 (diagonal off by 2.8e-9 -> 6e-10), 65 -> 80 at r = 9 (4.3e-9 ->
+// 7e-10), five at r = 24 348 -> 371 us (1.2e-8 -> 5e-9), eight at r = 32 520 -> 756 us (1.1e-8 -> 1.3e-9).
 // Before (4 columns, one G column group conflicting at r = 32, double buffer): n = 20, r = 16, 5 blocks 337 us, now 262;
 // projection and Gram of 5 blocks 463 (4 inputs) -> 402 us; n = 22, r = 32, 5 blocks 7.7 -> 3.6 ms and 17.2 -> 7.0 ms.
 template <int R> struct TS3 {
@@ -518,7 +523,9 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
   constexpr int NPH = 256 / MTS;
   constexpr int TPW = 32 / NPH;
   constexpr int CH = R / 2;                 // 16-byte chunks per row
-  constexpr int FLUSHT = (R == 32 ? 256 : (R == 16 ? 128 : 32)) * NPH / TR;   // tiles between flushes
+  // rows a lane sums in plain FP32, and the tiles between flushes
+  constexpr int LROWS = R == 32 ? (GMAX > 5 ? 32 : (PAD ? 128 : 256)) : (R == 16 ? (PAD ? (GMAX > 3 ? 24 : 16) : 128) : (PAD ? 16 : 32));
+  constexpr int FLUSHT = LROWS * NPH / TR;
   constexpr int CNT = R / (KW * KX);
   static_assert(NPH >= 2 && NPH <= 32 && (RS * 8) % 16 == 0 && FLUSHT >= 1 && TR / 16 * KX == 8, "r in {8, 16, 32}");
   extern __shared__ __align__(16) unsigned char smem3[];
@@ -589,8 +596,17 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
       for (int y = 0; y < 8; ++y) acc[m][x][y] = mk<float>(0.f, 0.f);
 
   // The lanes of a micro-tile (bits TPW .. 16 of the lane) halve their columns three times, further ones are summed
-  // whole; then the pairs in the partial: (sum, error) of re and im, or with last their final values.
+  // whole; then the pairs in the partial: (sum, error) of re and im, or with last their final values.  All of it with the
+  // rounding errors kept (TwoSum): sums of LROWS rows are the only plain ones.
   bool first = true;
+  auto add_from = [&](float2 &f, float2 &e, float2 send, float2 sende, int o, bool errs) {   // (f, e) += the other lane's pair
+    two_sum_acc(f.x, e.x, __shfl_xor_sync(0xffffffffu, send.x, o));
+    two_sum_acc(f.y, e.y, __shfl_xor_sync(0xffffffffu, send.y, o));
+    if (errs) {
+      e.x += __shfl_xor_sync(0xffffffffu, sende.x, o);
+      e.y += __shfl_xor_sync(0xffffffffu, sende.y, o);
+    }
+  };
   auto flush = [&](bool last) {
     constexpr int LV = NPH == 2 ? 1 : (NPH == 4 ? 2 : 3), LEFT = 8 >> LV;
     int y0 = 0;
@@ -601,10 +617,11 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
       if (EXACT || m < g) {
 #pragma unroll
         for (int x = 0; x < A; ++x) {
-          float2 f[8];
+          float2 f[8], er[8];
 #pragma unroll
           for (int y = 0; y < 8; ++y) {
             f[y] = make_float2(acc[m][x][y].re, acc[m][x][y].im);
+            er[y] = make_float2(0.f, 0.f);
             acc[m][x][y] = mk<float>(0.f, 0.f);
           }
 #pragma unroll
@@ -613,16 +630,16 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
             const bool up = lane & o;
 #pragma unroll
             for (int y = 0; y < h; ++y) {
-              const float2 send = up ? f[y] : f[y + h], keep = up ? f[y + h] : f[y];
-              f[y].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, o);
-              f[y].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, o);
+              const float2 send = up ? f[y] : f[y + h], sende = up ? er[y] : er[y + h];
+              if (up) {
+                f[y] = f[y + h];
+                er[y] = er[y + h];
+              }
+              add_from(f[y], er[y], send, sende, o, v > 0);
             }
           }
 #pragma unroll
-          for (int o = 16 >> LV; o >= TPW; o >>= 1) {
-            f[0].x += __shfl_xor_sync(0xffffffffu, f[0].x, o);
-            f[0].y += __shfl_xor_sync(0xffffffffu, f[0].y, o);
-          }
+          for (int o = 16 >> LV; o >= TPW; o >>= 1) add_from(f[0], er[0], f[0], er[0], o, true);
           if ((lane & ((32 >> LV) - 1)) < TPW) {
 #pragma unroll
             for (int y = 0; y < LEFT; ++y) {
@@ -632,6 +649,8 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
               float4 s = first ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<float4 *>(slot);
               two_sum_acc(s.x, s.y, f[y].x);
               two_sum_acc(s.z, s.w, f[y].y);
+              s.y += er[y].x;
+              s.w += er[y].y;
               if (last) *slot = make_double2((double)s.x + (double)s.y, (double)s.z + (double)s.w);
               else *reinterpret_cast<float4 *>(slot) = s;
             }
@@ -649,6 +668,9 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
     asm volatile("cp.async.commit_group;\n" ::);
   }
   int since = 0;
+  // padded ranks with two tiles per CTA (ts2_kernel has twice the CTAs): after each; above 28 its tiles are shorter beside
+  // the coefficients
+  const int every = PAD && ntiles <= 2 * (long long)gridDim.x ? 1 : (PAD && R == 32 && GMAX <= 5 && mode != 0 && r > 28 ? FLUSHT / 2 : FLUSHT);
   for (; tile < ntiles; tile += gridDim.x) {
     switch (nst) {   // all but the newest nst - 2 groups: this tile is there
       case 2: asm volatile("cp.async.wait_group 0;\n" ::); break;
@@ -787,7 +809,7 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
         }
       }
     }
-    if (++since >= FLUSHT) {
+    if (++since >= every) {
       since = 0;
       flush(false);
     }
@@ -906,10 +928,10 @@ static int launch_ts_v1(const TSArgs &a, int nsm, cudaStream_t st) {
 // micro-tile up to 4 Gram blocks at r = 16 (4: 206 against 256 us at n = 20) and 3 at r = 32 (3: 2.4 against 2.6 ms at
 // n = 22; 4: 3.3 against 3.15); 64-row tiles halve the barriers of 32-row ones (r = 16, one block: 79 -> 71 us) and are
 // taken where two stages of them fit.
-// Ranks that are no width are padded: Grams of 2 and 5 blocks at n = 18 took, by ts2_kernel and here, 84 and 44 us (5 blocks) at
-// r = 1, 74 / 102 and 38 / 54 at r = 5, 91 / 158 and 64 / 105 at r = 9, 82 / 169 and 67 / 111 at r = 12; from 17 on the width 32 costs more than
-// ts2_kernel (133 / 294 against 187 / 333 at r = 17, 166 against 195 for two blocks at r = 24) except for many blocks of
-// a rank near it (534 against 348 us for five at r = 24).
+// Ranks that are no width are padded: Grams of 2 and 5 blocks at n = 18 took, by ts2_kernel and here, 89 and 51 us (5 blocks) at
+// r = 1, 76 / 106 and 42 / 62 at r = 5, 91 / 172 and 80 / 130 at r = 9, 84 / 174 and 78 / 135 at r = 12; from 17 on the width 32 costs
+// more than ts2_kernel (133 / 294 against 187 / 333 and more at r = 17, 166 against 195 for two blocks at r = 24) except for many
+// blocks of a rank near it (r = 24: 317 against 320 us for four, 534 against 371 for five; r = 25: 612 against 327 for four).
 struct TS3Plan {
   int R, tr, two, nst;
   size_t bytes;
