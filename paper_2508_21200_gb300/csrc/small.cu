@@ -560,26 +560,31 @@ __global__ void __launch_bounds__(512) jacobi64_kernel(const zd *__restrict__ Ai
     A[2 * ((e / kp) * ld + e % kp) + 1] *= scale;
   }
   __syncthreads();
-  // off-diagonal Frobenius norm <= k max |re|, |im| (off-diagonal) * sqrt(2); total >= max |diagonal|
-  const float thr = (float)tol / (1.5f * (float)k);
+  // Stop when the off-diagonal Frobenius norm is below tol times the whole one, both in FP32: entries are below 2 and the largest is
+  // at least 1, so squares that FP32 flushes (below 1e-38) are far below tol^2 = 1e-30.  A bound on the largest entry that
+  // implies this lies below the entries' own rounding at k = 32 (7 sweeps a call at r = 16 for equal weights, 20 at 32; none so).
+  const float tol2 = (float)(tol * tol);
   const int nA = (np * (np + 1) / 2 * 8 + 31) & ~31, nU = (np * kp * 4 + 31) & ~31;
   int sweep = 0;
   for (; finite && sweep < max_sweeps; ++sweep) {
-    unsigned off = 0, dia = 0;
+    float off = 0.f, dia = 0.f;
     for (int e = t; e < kp * kp; e += nt) {
       const int i = e % kp, j = e / kp;
       if (i > j) continue;
-      const unsigned m = max(__float_as_uint(fabsf(f32_bits(A[2 * (j * ld + i)]))),
-                             __float_as_uint(fabsf(f32_bits(A[2 * (j * ld + i) + 1]))));
-      if (i == j) dia = max(dia, m);
-      else off = max(off, m);
+      const float re = f32_bits(A[2 * (j * ld + i)]), im = f32_bits(A[2 * (j * ld + i) + 1]), v = fmaf(re, re, im * im);
+      if (i == j) dia += v;
+      else off += 2.f * v;
     }
-    off = __reduce_max_sync(0xffffffffu, off);
-    dia = __reduce_max_sync(0xffffffffu, dia);
-    if (lane == 0) { red[0][wp] = off; red[1][wp] = dia; }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      dia += __shfl_xor_sync(0xffffffffu, dia, o);
+    }
+    if (lane == 0) { red[0][wp] = __float_as_uint(off); red[1][wp] = __float_as_uint(dia); }
     __syncthreads();
-    for (int w = 0; w < nw; ++w) { off = max(off, red[0][w]); dia = max(dia, red[1][w]); }
-    if (__uint_as_float(off) <= thr * __uint_as_float(dia)) break;
+    off = dia = 0.f;
+    for (int w = 0; w < nw; ++w) { off += __uint_as_float(red[0][w]); dia += __uint_as_float(red[1][w]); }
+    if (off <= tol2 * (off + dia)) break;
     for (int round = 0; round < kp - 1; ++round) {
       if (t < np) {
         int p, q;
