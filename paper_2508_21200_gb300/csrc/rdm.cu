@@ -114,7 +114,6 @@ namespace {
 // chain, a division or square root 7 to 11 of these, so the angle is taken in FP32 (which annihilates to 1e-7 a
 // round) and made unitary in FP64 by two Newton steps for c = sqrt(1 - |s|^2).  A is scaled by a power of two to entries
 // below 2, so that FP32 has the range.  (One thread per matrix with FP64 angles: 5.0 ms for the 120 pairs of n = 16.)
-__device__ __forceinline__ float to_f32(double x) { return (float)x; }
 __device__ __forceinline__ double flip(double x, bool c) { return c ? -x : x; }
 __device__ void herm4_eig(const zd *A, zd *U, double *w) {
   const unsigned all = 0xffffffffu;
@@ -126,19 +125,25 @@ __device__ void herm4_eig(const zd *A, zd *U, double *w) {
   const int es = emax == 0 || !finite ? 1023 : max(1, 2046 - (int)emax);
   a *= __hiloint2double(es << 20, 0);
   for (int sweep = 0; finite && sweep < 30; ++sweep) {
-    const unsigned v = __float_as_uint(fabsf(to_f32(a)));
-    const float off = __uint_as_float(__reduce_max_sync(all, i != j ? v : 0u));
-    const float dia = __uint_as_float(__reduce_max_sync(all, i == j ? v : 0u));
-    if (off <= 2e-17f * dia) break;   // off-diagonal norm <= sqrt(24) max |re|, |im| <= 1e-16 of the total
+    // off-diagonal Frobenius norm against 1e-16 of the whole (a bound on the largest entry that implies it is below the
+    // entries' rounding: 4096 multiples of the identity took 2.7 ms a call, and 1.2 when they were exact)
+    const float v = (float)a * (float)a;
+    float off = i != j ? v : 0.f, tot = v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(all, off, o);
+      tot += __shfl_xor_sync(all, tot, o);
+    }
+    if (off <= 1e-32f * tot) break;
 #pragma unroll
     for (int mask = 1; mask < 4; ++mask) {
       const int p = min(j, j ^ mask), q = max(j, j ^ mask);
       const double app = __shfl_sync(all, a, 8 * p + 2 * p), aqq = __shfl_sync(all, a, 8 * q + 2 * q);
-      const float br = to_f32(__shfl_sync(all, a, 8 * p + 2 * q)), bi = to_f32(__shfl_sync(all, a, 8 * p + 2 * q + 1));
+      const float br = (float)(__shfl_sync(all, a, 8 * p + 2 * q)), bi = (float)(__shfl_sync(all, a, 8 * p + 2 * q + 1));
       const float n2 = fmaf(br, br, bi * bi);
       double c = 1.0, sr = 0.0, si = 0.0;   // [[c, s], [-conj(s), c]] on (p, q)
       if (n2 > 1e-37f) {
-        const float h = 0.5f * to_f32(aqq - app), g = fmaf(h, h, n2);
+        const float h = 0.5f * (float)(aqq - app), g = fmaf(h, h, n2);
         const float f = copysignf(__fdividef(1.f, fabsf(h) + g * rsqrtf(g)), h), vv = fmaf(n2 * f, f, 1.f), cf = rsqrtf(vv);
         sr = (double)(cf * f * br);
         si = (double)(cf * f * bi);
