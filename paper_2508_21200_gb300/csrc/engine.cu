@@ -264,8 +264,10 @@ __global__ void lhl_kernel(const zd *__restrict__ L, int r, const double *__rest
 // Observables from the Gram blocks of the observable pass (one CTA, r <= 32).
 // The stored factor V is orthonormalised implicitly: with V^*V = L L^H and X = L^{-1},
 // Tr(rho A) = Tr(Lambda X (V^*AV) X^H) = Tr(W V^*AV), W = X^H Lambda X: the products by X are done once (W, and
-// W2 = X^H Lambda^2 X for Tr(rho^2 H^2)), each observable is a sum over r^2 entries, and Tr(rho H rho H) the one of P P,
-// P = W V^*HV.  FP64 instructions bound it (an SM issues one per 19 cycles): an entry's sum is split over four lanes.
+// W2 = X^H Lambda^2 X for Tr(rho^2 H^2)) and each observable is a sum over r^2 entries.  Tr(rho H rho H) takes
+// Gbar = X V^*HV X^H itself, sum lambda_i lambda_j |Gbar_ij|^2: as the trace of P P, P = W V^*HV (similar to Lambda Gbar by X^H), it
+// would lose another condition number of V (of which the allocation-free call takes any).  FP64 instructions bound it (an SM issues
+// one per 19 cycles): an entry's sum is split over four lanes.
 // (With X A X^H formed per observable and square roots in the factor's chain: 179 us at r = 8, 2310 us at r = 32.)
 // With Werner weight p (Sec. 5, eq. werner-sol) the state is rho = p I/N + (1 - p) rho_hat, rho_hat the
 // stored low-rank state: H and the magnetisations are traceless, so their expectations and [rho, H] scale
@@ -315,33 +317,38 @@ __global__ void __launch_bounds__(512) obs_final_kernel(const double *__restrict
     }
   }
   __syncthreads();
-  for (int base = 0; base < rr; base += nt / 4) {      // P = W V^*HV
+  for (int base = 0; base < rr; base += nt / 4) {      // P = X V^*HV: sums over m <= i
     const int e = base + (t >> 2), i = e % r, j = e / r;
     zd v = mk<double>(0, 0);
     if (e < rr)
-      for (int m = q4; m < r; m += 4) fma_(v, W[m * r + i], B[j * r + m]);
+      for (int m = q4; m <= i; m += 4) fma_(v, X[m * r + i], B[j * r + m]);
     v = quad_sum(v);
     if (e < rr && q4 == 0) P[e] = v;
   }
   __syncthreads();
-  // sums: 0 Tr P, 1 Tr(W2 A1), 2..4 Tr(W A3..5), 5 Tr(P P), 6 trace, 7 purity; maxima (squares): V^*V - I, V^*HV - its
-  // conjugate transpose, V^*HV
+  // sums: 0 Tr(W A0), 1 Tr(W2 A1), 2..4 Tr(W A3..5), 5 sum lambda_i lambda_j |Gbar_ij|^2, 6 trace, 7 purity; maxima
+  // (squares): V^*V - I, V^*HV - its conjugate transpose, V^*HV
   double acc[NSUM] = {0, 0, 0, 0, 0, 0, 0, 0};
   double mx[NMAX] = {0, 0, 0};
+  for (int base = 0; base < rr; base += nt / 4) {      // Gbar = P X^H: sums over m <= j
+    const int e = base + (t >> 2), i = e % r, j = e / r;
+    zd g = mk<double>(0, 0);
+    if (e < rr)
+      for (int m = q4; m <= j; m += 4) fma_(g, P[m * r + i], conj(X[m * r + j]));
+    g = quad_sum(g);
+    if (e < rr && q4 == 0) acc[5] = fma(lams[i] * lams[j], norm2(g), acc[5]);
+  }
   auto dot = [](double &a, zd x, zd y) { a = fma(x.re, y.re, fma(-x.im, y.im, a)); };   // a += Re(x y)
   for (int e = t; e < rr; e += nt) {
     const int i = e % r, j = e / r, et = i * r + j;
     const zd w = W[et], g = Gam[e], h = B[e], ht = B[et];
+    dot(acc[0], w, h);
     dot(acc[1], W2[et], B[rr + e]);
     dot(acc[2], w, B[3 * rr + e]);
     dot(acc[3], w, B[4 * rr + e]);
     dot(acc[4], w, B[5 * rr + e]);
-    dot(acc[5], P[e], P[et]);
     acc[7] = fma(lams[i] * lams[j], norm2(g), acc[7]);
-    if (i == j) {
-      acc[0] += P[e].re;
-      acc[6] = fma(lams[i], g.re, acc[6]);
-    }
+    if (i == j) acc[6] = fma(lams[i], g.re, acc[6]);
     mx[0] = fmax(mx[0], norm2(i == j ? mk<double>(g.re - 1.0, g.im) : g));
     mx[1] = fmax(mx[1], norm2(h - conj(ht)));
     mx[2] = fmax(mx[2], norm2(h));
