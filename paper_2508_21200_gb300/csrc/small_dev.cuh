@@ -83,21 +83,30 @@ __device__ __forceinline__ void eliminate(zd *Ls, zd *X, int k, const double *to
 inline int eliminate_threads(int k) { return k * (k + 1) >= 512 ? 512 : (k * (k + 1) + 31) / 32 * 32; }
 
 // X = L^{-1} for A = L L^H (k x k, leading dimension lda, positive definite: a pivot counts as at least 1e-300, k <= MAX_R), by
-// the whole CTA.  Ls: work, k x k.
+// the whole CTA.  Ls: work, k x k.  The columns are scaled by powers of two to a diagonal in [1, 4): the products of two
+// entries that the elimination forms stay in range for every A that does (exactly the same X).
 __device__ __forceinline__ void chol_inv_cta(const zd *A, int lda, int k, zd *Ls, zd *X) {
-  __shared__ double inv[MAX_R], tolref[MAX_R];
+  __shared__ double inv[MAX_R], tolref[MAX_R], scale[MAX_R];
   __shared__ int dead[MAX_R];
   __syncthreads();
+  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+    const int e = ((__double2hiint(A[(size_t)i * lda + i].re) >> 20) & 0x7ff) - 1023;      // a negative, zero or non-finite entry as it is
+    const bool ok = A[(size_t)i * lda + i].re > 0.0 && e < 1024;
+    scale[i] = __hiloint2double((1023 - (ok ? e >> 1 : 0)) << 20, 0);
+    tolref[i] = 1e-300 * scale[i] * scale[i];
+  }
+  __syncthreads();
   for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-    Ls[e] = A[(size_t)(e / k) * lda + e % k];
+    const zd a = A[(size_t)(e / k) * lda + e % k];
+    const double si = scale[e % k], sj = scale[e / k];
+    Ls[e] = mk<double>(a.re * si * sj, a.im * si * sj);
     X[e] = mk<double>(e % k == e / k ? 1.0 : 0.0, 0);
   }
-  for (int i = threadIdx.x; i < k; i += blockDim.x) tolref[i] = 1e-300;
   __syncthreads();
   eliminate(Ls, X, k, tolref, inv, dead);
-  for (int i = threadIdx.x; i < k; i += blockDim.x) inv[i] = dead[i] ? 1e150 : newton_rsqrt(Ls[i * k + i].re);
+  for (int i = threadIdx.x; i < k; i += blockDim.x) inv[i] = dead[i] ? 1e150 / scale[i] : newton_rsqrt(Ls[i * k + i].re);
   __syncthreads();
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) X[e] = inv[e % k] * X[e];
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) X[e] = inv[e % k] * (scale[e / k] * X[e]);
   __syncthreads();
 }
 

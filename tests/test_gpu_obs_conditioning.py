@@ -45,7 +45,7 @@ def _unitary(r, rng):
     return np.linalg.qr(rng.standard_normal((r, r)) + 1j * rng.standard_normal((r, r)))[0]
 
 
-@pytest.mark.parametrize("scale", [1.0])
+@pytest.mark.parametrize("scale", [1.0, 1e-100, 1e100])
 @pytest.mark.parametrize("condition", [1e2, 1e4, 1e5])
 def test_commutator(condition, scale):
     r = 8
