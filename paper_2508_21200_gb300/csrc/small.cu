@@ -205,6 +205,8 @@ void sm_trsv(char op, const zd *L, int ldl, int k, zd *B, int ldb, int ncols, cu
 // Cholesky A = L L^H of a Hermitian k x k matrix (k <= 64) and the inverse of L, in one CTA: Gaussian elimination on
 // [A | I] (eliminate), and the columns are scaled by A_jj^{-1/2} at the end.  The inverse rides along in the chain of the
 // steps (a triangular solve of its own took 24 us at k = 16).
+// The elimination multiplies two entries before it divides by the pivot, so when a diagonal entry is beyond 2^+-400 the columns are
+// scaled by powers of two to a diagonal in [1, 4) first (an unusual unit of energy: the Gram of H V has its square).
 // Column j is dead when its pivot is not above tol times a reference: the j-th diagonal entry of `ref` when given (the
 // squared norm of the raw column), else the largest diagonal entry of A.  A dead column gets L[j][j] = 1 and a zero
 // sub-column (and, with zero_row, a zero row).
@@ -214,13 +216,29 @@ __global__ void __launch_bounds__(512) chol_kernel(const zd *__restrict__ A, int
                                                    const zd *__restrict__ ref, int ldref) {
   extern __shared__ zd Ls[];   // k x k: A's lower triangle, then L before scaling; and k x k: the inverse before scaling
   zd *X = Ls + (size_t)k * k;
-  __shared__ double rs[64], tolref[64], inv[64];
+  __shared__ double rs[64], tolref[64], inv[64], scale[64];
   __shared__ int deads[64];
   const int t = threadIdx.x, nt = blockDim.x;
+  // the diagonal's high words (k <= 64), the same in every warp
+  const int i0 = t & 31, i1 = i0 + 32;
+  const int h0 = i0 < k ? __double2hiint(A[(size_t)i0 * lda + i0].re) : 0, h1 = i1 < k ? __double2hiint(A[(size_t)i1 * lda + i1].re) : 0;
   for (int e = t; e < k * k; e += nt) {
     const int i = e % k, j = e / k;
     Ls[e] = (i >= j) ? A[(size_t)j * lda + i] : mk<double>(0, 0);
     X[e] = mk<double>(i == j ? 1.0 : 0.0, 0);
+  }
+  auto exponent = [](int hi) { return (hi >> 20) - 1023; };
+  auto usable = [&](int hi) { return hi > 0 && exponent(hi) < 1024; };   // positive and finite
+  const bool far = __any_sync(0xffffffffu, (usable(h0) && abs(exponent(h0)) > 400) || (usable(h1) && abs(exponent(h1)) > 400));
+  if (far) {
+    auto factor = [&](int hi) { return __hiloint2double((1023 - (usable(hi) ? exponent(hi) >> 1 : 0)) << 20, 0); };
+    if (t < 32 && i0 < k) scale[i0] = factor(h0);
+    if (t < 32 && i1 < k) scale[i1] = factor(h1);
+    __syncthreads();
+    for (int e = t; e < k * k; e += nt) {
+      const double si = scale[e % k], sj = scale[e / k];
+      Ls[e] = mk<double>(Ls[e].re * si * sj, Ls[e].im * si * sj);
+    }
   }
   if (t < 32) {
     double m = 0.0;
@@ -234,6 +252,7 @@ __global__ void __launch_bounds__(512) chol_kernel(const zd *__restrict__ A, int
     for (int i = t; i < k; i += 32) {
       const double r = ref ? ref[(size_t)i * ldref + i].re : m;
       tolref[i] = r > 0.0 ? tol * r : __longlong_as_double(0x7ff0000000000000ll);   // no positive reference: dead
+      if (far) tolref[i] = tolref[i] * scale[i] * scale[i];
     }
   }
   __syncthreads();
@@ -249,11 +268,13 @@ __global__ void __launch_bounds__(512) chol_kernel(const zd *__restrict__ A, int
     } else if (i == j) {
       l.re = deads[j] ? 1.0 : Ls[e].re * rs[j];
     }
+    if (far && !(i == j && deads[j])) l = (1.0 / scale[i]) * l;
     if (Lout) Lout[(size_t)j * ldl + i] = l;
     if (Iout) {
       zd x = mk<double>(0, 0);
       if (i > j && !row0) x = mk<double>(X[e].re * rs[i], X[e].im * rs[i]);
       else if (i == j) x.re = rs[i];
+      if (far) x = deads[i] ? (scale[j] / scale[i]) * x : scale[j] * x;
       if (inv_h) Iout[(size_t)i * ldi + j] = conj(x);
       else Iout[(size_t)j * ldi + i] = x;
     }
