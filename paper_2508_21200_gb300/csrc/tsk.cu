@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__
     for (int m = 0; m < nq; ++m) {
       const cx<T> *qm = reinterpret_cast<const cx<T> *>(a.q[m]) + (size_t)row0 * r;
       cx<T> *dst = qs + (size_t)m * BS;
-      if (rp == r && (r % 2 == 0) && sizeof(T) == 4) {
+      if (rp == r && CPT > 1 && sizeof(T) == 4) {
         // 16-byte vectors: two complex64 per load
         const int hr = r / 2;
         for (int e = tid; e < tr * hr; e += TS_THREADS) {
@@ -886,6 +886,16 @@ __global__ void __launch_bounds__(512) reduce_kernel(const double *__restrict__ 
 int ts_max_grid(int nsm) { return 2 * nsm; }
 size_t ts_partial_doubles(int gram_left, int r) { return (size_t)(gram_left + 1) * r * r * 2; }
 
+// The widest column group that the row length and the alignment of the blocks allow (two complex64 are loaded as 16 bytes; a
+// caller's block may start on any element).
+static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+template <typename T>
+static int ts_cpt(const TSArgs &a) {
+  bool ok = a.r % 2 == 0 && (a.mode == 2 || aligned16(a.src));
+  for (int m = 0; m < a.nq; ++m) ok = ok && aligned16(a.q[m]);
+  return !ok ? 1 : (sizeof(T) == 4 && a.r % 4 == 0 ? 4 : 2);
+}
+
 template <typename T>
 static int launch_ts_v1(const TSArgs &a, int nsm, cudaStream_t st) {
   const int r = a.r;
@@ -910,11 +920,7 @@ static int launch_ts_v1(const TSArgs &a, int nsm, cudaStream_t st) {
   const long long ntiles = (a.N + tr - 1) / tr;
   int grid = (int)(ntiles < (long long)ts_max_grid(nsm) ? ntiles : ts_max_grid(nsm));
   if (grid < 1) grid = 1;
-  // pick the widest column group the row length and alignment allow
-  const int cpt_max = sizeof(T) == 4 ? 4 : 2;
-  int cpt = 1;
-  if (r % cpt_max == 0) cpt = cpt_max;
-  else if (r % 2 == 0) cpt = 2;
+  const int cpt_max = sizeof(T) == 4 ? 4 : 2, cpt = ts_cpt<T>(a);
   auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(a, tr, coef_smem ? 1 : 0, coefg); };
   if (cpt == 4) go(ts_kernel<T, (sizeof(T) == 4 ? 4 : 2)>);
   else if (cpt == 2) go(ts_kernel<T, 2>);
@@ -942,11 +948,10 @@ static TS3Plan ts3_plan(const TSArgs &a) {
   const int nq = a.nq, gl = a.gram_left, mode = a.mode;
   const int nb = nq + (mode != 2 ? 1 : 0);
   if (nb < 1 || nb > 8 || gl + 1 > 8 || gl > nq || (mode == 2 && nq < 1)) return p;
-  auto al = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
   for (int m = 0; m < nq; ++m)
-    if (!al(a.q[m])) return p;
-  if (mode != 2 && !al(a.src)) return p;
-  if (a.out && !al(a.out)) return p;
+    if (!aligned16(a.q[m])) return p;
+  if (mode != 2 && !aligned16(a.src)) return p;
+  if (a.out && !aligned16(a.out)) return p;
   const int r = p.R = a.r <= 8 ? 8 : (a.r <= 16 ? 16 : 32);
   if (r == 32 && a.r < 32 && (a.r < 24 || gl + 1 < 4)) return p;
   const int two = r != a.r ? 0 : (r == 16 ? gl + 1 <= 4 : (r == 32 ? gl + 1 <= 3 : 0));
@@ -1037,10 +1042,7 @@ static int launch_ts_t(const TSArgs &a, int nsm, cudaStream_t st) {
   const long long ntiles = (a.N + tr - 1) / tr;
   int grid = (int)(ntiles < (long long)ts_max_grid(nsm) ? ntiles : ts_max_grid(nsm));
   if (grid < 1) grid = 1;
-  const int cpt_max = sizeof(T) == 4 ? 4 : 2;
-  int cpt = 1;
-  if (r % cpt_max == 0) cpt = cpt_max;
-  else if (r % 2 == 0) cpt = 2;
+  const int cpt_max = sizeof(T) == 4 ? 4 : 2, cpt = ts_cpt<T>(a);
   auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(a, tr, coefg); };
   if (mt == 1) {
     if (cpt == cpt_max && cpt_max == 4) go(ts2_kernel<T, (sizeof(T) == 4 ? 4 : 2), 1>);
@@ -1159,7 +1161,7 @@ void launch_reduce(const double *partial, int nparts, int len_doubles, double *o
 void launch_hv(bool fp64, const ModelArgs &M, const void *X, void *Y, long long N, int r, int nsm, cudaStream_t st,
                int *status) {
   if (launch_hv_tiled(fp64, M, X, Y, N, r, nsm, st, status)) return;
-  // rows that are not a multiple of 16 bytes, or fewer than 16 rows: the per-row gather
+  // rows that are not a multiple of 16 bytes, blocks that do not start on one, or fewer than 16 rows: the per-row gather
   auto grid_for = [&](int cpt) {
     long long total = N * (r / cpt);
     long long g = (total + 255) / 256;
@@ -1172,8 +1174,8 @@ void launch_hv(bool fp64, const ModelArgs &M, const void *X, void *Y, long long 
     else { ::lrei::count_launch(); hv_kernel<T, 1><<<grid_for(1), 256, 0, st>>>(M, (const cx<T> *)X, (cx<T> *)Y, N, r); }
   } else {
     using T = float;
-    if (r % 4 == 0) { ::lrei::count_launch(); hv_kernel<T, 4><<<grid_for(4), 256, 0, st>>>(M, (const cx<T> *)X, (cx<T> *)Y, N, r); }
-    else if (r % 2 == 0) { ::lrei::count_launch(); hv_kernel<T, 2><<<grid_for(2), 256, 0, st>>>(M, (const cx<T> *)X, (cx<T> *)Y, N, r); }
+    if (r % 4 == 0 && aligned16(X)) { ::lrei::count_launch(); hv_kernel<T, 4><<<grid_for(4), 256, 0, st>>>(M, (const cx<T> *)X, (cx<T> *)Y, N, r); }
+    else if (r % 2 == 0 && aligned16(X)) { ::lrei::count_launch(); hv_kernel<T, 2><<<grid_for(2), 256, 0, st>>>(M, (const cx<T> *)X, (cx<T> *)Y, N, r); }
     else { ::lrei::count_launch(); hv_kernel<T, 1><<<grid_for(1), 256, 0, st>>>(M, (const cx<T> *)X, (cx<T> *)Y, N, r); }
   }
 }
