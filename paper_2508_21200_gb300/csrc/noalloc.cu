@@ -26,8 +26,8 @@ namespace {
 constexpr int NA_MAX_R = LREI_NOALLOC_MAX_R;
 constexpr int NA_PARTS = 152;                               // partial sums (CTAs) at most
 constexpr size_t NA_ENT = 6ull * NA_MAX_R * NA_MAX_R * 2;    // doubles per partial (6 r x r Grams)
-// partials + 16 reduction slices + reduced Grams + spectrum + outputs
-constexpr size_t NA_DOUBLES = (NA_PARTS + 16) * NA_ENT + NA_ENT + 64 + 64;
+// partials + reduced Grams + spectrum + outputs
+constexpr size_t NA_DOUBLES = NA_PARTS * NA_ENT + NA_ENT + 64 + 64;
 
 static __device__ __align__(256) double g_noalloc_scratch[NA_DOUBLES];
 
@@ -58,7 +58,7 @@ extern "C" int lrei_observables_noalloc(int n, const lrei_bonds *J, const double
   double *base = scratch_for_current_device(&code);
   if (!base) return code;
   double *partial = base;
-  double *red = base + (NA_PARTS + 16) * NA_ENT;
+  double *red = base + NA_PARTS * NA_ENT;
   double *lam = red + NA_ENT;
   double *res = lam + 64;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);

@@ -17,11 +17,6 @@ namespace lrei {
 // [0] FP32 Jacobi calls, [1] FP32 sweeps, [2] FP64 Jacobi calls, [3] FP64 sweeps (diagnostics)
 __device__ unsigned long long g_jacobi_counters[4];
 
-__device__ __forceinline__ zd zdiv_real(zd a, double d) { return mk<double>(a.re / d, a.im / d); }
-__device__ __forceinline__ zd zdiv(zd a, zd d) {
-  const double n = d.re * d.re + d.im * d.im;
-  return mk<double>((a.re * d.re + a.im * d.im) / n, (a.im * d.re - a.re * d.im) / n);
-}
 __device__ __forceinline__ zd warp_sum(zd v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -134,32 +129,27 @@ void sm_gemm_herm(char opA, char opB, int M, int K, zd alpha, const zd *A, int l
 }
 
 // ------------------------------------------------------- triangular solves
-// Triangular solves, one warp per right-hand side, four warps per CTA sharing one copy of the
+// Triangular solves (k <= MAX_R), one warp per right-hand side, four warps per CTA sharing one copy of the
 // triangle in shared memory.  Right-looking: x_j = b_j / d_j is broadcast from shared memory and
 // every lane updates the rows it owns, so the loop has no reductions and no divisions (the
-// reciprocal diagonal is precomputed).  Up to k = 90 the triangle is staged in shared memory
-// (column j of T holds the multipliers of x_j); larger k reads it from global memory.
-constexpr int TRSV_SMEM_K = 90;
+// reciprocal diagonal is precomputed).
 __global__ void __launch_bounds__(128) trsv_kernel(char op, const zd *__restrict__ L, int ldl, int k,
                                                    zd *__restrict__ B, int ldb, int ncols) {
   extern __shared__ zd trsv_sm[];
-  const bool staged = k <= TRSV_SMEM_K;
   zd *Ts = trsv_sm;                                  // k x k: Ts[j*k + i] = multiplier of x_j in row i
-  zd *xs = staged ? trsv_sm + (size_t)k * k : trsv_sm;    // 4 warps x k
+  zd *xs = trsv_sm + (size_t)k * k;                  // 4 warps x k
   double *rd = reinterpret_cast<double *>(xs + 4 * k);   // k reciprocal diagonal entries
   const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
   for (int i = t; i < k; i += blockDim.x) {
     const double d = L[(size_t)i * ldl + i].re;
     rd[i] = d != 0.0 ? 1.0 / d : 0.0;
   }
-  if (staged) {
-    for (int e = t; e < k * k; e += blockDim.x) {
-      const int i = e % k, j = e / k;
-      zd v = mk<double>(0, 0);
-      if (op == 'N') { if (i > j) v = L[(size_t)j * ldl + i]; }          // L(i, j)
-      else { if (i < j) v = conj(L[(size_t)i * ldl + j]); }               // (L^H)(i, j) = conj(L(j, i))
-      Ts[e] = v;
-    }
+  for (int e = t; e < k * k; e += blockDim.x) {
+    const int i = e % k, j = e / k;
+    zd v = mk<double>(0, 0);
+    if (op == 'N') { if (i > j) v = L[(size_t)j * ldl + i]; }          // L(i, j)
+    else { if (i < j) v = conj(L[(size_t)i * ldl + j]); }               // (L^H)(i, j) = conj(L(j, i))
+    Ts[e] = v;
   }
   const int col = blockIdx.x * 4 + wp;
   zd *x = xs + wp * k;
@@ -168,17 +158,13 @@ __global__ void __launch_bounds__(128) trsv_kernel(char op, const zd *__restrict
     for (int i = lane; i < k; i += 32) x[i] = bcol[i];
   __syncthreads();
   if (col < ncols) {
-    auto mult = [&](int i, int j) -> zd {
-      if (staged) return Ts[(size_t)j * k + i];
-      return op == 'N' ? L[(size_t)j * ldl + i] : conj(L[(size_t)i * ldl + j]);
-    };
     if (op == 'N') {
       for (int j = 0; j < k; ++j) {
         __syncwarp();
         const zd xj = mk<double>(x[j].re * rd[j], x[j].im * rd[j]);
         __syncwarp();
         if (lane == 0) x[j] = xj;
-        for (int i = j + 1 + lane; i < k; i += 32) x[i] = x[i] - mult(i, j) * xj;
+        for (int i = j + 1 + lane; i < k; i += 32) x[i] = x[i] - Ts[j * k + i] * xj;
       }
     } else {
       for (int j = k - 1; j >= 0; --j) {
@@ -186,7 +172,7 @@ __global__ void __launch_bounds__(128) trsv_kernel(char op, const zd *__restrict
         const zd xj = mk<double>(x[j].re * rd[j], x[j].im * rd[j]);
         __syncwarp();
         if (lane == 0) x[j] = xj;
-        for (int i = lane; i < j; i += 32) x[i] = x[i] - mult(i, j) * xj;
+        for (int i = lane; i < j; i += 32) x[i] = x[i] - Ts[j * k + i] * xj;
       }
     }
     __syncwarp();
@@ -196,7 +182,7 @@ __global__ void __launch_bounds__(128) trsv_kernel(char op, const zd *__restrict
 
 void sm_trsv(char op, const zd *L, int ldl, int k, zd *B, int ldb, int ncols, cudaStream_t st) {
   if (ncols <= 0 || k <= 0) return;
-  const size_t bytes = ((k <= TRSV_SMEM_K ? (size_t)k * k : 0) + 4 * (size_t)k) * sizeof(zd) + (size_t)k * 8;
+  const size_t bytes = ((size_t)k * k + 4 * (size_t)k) * sizeof(zd) + (size_t)k * 8;
   ::lrei::count_launch();
   trsv_kernel<<<(ncols + 3) / 4, 128, bytes, st>>>(op, L, ldl, k, B, ldb, ncols);
 }
@@ -994,16 +980,6 @@ __global__ void hermitize_kernel(zd *A, int lda, int k) {
 }
 void sm_hermitize(zd *A, int lda, int k, cudaStream_t st) { ::lrei::count_launch(); hermitize_kernel<<<grid_for((long long)k * k), 256, 0, st>>>(A, lda, k); }
 
-__global__ void scale_kernel(zd *A, int lda, int M, int N, double s) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < M * N; e += gridDim.x * blockDim.x) {
-    const int i = e % M, j = e / M;
-    A[(size_t)j * lda + i] = s * A[(size_t)j * lda + i];
-  }
-}
-void sm_scale_cols(zd *A, int lda, int M, int N, double s, cudaStream_t st) {
-  ::lrei::count_launch(); scale_kernel<<<grid_for((long long)M * N), 256, 0, st>>>(A, lda, M, N, s);
-}
-
 // B = (A + A^H)/2, k x k.
 __global__ void herm_copy_kernel(const zd *__restrict__ A, int lda, int k, zd *__restrict__ B, int ldb) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < k * k; e += gridDim.x * blockDim.x) {
@@ -1021,7 +997,6 @@ void sm_herm_copy(const zd *A, int lda, int k, zd *B, int ldb, cudaStream_t st) 
 namespace lrei {
 int sm_init() {
   const int lim = 210 * 1024;
-  cudaFuncSetAttribute(trsv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   cudaError_t a = cudaFuncSetAttribute(jacobi32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   return a == cudaSuccess ? 0 : -1;

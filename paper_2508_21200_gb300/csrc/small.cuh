@@ -17,7 +17,7 @@ void sm_gemm_herm(char opA, char opB, int M, int K, zd alpha, const zd *A, int l
                   const zd *Cin, int ldin, zd *C, int ldc, cudaStream_t st);
 
 // For each of ncols columns of B (in place): solve L x = b (op 'N') or L^H x = b (op 'C'),
-// L lower triangular k x k.  A zero diagonal entry gives x_i = 0.
+// L lower triangular k x k, k <= MAX_R.  A zero diagonal entry gives x_i = 0.
 void sm_trsv(char op, const zd *L, int ldl, int k, zd *B, int ldb, int ncols, cudaStream_t st);
 
 // Cholesky A = L L^H of a Hermitian k x k matrix (k <= 64), one CTA.  A pivot below
@@ -47,7 +47,6 @@ void sm_copy(const zd *A, int lda, int M, int N, zd *B, int ldb, cudaStream_t st
 void sm_zero(zd *A, int lda, int M, int N, cudaStream_t st);
 void sm_set_identity(zd *A, int lda, int M, int N, cudaStream_t st);                         // A = [I; 0]
 void sm_hermitize(zd *A, int lda, int k, cudaStream_t st);                                  // A <- (A + A^H)/2
-void sm_scale_cols(zd *A, int lda, int M, int N, double s, cudaStream_t st);
 void sm_herm_copy(const zd *A, int lda, int k, zd *B, int ldb, cudaStream_t st);              // B = (A + A^H)/2
 
 }  // namespace lrei

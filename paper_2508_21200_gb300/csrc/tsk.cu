@@ -1057,7 +1057,7 @@ static int launch_ts_t(const TSArgs &a, int nsm, cudaStream_t st) {
 }
 
 // ------------------------------------------- few rows
-// Passes of few rows are latency: tiles leave most SMs idle (one CTA per 256 rows in the complex128 pass) and their sums need
+// Passes of few rows are latency: tiles leave most SMs idle (8 to 256 of them at N = 256 .. 4096) and their sums need
 // a second launch.  Here every entry of the new block is a sum over eight lanes and every Gram entry one over a warp
 // or a CTA, in FP64 for both precisions (the coefficients as they are), and the Gram goes to a.red directly.
 // The rows of a CTA are read before one is written, so the new block may replace an input.

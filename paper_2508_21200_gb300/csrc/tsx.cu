@@ -719,7 +719,7 @@ int tsx_run(const TSArgs &a, bool proj, const XPlan &p, int nsm, cudaStream_t st
   const int occ = std::max(1, std::min(16 / w, 228 * 1024 / (p.bytes + 2048)));
   const long long ntiles = a.N / p.kt;
   long long gx = (long long)occ * nsm / gy;
-  // the caller's buffer holds (2 nsm + 16) partials of MAXB + 1 blocks, 16 of them for the reduction
+  // the caller's buffer holds at least 2 nsm partials of MAXB + 1 blocks
   if (!proj) gx = std::min(gx, 2LL * nsm * (MAXB + 1) / ng);
   gx = std::max(1LL, std::min(gx, ntiles));
   const dim3 grid((unsigned)gx, (unsigned)gy);
@@ -737,7 +737,7 @@ int tsx_run(const TSArgs &a, bool proj, const XPlan &p, int nsm, cudaStream_t st
 // 16-row tiles only, and the pass was slower than the two (n = 20, r = 16, five blocks: 7.1 ms against 2.6 + 1.9).
 // Measured against the general kernel (ts2_kernel) at n = 20, r = 16: Gram of 1 / 2 / 3 / 5 blocks 1.83 / 3.66 / 5.55 /
 // 10.96 ms there and 0.26 / 0.49 / 0.67 / 0.99 ms here (the five blocks' tensor work alone is 0.47 ms), the projection of
-// five blocks onto one 2.2 ms, an RK4 step 96.0 and 22.2 ms; at n = 8, r = 4 the Gram of four 22.8 and 19.5 us.
+// five blocks onto one 2.2 ms, an RK4 step 96.0 and 22.2 ms.
 int launch_tsx(const TSArgs &a, int nsm, cudaStream_t st) {
   if ((a.mode == 0 && a.out) || (a.mode != 0 && !a.out) || a.r > MAX_R || a.N < 256) return 0;
   auto off = [](const void *x) { return (reinterpret_cast<uintptr_t>(x) & 15) != 0; };
