@@ -11,10 +11,18 @@
 // others are below 2^-55 of the largest); those of equal s + t share an accumulator (a "class").  Every 128 complex summands
 // (the rows of a Gram, the columns of a projection: 2 x 128 x 4 x 2^14 = 2^24 for the first four classes; a class beyond
 // the fourth carries less than 2^-32 of the result) the classes go into two 64-bit integers per entry, without rounding.
-// A column keeps its exponent from tile to tile while the tile's largest entry stays within a few bits below it;
+// In a Gram a column keeps its exponent from tile to tile while the tile's largest entry stays within a few bits below it;
 // when it does not, the sums so far are flushed to the CTA's FP64 partial at the old exponents and the column
-// gets a new one, so no tile loses bits to a larger one.  A tile with infinities, NaN or entries near the ends of
-// the exponent range takes a direct path in FP64 FMAs.
+// gets a new one, so no tile loses bits to a larger one.  An entry is off by 2^-52 of its columns' norms: an entry of a column
+// beside a larger one of the same tile keeps fewer bits, which the sum over the rows does not see.
+// A projection does: each of its rows is a result.  There the exponents are those of the rows, after the columns are
+// weighted: with 2^(g_k) the largest coefficient of input column k,
+//     new_rj = sum_k (x_rk 2^(g_k)) (c_kj 2^(-g_k)),
+// the entries of row r share the exponent e_r of the largest weighted one and the coefficients of output j the exponent f_j, and
+// the result is off by 2^-52 K max_k |x_rk| max_j |c_kj| whatever the other rows of the tile hold (a column exponent per
+// tile lost as many bits of a row as it was smaller than the largest of 16 or 32 rows).  g and the digits of the
+// coefficients are made once per CTA.
+// A tile with infinities, NaN or entries near the ends of the exponent range takes a direct path in FP64 FMAs.
 //
 // Layout.  A column group is 8 complex columns of one block (ranks that are not a multiple of 8 are padded by
 // repeating the last column), a chunk is 16 rows.  A thread (g = lane / 4, q = lane % 4) of a cutting warp
@@ -58,6 +66,9 @@ constexpr int X_DRAIN = 128;          // complex summands between drains
 constexpr int X_SLACK = 2;            // bits a column's tile may stay below its exponent
 constexpr int X_EMIN = 530, X_EMAX = 1510;   // exponent fields that are cut; others take the direct path
 constexpr int E_UNSET = -100000;
+// projections: exponents of the rows that are cut, of the coefficients' largest (either side); a zero coefficient row; the
+// bias of a row's key (0: a zero row)
+constexpr int X_RMIN = -450, X_RMAX = 480, X_GMAX = 400, G_ZERO = -3000, X_BIAS = 8192;
 // named barriers: planes b full (BAR_FULL + b), free again (BAR_FREE + b), the multiplying and the cutting warps
 constexpr int BAR_FULL = 1, BAR_FREE = 3, BAR_MUL = 5, BAR_CUT = 6;
 
@@ -114,7 +125,7 @@ __device__ __forceinline__ unsigned long long fixed_biased_k(double x, int k) {
   const int E = (int)(b >> 52) & 0x7ff;
   unsigned long long m = (b & 0xfffffffffffffull) | (E ? 0x10000000000000ull : 0ull);
   const int sh = k + (E ? E : 1) - 1075;
-  if (sh >= 0) m <<= sh;
+  if (sh >= 0) m <<= min(sh, 63);   // a zero may come with any scale
   else if (sh > -56) m = (m + (1ull << (-sh - 1))) >> (-sh);
   else m = 0;
   return ((long long)b < 0 ? 0ull - m : m) + 0x80808080808080ull;
@@ -191,7 +202,9 @@ struct Geo {
   unsigned char *sums;    // [entry][nt] the threads' sums
   uint32_t *coef;         // [group][column group][digit][re, im][32]
   double *nv;             // [kt][ldnv] the new tile
-  uint32_t *key;          // [4][ncl] magnitude keys of the columns (tile & 3)
+  int *rowkey;            // projection: [4][kt] biased exponents of the weighted rows (tile & 3)
+  int *gam;               // projection: [ncl] exponents g of the input columns
+  uint32_t *key;          // Gram: [4][ncl] magnitude keys of the columns (tile & 3)
   int *ecol;              // [4][ncl] exponents of the columns in a tile (tile & 3)
   int *eacc;              // [ncl] exponents of the sums since the last flush
   int *fcol;              // [npb * 8] exponents of the coefficient columns
@@ -216,10 +229,13 @@ struct Geo {
     sums = tsx_smem + p.o_sums;
     coef = reinterpret_cast<uint32_t *>(tsx_smem + p.o_coef);
     nv = reinterpret_cast<double *>(tsx_smem + p.o_nv);
-    key = reinterpret_cast<uint32_t *>(tsx_smem + p.o_int);
-    ecol = reinterpret_cast<int *>(key + 4 * ncl);
+    int *at = reinterpret_cast<int *>(tsx_smem + p.o_int);
+    rowkey = at;
+    gam = rowkey + 4 * p.kt;
+    key = reinterpret_cast<uint32_t *>(at);
+    ecol = at + 4 * ncl;
     eacc = ecol + 4 * ncl;
-    fcol = eacc + ncl;
+    fcol = PROJ ? gam + ncl : eacc + ncl;
     flags = fcol + p.npb * 8;
     outp = reinterpret_cast<double2 *>(a.partial + (size_t)blockIdx.x * ng * a.r * a.r * 2);
   }
@@ -236,20 +252,35 @@ __device__ __forceinline__ zd coef_at(const TSArgs &a, int b, int i, int j) {
   return a.coefS ? a.coefS[(size_t)j * r + i] : mk<double>(0, 0);
 }
 
-// Digit planes of the coefficients, each row k scaled by its column's 2^(e_k - 7); by the multiplying warps.
-__device__ __forceinline__ void slice_coefs(const TSArgs &a, const XPlan &p, const Geo<true> &G, const int *ecol) {
-  const int tid = threadIdx.x, r = a.r, cpb = p.cpb, np = G.np, c0 = G.n0 * 8;
+// Exponents g of the coefficient rows of this CTA's columns; by the multiplying warps.
+__device__ __forceinline__ void weigh_columns(const TSArgs &a, const XPlan &p, const Geo<true> &G) {
+  const int c0 = G.n0 * 8, rc = min(G.np * 8, a.r - c0), tid = threadIdx.x;
+  for (int k = tid; k < G.ncl; k += G.nt) G.gam[k] = 0;
+  bar_sync(BAR_MUL, G.nt);
+#pragma unroll 4
+  for (int e = tid; e < G.ncl * rc; e += G.nt) {
+    const int k = e % G.ncl, j = e / G.ncl;
+    const zd v = coef_at(a, k / (p.cpb * 8), k % (p.cpb * 8), c0 + j);
+    atomicMax(&G.gam[k], (int)max(mag_key(v.re), mag_key(v.im)));
+  }
+  bar_sync(BAR_MUL, G.nt);
+  for (int k = tid; k < G.ncl; k += G.nt) {
+    const int m = G.gam[k], g = (m >> 20) - 1022;
+    G.gam[k] = m ? g : G_ZERO;
+    if (m && abs(g) > X_GMAX) G.flags[0] = 1;   // also infinities and NaN: every tile directly
+  }
+}
+
+// Digit planes of the weighted coefficients; by the multiplying warps.
+__device__ __forceinline__ void slice_coefs(const TSArgs &a, const XPlan &p, const Geo<true> &G) {
+  const int tid = threadIdx.x, cpb = p.cpb, np = G.np, c0 = G.n0 * 8;
   for (int j = tid; j < np * 8; j += G.nt) G.fcol[j] = E_UNSET;
   bar_sync(BAR_MUL, G.nt);
   for (int e = tid; e < G.ncg * 8 * np * 8; e += G.nt) {
     const int j = e / (G.ncg * 8), k = e % (G.ncg * 8), b = k / (cpb * 8), i = k % (cpb * 8);
-    const int ek = ecol[k];
-    if (i >= r || ek == E_UNSET) continue;
     const zd v = coef_at(a, b, i, c0 + j);
     const uint32_t m = max(mag_key(v.re), mag_key(v.im));
-    const int E = (int)(m >> 20);
-    if (E >= 0x7ff) G.flags[0] = 1;
-    if (m >= (1u << 20)) atomicMax(&G.fcol[j], E - 1022 + ek - 7);
+    if (m >= (1u << 20)) atomicMax(&G.fcol[j], (int)(m >> 20) - 1022 - G.gam[k]);
   }
   bar_sync(BAR_MUL, G.nt);
   // word (group, column group, lane): rows 2q, 2q+1 of the group, output column g
@@ -257,15 +288,14 @@ __device__ __forceinline__ void slice_coefs(const TSArgs &a, const XPlan &p, con
     const int l = e & 31, gn = e >> 5, n = gn % np, cg = gn / np;
     const int j = n * 8 + (l >> 2), b = cg / cpb, i = (cg % cpb) * 8 + 2 * (l & 3);
     const int f = G.fcol[j];
-    const int e0 = ecol[cg * 8 + 2 * (l & 3)], e1 = ecol[cg * 8 + 2 * (l & 3) + 1];
     uint32_t dr[NS], di[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) dr[s] = di[s] = 0;
     if (f != E_UNSET && !G.flags[0]) {
-      const zd z = mk<double>(0, 0);
-      const zd v0 = e0 == E_UNSET ? z : coef_at(a, b, i, c0 + j), v1 = e1 == E_UNSET ? z : coef_at(a, b, i + 1, c0 + j);
-      digit_planes(fixed_biased_k(v0.re, e0 - f + 48), fixed_biased_k(v1.re, e1 - f + 48), dr);
-      digit_planes(fixed_biased_k(v0.im, e0 - f + 48), fixed_biased_k(v1.im, e1 - f + 48), di);
+      const zd v0 = coef_at(a, b, i, c0 + j), v1 = coef_at(a, b, i + 1, c0 + j);
+      const int k0 = 55 - f - G.gam[cg * 8 + 2 * (l & 3)], k1 = 55 - f - G.gam[cg * 8 + 2 * (l & 3) + 1];
+      digit_planes(fixed_biased_k(v0.re, k0), fixed_biased_k(v1.re, k1), dr);
+      digit_planes(fixed_biased_k(v0.im, k0), fixed_biased_k(v1.im, k1), di);
     }
     uint32_t *w = G.coef + (size_t)gn * NS * 64;
 #pragma unroll
@@ -330,13 +360,30 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(full_a));
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  for (int i = tid; i < 4 * ncl; i += all) {
-    G.key[i] = 0;
-    G.ecol[i] = E_UNSET;
-  }
-  for (int i = tid; i < ncl; i += all) G.eacc[i] = E_UNSET;
+  // thread nt (the first that cuts): the blocks' tiles by one bulk copy each
+  const uint32_t tile_bytes = (uint32_t)p.kt * r * 16u;
+  auto fetch = [&](long long tile) {
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(G.raw);
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(full_a), "r"(tile_bytes * G.nload) : "memory");
+    for (int b = 0; b < G.nload; ++b)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                       dst + (uint32_t)(b * p.kt * r) * 16u),
+                   "l"(G.block(a, b) + (size_t)tile * p.kt * r), "r"(tile_bytes), "r"(full_a)
+                   : "memory");
+  };
   if (tid < 12) G.flags[tid] = 0;
-  if (!PROJ) {
+  if constexpr (PROJ) {
+    for (int i = tid; i < 4 * p.kt; i += all) G.rowkey[i] = 0;
+    __syncthreads();   // the flags and the barrier are set
+    if (tid == nt) fetch(blockIdx.x);
+    if (warp < p.wm) weigh_columns(a, p, G);
+  } else {
+    for (int i = tid; i < 4 * ncl; i += all) {
+      G.key[i] = 0;
+      G.ecol[i] = E_UNSET;
+    }
+    for (int i = tid; i < ncl; i += all) G.eacc[i] = E_UNSET;
     const int nr = (G.rb1 - G.rb0) * r;   // the partial: zero until the first flush
     for (int e = tid; e < nr * r; e += all)
       G.outp[(size_t)(e / nr) * (a.gram_left + 1) * r + G.rb0 * r + e % nr] = make_double2(0.0, 0.0);
@@ -363,21 +410,9 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
     }
     const int rs = 4 * r;
     uint32_t *const dig32 = reinterpret_cast<uint32_t *>(G.dig);
-    // thread ct = 0: the blocks' tiles by one bulk copy each
-    const uint32_t tile_bytes = (uint32_t)p.kt * r * 16u;
-    auto fetch = [&](long long tile) {
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(G.raw);
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(full_a), "r"(tile_bytes * G.nload) : "memory");
-      for (int b = 0; b < G.nload; ++b)
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                         dst + (uint32_t)(b * p.kt * r) * 16u),
-                     "l"(G.block(a, b) + (size_t)tile * p.kt * r), "r"(tile_bytes), "r"(full_a)
-                     : "memory");
-    };
-    if (ct == 0) fetch(blockIdx.x);
+    if (!PROJ && ct == 0) fetch(blockIdx.x);
     for (int i = 0; i < mine; ++i) {
-      uint32_t *key = G.key + (i & 3) * ncl;
+      uint32_t *key = G.key + (i & 3) * ncl;   // Gram
       // after a copy that never landed nothing more is fetched or waited for; the loop runs on for its barriers
       if (!G.flags[1] && !wait_phase(full_a, (uint32_t)(i & 1))) G.flags[1] = 1;
       zd raw[CUT_UNITS][4];
@@ -388,50 +423,96 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
 #pragma unroll
           for (int k = 0; k < 4; ++k) raw[x][k] = v[k * rs];
         }
-      uint32_t m = 0;
+      if constexpr (PROJ) {
+        // the rows' largest weighted exponents over this warp's columns: per chunk, rows q + 4 k
+        int rv[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
 #pragma unroll
-      for (int x = 0; x < CUT_UNITS; ++x)
-        if (x < nu) {
+        for (int x = 0; x < CUT_UNITS; ++x)
+          if (x < nu) {
+            const int gk = G.gam[ucol[x]];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) m = max(m, max(mag_key(raw[x][k].re), mag_key(raw[x][k].im)));
-          if (((x + 1) & (nkc - 1)) == 0) {   // the group's last chunk (nkc is 1 or 2): over the lanes of a column
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-            if (q == 0) key[ucol[x]] = m;
-            m = 0;
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t m = max(mag_key(raw[x][k].re), mag_key(raw[x][k].im));
+              const int E = (int)(m >> 20);
+              // infinities and NaN count whatever their coefficients
+              const int v = E == 0x7ff ? 1 << 20 : (m == 0 || gk == G_ZERO ? 0 : E + gk + X_BIAS);
+              if (nkc == 1 || (x & 1) == 0) rv[0][k] = max(rv[0][k], v);
+              else rv[1][k] = max(rv[1][k], v);
+            }
           }
-        }
+        int *rk = G.rowkey + (i & 3) * p.kt;
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          if (c < nkc) {   // over the columns (lane bits 2..4): halving the rows twice
+            const bool u4 = lane & 16, u3 = lane & 8;
+            const int s0 = u4 ? rv[c][0] : rv[c][2], s1 = u4 ? rv[c][1] : rv[c][3];
+            const int a0 = max(u4 ? rv[c][2] : rv[c][0], __shfl_xor_sync(0xffffffffu, s0, 16));
+            const int a1 = max(u4 ? rv[c][3] : rv[c][1], __shfl_xor_sync(0xffffffffu, s1, 16));
+            int v = max(u3 ? a1 : a0, __shfl_xor_sync(0xffffffffu, u3 ? a0 : a1, 8));
+            v = max(v, __shfl_xor_sync(0xffffffffu, v, 4));
+            if (!(lane & 4) && v) atomicMax(&rk[c * 16 + q + (u4 ? 8 : 0) + (u3 ? 4 : 0)], v);
+          }
+        // the keys of tile i - 3 become those of tile i + 1 (they were last read before its planes were released)
+        if (ct < p.kt) G.rowkey[((i + 1) & 3) * p.kt + ct] = 0;
+      } else {
+        uint32_t m = 0;
+#pragma unroll
+        for (int x = 0; x < CUT_UNITS; ++x)
+          if (x < nu) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) m = max(m, max(mag_key(raw[x][k].re), mag_key(raw[x][k].im)));
+            if (((x + 1) & (nkc - 1)) == 0) {   // the group's last chunk (nkc is 1 or 2): over the lanes of a column
+              m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+              m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+              if (q == 0) key[ucol[x]] = m;
+              m = 0;
+            }
+          }
+      }
       bar_sync(BAR_CUT, ncut);   // the raw tile is in registers: the next one goes out behind the arithmetic
       if (ct == 0 && i + 1 < mine && !G.flags[1]) fetch(blockIdx.x + (long long)(i + 1) * gridDim.x);
       // planes i & 1 are free once tile i - 2 is multiplied; its flags go with them
       if (i >= 2) bar_sync(BAR_FREE + (i & 1), all);
       int *flag = G.flags + 4 + 2 * (i & 3);
-      const int *el = G.ecol + ((i + 3) & 3) * ncl;   // before this tile: those of tile i - 1
+      const int *el = G.ecol + ((i + 3) & 3) * ncl;   // Gram, before this tile: those of tile i - 1
       uint32_t *cut = dig32 + (i & 1) * dig_words;
       int e = 0;
 #pragma unroll
       for (int x = 0; x < CUT_UNITS; ++x)
         if (x < nu) {
-          if ((x & (nkc - 1)) == 0) {
-            const uint32_t k = key[ucol[x]];
-            const int E = (int)(k >> 20), ex = E - 1022;   // |x| < 2^ex
-            e = el[ucol[x]];
-            if (k != 0 && (E < X_EMIN || E > X_EMAX)) {
-              flag[1] = 1;
-            } else if (k != 0 && (ex > e || ex < e - X_SLACK)) {
-              e = ex + 1;
-              flag[0] = 1;
+          int er[4];   // the exponents of the four values
+          if constexpr (PROJ) {
+            const int *rk = G.rowkey + (i & 3) * p.kt + (x & (nkc - 1)) * 16 + q, gk = G.gam[ucol[x]];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int v = rk[4 * k], ex = v - X_BIAS - 1022;
+              if (v && (ex < X_RMIN || ex > X_RMAX)) flag[1] = 1;
+              er[k] = (v ? ex : 0) - gk;
             }
-            G.ecol[(i & 3) * ncl + ucol[x]] = e;
-            if (e == E_UNSET) e = 0;   // zero so far: any exponent gives zero digits
+          } else {
+            if ((x & (nkc - 1)) == 0) {
+              const uint32_t k = key[ucol[x]];
+              const int E = (int)(k >> 20), ex = E - 1022;   // |x| < 2^ex
+              e = el[ucol[x]];
+              if (k != 0 && (E < X_EMIN || E > X_EMAX)) {
+                flag[1] = 1;
+              } else if (k != 0 && (ex > e || ex < e - X_SLACK)) {
+                e = ex + 1;
+                flag[0] = 1;
+              }
+              G.ecol[(i & 3) * ncl + ucol[x]] = e;
+              if (e == E_UNSET) e = 0;   // zero so far: any exponent gives zero digits
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) er[k] = e;
           }
           uint32_t *w = cut + udig[x];
 #pragma unroll
           for (int h = 0; h < 2; ++h) {   // rows q, q+4 and rows q+8, q+12; matrices re, re, im, im
             uint32_t dr[NS], di[NS];
             const zd u = raw[x][2 * h], v = raw[x][2 * h + 1];
-            digit_planes(fixed_biased(u.re, e), fixed_biased(v.re, e), dr);
-            digit_planes(fixed_biased(u.im, e), fixed_biased(v.im, e), di);
+            digit_planes(fixed_biased(u.re, er[2 * h]), fixed_biased(v.re, er[2 * h + 1]), dr);
+            digit_planes(fixed_biased(u.im, er[2 * h]), fixed_biased(v.im, er[2 * h + 1]), di);
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
               w[s * 128 + h * 32] = dr[s];
@@ -450,21 +531,14 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
 
   // ==== multiplying warps
   if constexpr (PROJ) {
-    bool sliced = false;
+    slice_coefs(a, p, G);
     zd *out = reinterpret_cast<zd *>(a.out);
     const int c0 = G.n0 * 8, rc = min(np * 8, r - c0);
     for (int i = 0; i < mine; ++i) {
       const long long row0 = (blockIdx.x + (long long)i * gridDim.x) * p.kt;
-      const int *el = G.ecol + (i & 3) * ncl;
+      const int *rk = G.rowkey + (i & 3) * p.kt;
       bar_sync(BAR_FULL + (i & 1), all);
-      const bool changed = G.flags[4 + 2 * (i & 3)] != 0;
-      bool direct = G.flags[5 + 2 * (i & 3)] != 0 || G.flags[0] != 0;
-      if (changed) sliced = false;   // also when this tile is direct: the next one that is cut has the new exponents
-      if (!direct && !sliced) {
-        slice_coefs(a, p, G, el);
-        sliced = true;
-        direct = G.flags[0] != 0;
-      }
+      const bool direct = G.flags[5 + 2 * (i & 3)] != 0 || G.flags[0] != 0;
       if (direct) {
         direct_new(a, p, G, row0);
       } else {
@@ -519,9 +593,9 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
             const int lr = kc * 16 + (k >= 2 ? 8 : 0) + (g & 1) * 4 + (g >> 1), j = n * 8 + 2 * q + (k & 1);
             if (c0 + j >= r) continue;
             const long long row = row0 + lr;
-            const int f = G.fcol[j] - 7;
+            const int f = G.fcol[j];
             double v = 0.0;
-            if (f != E_UNSET - 7 && row >= a.zero_rows) v = ints_value(hh[k], ll[k], f);
+            if (f != E_UNSET && row >= a.zero_rows) v = ints_value(hh[k], ll[k], rk[lr] - X_BIAS - 1022 + f - 14);
             G.nv[lr * p.ldnv + 2 * j + h] = v;
           }
         }
@@ -704,7 +778,7 @@ bool tsx_plan(const TSArgs &a, bool proj, XPlan *out) {
       b += proj ? kt * p.ldnv * 8 : 0;
       b = (b + 15) & ~15;
       p.o_int = b;
-      b += (9 * ncg * 8 + p.npb * 8 + 12) * 4;
+      b += ((proj ? 4 * kt + ncg * 8 : 9 * ncg * 8) + p.npb * 8 + 12) * 4;
       p.bytes = b;
       if (b > TSX_SMEM) continue;
       *out = p;

@@ -189,3 +189,28 @@ def test_sums_of_the_largest_digits(project, r, nq):
     err = max(abs(int(got[k, j]) - re[rows[N // 2 + k], j]) / re[rows[N // 2 + k], j] for k in range(0, N // 2, 7)
               for j in range(r))
     assert err < 4e-15
+
+
+@pytest.mark.parametrize("r,nq,extend", [(1, 1, False), (3, 1, False), (8, 2, True), (16, 4, True), (17, 3, False), (32, 4, True)])
+@pytest.mark.parametrize("columns", ["alike", "apart"])
+def test_rows_of_very_different_size(project, r, nq, extend, columns):
+    # Neighbouring rows 2^-90 .. 2^90 apart, and with "apart" the columns of the blocks too, undone by the rows of C: each row is as
+    # good as its own entries allow.  An entry x_rk is off by half of 2^-55 of the next power of two above the largest |x_rk| a_k, a_k
+    # the next above max_j |c_kj|, and so are the coefficients, of one: K 2^-53 x 4 together with the products left out (K 2^-52),
+    # below K 2^-49 max_k |x_rk| max_j |c_kj|, in which 2^3 covers the modulus of complex entries and torch's own sum.
+    N, m = 1 << 15, nq + (1 if extend else 0)
+    K = m * r
+    g = torch.Generator(device="cuda")
+    g.manual_seed(r * 10 + nq)
+    uniform = lambda n, bits: (2.0 ** (bits * (2 * torch.rand(n, dtype=torch.float64, device="cuda", generator=g) - 1)))  # noqa: E731
+    X = torch.randn((N, K), dtype=torch.complex128, device="cuda", generator=g) * uniform(N, 90)[:, None]
+    X[17::64] = 0
+    C = torch.randn((K, r), dtype=torch.complex128, device="cuda", generator=g)
+    if columns == "apart":
+        s = uniform(K, 60)
+        X, C = X * s, C / s[:, None]
+    blocks = [X[:, i * r:(i + 1) * r].contiguous() for i in range(m)]
+    out = project(blocks[:nq], blocks[nq] if extend else None, C)
+    M = (X.abs() * C.abs().amax(1)).amax(1, keepdim=True)
+    assert float(((out - X @ C).abs() - K * 2.0 ** -49 * M).max()) <= 0.0
+    assert float(out[17::64].abs().max()) == 0.0
