@@ -13,8 +13,8 @@
 // the fourth carries less than 2^-32 of the result) the classes go into two 64-bit integers per entry, without rounding.
 // In a Gram a column keeps its exponent from tile to tile while the tile's largest entry stays within a few bits below it;
 // when it does not, the sums so far are flushed to the CTA's FP64 partial at the old exponents and the column
-// gets a new one, so no tile loses bits to a larger one.  An entry is off by 2^-52 of its columns' norms: an entry of a column
-// beside a larger one of the same tile keeps fewer bits, which the sum over the rows does not see.
+// gets a new one, so no tile loses bits to a larger one.  An entry is off by some 2^-52 of its columns' norms: a value
+// beside a larger one of its column in the tile keeps fewer bits, which the sum over the rows does not see.
 // A projection does: each of its rows is a result.  There the exponents are those of the rows, after the columns are
 // weighted: with 2^(g_k) the largest coefficient of input column k,
 //     new_rj = sum_k (x_rk 2^(g_k)) (c_kj 2^(-g_k)),
