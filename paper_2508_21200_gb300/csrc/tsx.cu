@@ -11,10 +11,10 @@
 // others are below 2^-55 of the largest); those of equal s + t share an accumulator (a "class").  Every 128 complex summands
 // (the rows of a Gram, the columns of a projection: 2 x 128 x 4 x 2^14 = 2^24 for the first four classes; a class beyond
 // the fourth carries less than 2^-32 of the result) the classes go into two 64-bit integers per entry, without rounding.
-// In a Gram a column keeps its exponent from tile to tile while the tile's largest entry stays within a few bits below it;
+// In a Gram a column keeps its exponent from tile to tile while the tile's largest entry stays within ten bits below it;
 // when it does not, the sums so far are flushed to the CTA's FP64 partial at the old exponents and the column
-// gets a new one, so no tile loses bits to a larger one.  An entry is off by some 2^-52 of its columns' norms: a value
-// beside a larger one of its column in the tile keeps fewer bits, which the sum over the rows does not see.
+// gets a new one.  A value is off by 2^-56 of the power of two above the largest of its column so far, an entry of the Gram by
+// some 2^-55 of its columns' norms: a value beside a larger one keeps fewer bits, which the sum over the rows does not see.
 // A projection does: each of its rows is a result.  There the exponents are those of the rows, after the columns are
 // weighted: with 2^(g_k) the largest coefficient of input column k,
 //     new_rj = sum_k (x_rk 2^(g_k)) (c_kj 2^(-g_k)),
@@ -63,7 +63,10 @@ constexpr int NS = 7;                 // digits
 constexpr int CUT_UNITS = 4;          // units a cutting warp holds in registers
 constexpr int X_THREADS = 512;        // most threads of a CTA (128 registers)
 constexpr int X_DRAIN = 128;          // complex summands between drains
-constexpr int X_SLACK = 2;            // bits a column's tile may stay below its exponent
+// Gram: bits that a column's tiles may stay below its exponent.  H V of a spin chain varies by 2^7 from tile to tile (the diagonal
+// and the number of flips do), so with 2 bits 60 to 97 of 100 tiles flushed the sums of their CTA, with 10 three to thirteen do
+// (a tile above the largest so far).  A new exponent is the tile's own: a bit above it would halve the flushes, at twice the error.
+constexpr int X_SLACK = 10;
 constexpr int X_EMIN = 530, X_EMAX = 1510;   // exponent fields that are cut; others take the direct path
 constexpr int E_UNSET = -100000;
 // projections: exponents of the rows that are cut, of the coefficients' largest (either side); a zero coefficient row; the
@@ -497,7 +500,7 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
               if (k != 0 && (E < X_EMIN || E > X_EMAX)) {
                 flag[1] = 1;
               } else if (k != 0 && (ex > e || ex < e - X_SLACK)) {
-                e = ex + 1;
+                e = ex;
                 flag[0] = 1;
               }
               G.ecol[(i & 3) * ncl + ucol[x]] = e;
