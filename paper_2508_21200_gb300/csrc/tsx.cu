@@ -823,6 +823,9 @@ int launch_tsx(const TSArgs &a, int nsm, cudaStream_t st) {
   if ((a.mode != 2 && off(a.src)) || (a.mode != 0 && off(a.out))) return 0;
   XPlan p, pg;
   TSArgs b = a;
+  // projections of ranks 1 and 2 from 2^16 rows on: eight columns are cut for one or two, and the FMAs of so few cost less (r = 1, five
+  // blocks at n = 18: 150 us there, 218 here; at n = 14 29 and 28)
+  if (a.mode != 0 && a.r <= 2 && a.N >= 65536) return 0;
   if (a.mode != 0) {
     b.mode = 0;
     b.src = a.out;
