@@ -1111,11 +1111,16 @@ __global__ void __launch_bounds__(128) few_gram_kernel(TSArgs a, const cx<T> *__
   if (t == 0 && e < ldg * r) reinterpret_cast<zd *>(a.red)[e] = s;
 }
 
-// Up to 4096 rows and 2^20 multiply-adds per Gram, where these launches take less than the tiles' shortest:
-// FP64 at n = 8, r = 4, 5 blocks: Gram 24 us as tiles and their sum, 4 here; projection and Gram 20, 8 here.
+// Up to 4096 rows and 2^20 multiply-adds per Gram in complex128, where these launches take less than the tiles' shortest:
+// n = 8, r = 4, 5 blocks: Gram 24 us as tiles and their sum, 4 here; projection and Gram 20, 8 here.  In complex64 the tiles sum
+// in FP32 and these in FP64, so the line is at 256 rows, and for the tile widths (where a tile's copies are whole chunks) at 64 and
+// without the combine: Gram of 4 at n = 8, r = 5 9.6 us as tiles, 6 here; the combine of five at n = 12, r = 16 9 and 89 us, at n = 8,
+// r = 8 7 and 10.
 template <typename T> static bool launch_few(const TSArgs &a, cudaStream_t st) {
   const int g = a.gram_left + 1;
   if (!a.red || a.N > 4096 || a.N * g * a.r * a.r > (1 << 20) || a.nq + 1 > MAXB + 1) return false;
+  const bool width = a.r == 8 || a.r == 16 || a.r == 32;
+  if (sizeof(T) == 4 && (width ? a.N > 64 || a.mode == 2 : a.N > 256)) return false;
   if (a.mode == 0 ? a.out != nullptr : a.out == nullptr) return false;
   if (a.mode != 2 && !a.src) return false;
   if (a.mode != 0)
