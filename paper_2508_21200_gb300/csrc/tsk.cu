@@ -400,10 +400,20 @@ __global__ void __launch_bounds__(TS_THREADS) ts2_kernel(const __grid_constant__
           d[1] = mk<T>((T)v.z, (T)v.w);
         }
       } else {
-        for (int e = tid; e < tr * rp; e += TS_THREADS) {
-          const int lr = e / rp, c = e % rp;
-          dst[lr * RS + c] = (lr < rows && c < r) ? ldg1(qm + (size_t)lr * r + c) : mk<T>(0, 0);
-        }
+        // at most 64 x 32 elements: all of a thread's loads are in flight before the first store (a loop of a fixed unroll leaves its
+        // remainder in series: five blocks at n = 18, r = 17 / 23 took 317 / 700 us, now 225 / 460)
+        cx<T> v[64 * 32 / TS_THREADS];
+        int at[64 * 32 / TS_THREADS];
+#pragma unroll
+        for (int x = 0; x < 64 * 32 / TS_THREADS; ++x)
+          if (x * TS_THREADS < tr * rp) {
+            const int e = tid + x * TS_THREADS, lr = e / rp, c = e - lr * rp;
+            at[x] = lr * RS + c;
+            v[x] = (lr < rows && c < r) ? ldg1(qm + (size_t)lr * r + c) : mk<T>(0, 0);
+          }
+#pragma unroll
+        for (int x = 0; x < 64 * 32 / TS_THREADS; ++x)
+          if (tid + x * TS_THREADS < tr * rp) dst[at[x]] = v[x];
       }
     }
     __syncthreads();
@@ -920,7 +930,7 @@ static int launch_ts_v1(const TSArgs &a, int nsm, cudaStream_t st) {
   const long long ntiles = (a.N + tr - 1) / tr;
   int grid = (int)(ntiles < (long long)ts_max_grid(nsm) ? ntiles : ts_max_grid(nsm));
   if (grid < 1) grid = 1;
-  const int cpt_max = sizeof(T) == 4 ? 4 : 2, cpt = ts_cpt<T>(a);
+  const int cpt = ts_cpt<T>(a);
   auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(a, tr, coef_smem ? 1 : 0, coefg); };
   if (cpt == 4) go(ts_kernel<T, (sizeof(T) == 4 ? 4 : 2)>);
   else if (cpt == 2) go(ts_kernel<T, 2>);
@@ -1042,14 +1052,14 @@ static int launch_ts_t(const TSArgs &a, int nsm, cudaStream_t st) {
   const long long ntiles = (a.N + tr - 1) / tr;
   int grid = (int)(ntiles < (long long)ts_max_grid(nsm) ? ntiles : ts_max_grid(nsm));
   if (grid < 1) grid = 1;
-  const int cpt_max = sizeof(T) == 4 ? 4 : 2, cpt = ts_cpt<T>(a);
+  const int cpt = ts_cpt<T>(a);
   auto go = [&](auto kern) { ::lrei::count_launch(); kern<<<grid, TS_THREADS, bytes, st>>>(a, tr, coefg); };
   if (mt == 1) {
-    if (cpt == cpt_max && cpt_max == 4) go(ts2_kernel<T, (sizeof(T) == 4 ? 4 : 2), 1>);
+    if (cpt == 4) go(ts2_kernel<T, (sizeof(T) == 4 ? 4 : 2), 1>);
     else if (cpt == 2) go(ts2_kernel<T, 2, 1>);
     else go(ts2_kernel<T, 1, 1>);
   } else {
-    if (cpt == cpt_max && cpt_max == 4) go(ts2_kernel<T, (sizeof(T) == 4 ? 4 : 2), 2>);
+    if (cpt == 4) go(ts2_kernel<T, (sizeof(T) == 4 ? 4 : 2), 2>);
     else if (cpt == 2) go(ts2_kernel<T, 2, 2>);
     else go(ts2_kernel<T, 1, 2>);
   }
