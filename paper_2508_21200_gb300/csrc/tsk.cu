@@ -678,9 +678,12 @@ __global__ void __launch_bounds__(256, MINB) ts3_kernel(const __grid_constant__ 
     asm volatile("cp.async.commit_group;\n" ::);
   }
   int since = 0;
-  // padded ranks with two tiles per CTA (ts2_kernel has twice the CTAs): after each; above 28 its tiles are shorter beside
-  // the coefficients
-  const int every = PAD && ntiles <= 2 * (long long)gridDim.x ? 1 : (PAD && R == 32 && GMAX <= 5 && mode != 0 && r > 28 ? FLUSHT / 2 : FLUSHT);
+  // three kinds that ts2_kernel or shared memory sums treat otherwise: width 16 padded with two tiles per CTA (there twice the
+  // CTAs): after each; above rank 28 beside coefficients (there shorter tiles): half; six blocks at width 32: as fewer blocks
+  int every = FLUSHT;
+  if (PAD && R == 16 && GMAX <= 3 && ntiles <= 2 * (long long)gridDim.x) every = 1;
+  if (PAD && R == 32 && GMAX <= 5 && mode != 0 && r > 28) every = FLUSHT / 2;
+  if (R == 32 && GMAX > 5 && g <= 6 && mode == 0 && (!PAD || r <= 28)) every = (PAD ? 4 : 8) * FLUSHT;
   for (; tile < ntiles; tile += gridDim.x) {
     switch (nst) {   // all but the newest nst - 2 groups: this tile is there
       case 2: asm volatile("cp.async.wait_group 0;\n" ::); break;
