@@ -1071,10 +1071,11 @@ static int launch_ts_t(const TSArgs &a, int nsm, cudaStream_t st) {
 
 // ------------------------------------------- few rows
 // Passes of few rows are latency: tiles leave most SMs idle (8 to 256 of them at N = 256 .. 4096) and their sums need
-// a second launch.  Here every entry of the new block is a sum over eight lanes and every Gram entry one over a warp
-// or a CTA, in FP64 for both precisions (the coefficients as they are), and the Gram goes to a.red directly.
+// a second launch.  Here every entry of the new block is a sum over a few lanes and every Gram entry one over a warp
+// or a CTA, and the Gram goes to a.red directly.  Sums are in FP64, or for complex64 as good: products and sums with
+// their rounding errors kept (fma and TwoSum: 9 FP32 instructions a product, where an FP64 multiply-add takes 64 cycles), and
+// the coefficients as pairs of FP32.
 // The rows of a CTA are read before one is written, so the new block may replace an input.
-template <typename T>
 __global__ void __launch_bounds__(256) few_new_kernel(TSArgs a) {
   const int r = a.r, rows = 32 / r, o = threadIdx.x >> 3, q = threadIdx.x & 7, j = o % r;
   const long long row = (long long)blockIdx.x * rows + o / r;
@@ -1084,10 +1085,10 @@ __global__ void __launch_bounds__(256) few_new_kernel(TSArgs a) {
   if (in)
     for (int k = q; k < K; k += 8) {
       const int m = k / r, i = k % r;
-      const cx<T> x = reinterpret_cast<const cx<T> *>(m < a.nq ? a.q[m] : a.src)[(size_t)row * r + i];
+      const zd x = reinterpret_cast<const zd *>(m < a.nq ? a.q[m] : a.src)[(size_t)row * r + i];
       const zd c = m < a.nq ? (a.coefQ ? a.coefQ[(size_t)j * a.nq * r + k] : mk<double>(0, 0))
                             : (a.coefS ? a.coefS[(size_t)j * r + i] : mk<double>(0, 0));
-      fma_(s, cvt<double>(x), c);
+      fma_(s, x, c);
     }
 #pragma unroll
   for (int x = 4; x > 0; x >>= 1) {
@@ -1095,8 +1096,74 @@ __global__ void __launch_bounds__(256) few_new_kernel(TSArgs a) {
     s.im += __shfl_xor_sync(0xffffffffu, s.im, x);
   }
   __syncthreads();
+  if (in && q == 0) reinterpret_cast<zd *>(a.out)[(size_t)row * r + j] = row < a.zero_rows ? mk<double>(0, 0) : s;
+}
+
+// (hi, lo) += x y
+__device__ __forceinline__ void two_prod_acc(float &hi, float &lo, float x, float y) {
+  const float p = x * y;
+  lo += fmaf(x, y, -p);
+  two_sum_acc(hi, lo, p);
+}
+
+// x as a pair of FP32: truncated, and the 29 bits left; by the bits (a conversion from FP64 runs at its rate).  Zero below 2^-126,
+// infinite from 2^128 on.
+__device__ __forceinline__ float2 fp32_pair(double x) {
+  const int h = __double2hiint(x), l = __double2loint(x), sg = h & 0x80000000, e = ((h >> 20) & 0x7ff) - 896;
+  if (e <= 0) return make_float2(0.f, 0.f);
+  if (e >= 255) return make_float2((float)x, 0.f);
+  const float rest = (float)(l & 0x1fffffff) * __int_as_float(max(e - 52, 0) << 23);   // below 2^-74: zero
+  return make_float2(__int_as_float(sg | e << 23 | (h & 0xfffff) << 3 | (int)((unsigned)l >> 29)), sg ? -rest : rest);
+}
+
+// rb rows per CTA, ln lanes per entry of the new block (rb r ln <= 256); the coefficients by blocks of r rows through shared
+// memory, so that a CTA splits each of them once.
+constexpr int FEW_COEFS = 2048;
+__global__ void __launch_bounds__(256) few_new32_kernel(TSArgs a, int rb, int ln) {
+  __shared__ float4 cs[FEW_COEFS];   // (re, im), then what their FP32 values leave
+  const int r = a.r, nb = a.nq + (a.mode == 1 ? 1 : 0), per = FEW_COEFS / (r * r);
+  const int o = threadIdx.x / ln, q = threadIdx.x % ln, j = o % r, lr = o / r;
+  const long long row = (long long)blockIdx.x * rb + lr;
+  const bool in = lr < rb && row < a.N;
+  float2 hi = make_float2(0.f, 0.f), lo = hi;
+  for (int m0 = 0; m0 < nb; m0 += per) {
+    const int n = min(per, nb - m0) * r;
+    __syncthreads();
+    for (int e = threadIdx.x; e < n * r; e += 256) {
+      const int jj = e / n, kk = e - jj * n, k = m0 * r + kk;
+      const zd c = k < a.nq * r ? (a.coefQ ? a.coefQ[(size_t)jj * a.nq * r + k] : mk<double>(0, 0))
+                                : (a.coefS ? a.coefS[(size_t)jj * r + k - a.nq * r] : mk<double>(0, 0));
+      const float2 re = fp32_pair(c.re), im = fp32_pair(c.im);
+      cs[kk * r + jj] = make_float4(re.x, im.x, re.y, im.y);
+    }
+    __syncthreads();
+    if (in)
+      for (int m = m0; m < min(nb, m0 + per); ++m) {
+        const cx<float> *x = reinterpret_cast<const cx<float> *>(m < a.nq ? a.q[m] : a.src) + (size_t)row * r;
+        const float4 *c = cs + (m - m0) * r * r + j;
+#pragma unroll 8
+        for (int i = q; i < r; i += ln) {
+          const cx<float> v = x[i];
+          const float4 w = c[i * r];
+          two_prod_acc(hi.x, lo.x, v.re, w.x);
+          two_prod_acc(hi.x, lo.x, -v.im, w.y);
+          two_prod_acc(hi.y, lo.y, v.re, w.y);
+          two_prod_acc(hi.y, lo.y, v.im, w.x);
+          lo.x = fmaf(v.re, w.z, fmaf(-v.im, w.w, lo.x));
+          lo.y = fmaf(v.re, w.w, fmaf(v.im, w.z, lo.y));
+        }
+      }
+  }
+  for (int x = ln >> 1; x > 0; x >>= 1) {
+    const float2 h = make_float2(__shfl_xor_sync(0xffffffffu, hi.x, x), __shfl_xor_sync(0xffffffffu, hi.y, x));
+    lo.x += __shfl_xor_sync(0xffffffffu, lo.x, x);
+    lo.y += __shfl_xor_sync(0xffffffffu, lo.y, x);
+    two_sum_acc(hi.x, lo.x, h.x);
+    two_sum_acc(hi.y, lo.y, h.y);
+  }
+  __syncthreads();
   if (in && q == 0)
-    reinterpret_cast<cx<T> *>(a.out)[(size_t)row * r + j] = row < a.zero_rows ? mk<T>(0, 0) : cvt<T>(s);
+    reinterpret_cast<cx<float> *>(a.out)[(size_t)row * r + j] = row < a.zero_rows ? mk<float>(0.f, 0.f) : mk<float>(hi.x + lo.x, hi.y + lo.y);
 }
 
 // TPE threads per entry, 128 per CTA.
@@ -1108,8 +1175,21 @@ __global__ void __launch_bounds__(128) few_gram_kernel(TSArgs a, const cx<T> *__
   zd s = mk<double>(0, 0);
   if (e < ldg * r) {
     const cx<T> *L = m < a.gram_left ? reinterpret_cast<const cx<T> *>(a.q[m]) : G;
+    if constexpr (sizeof(T) == 8) {
 #pragma unroll 4
-    for (int b = t; b < (int)a.N; b += TPE) fmac_(s, cvt<double>(L[(size_t)b * r + i]), cvt<double>(G[(size_t)b * r + j]));
+      for (int b = t; b < (int)a.N; b += TPE) fmac_(s, L[(size_t)b * r + i], G[(size_t)b * r + j]);
+    } else {
+      float2 hi = make_float2(0.f, 0.f), lo = hi;
+#pragma unroll 8
+      for (int b = t; b < (int)a.N; b += TPE) {
+        const cx<float> x = L[(size_t)b * r + i], y = G[(size_t)b * r + j];
+        two_prod_acc(hi.x, lo.x, x.re, y.re);
+        two_prod_acc(hi.x, lo.x, x.im, y.im);
+        two_prod_acc(hi.y, lo.y, x.re, y.im);
+        two_prod_acc(hi.y, lo.y, -x.im, y.re);
+      }
+      s = mk<double>((double)hi.x + (double)lo.x, (double)hi.y + (double)lo.y);
+    }
   }
 #pragma unroll
   for (int x = 16; x > 0; x >>= 1) {
@@ -1124,16 +1204,13 @@ __global__ void __launch_bounds__(128) few_gram_kernel(TSArgs a, const cx<T> *__
   if (t == 0 && e < ldg * r) reinterpret_cast<zd *>(a.red)[e] = s;
 }
 
-// Up to 4096 rows and 2^20 multiply-adds per Gram in complex128, where these launches take less than the tiles' shortest:
-// n = 8, r = 4, 5 blocks: Gram 24 us as tiles and their sum, 4 here; projection and Gram 20, 8 here.  In complex64 the tiles sum
-// in FP32 and these in FP64, so the line is at 256 rows, and for the tile widths (where a tile's copies are whole chunks) at 64 and
-// without the combine: Gram of 4 at n = 8, r = 5 9.6 us as tiles, 6 here; the combine of five at n = 12, r = 16 9 and 89 us, at n = 8,
-// r = 8 7 and 10.
+// Up to 4096 rows and 2^20 multiply-adds per Gram, where these launches take less than the tiles' shortest:
+// FP64 at n = 8, r = 4, 5 blocks: Gram 24 us as tiles and their sum, 4 here; projection and Gram 20, 8 here.  Complex64 has the same
+// lines for its accuracy: tiles take 9 us for the combine of five blocks at n = 12, r = 16 (here 31, with FP64 arithmetic 89) and 6 for
+// one block's Gram (13 and 21), but sum in FP32; below 2^10 rows or rank 8 these launches are the faster ones.
 template <typename T> static bool launch_few(const TSArgs &a, cudaStream_t st) {
   const int g = a.gram_left + 1;
   if (!a.red || a.N > 4096 || a.N * g * a.r * a.r > (1 << 20) || a.nq + 1 > MAXB + 1) return false;
-  const bool width = a.r == 8 || a.r == 16 || a.r == 32;
-  if (sizeof(T) == 4 && (width ? a.N > 64 || a.mode == 2 : a.N > 256)) return false;
   if (a.mode == 0 ? a.out != nullptr : a.out == nullptr) return false;
   if (a.mode != 2 && !a.src) return false;
   if (a.mode != 0)
@@ -1141,9 +1218,16 @@ template <typename T> static bool launch_few(const TSArgs &a, cudaStream_t st) {
       if (a.q[m] == a.out) return false;
   const cx<T> *G = reinterpret_cast<const cx<T> *>(a.mode == 0 ? a.src : a.out);
   if (a.mode != 0) {
-    const int rows = 32 / a.r;
     ::lrei::count_launch();
-    few_new_kernel<T><<<(int)((a.N + rows - 1) / rows), 256, 0, st>>>(a);
+    if (sizeof(T) == 8) {
+      const int rows = 32 / a.r;
+      few_new_kernel<<<(int)((a.N + rows - 1) / rows), 256, 0, st>>>(a);
+    } else {
+      int rb = 1, ln = 1;   // about 256 CTAs
+      while (rb * 256 < a.N && 2 * rb * a.r <= 256) rb *= 2;
+      while (ln < 8 && 2 * ln * rb * a.r <= 256) ln *= 2;
+      few_new32_kernel<<<(int)((a.N + rb - 1) / rb), 256, 0, st>>>(a, rb, ln);
+    }
   }
   const int entries = g * a.r * a.r;
   ::lrei::count_launch();
