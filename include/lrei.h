@@ -59,7 +59,10 @@ typedef enum {
 /* Arithmetic of the N-length (bulk) work.  Small r x r / k x k solves are
  * FP64 in every mode. */
 typedef enum {
-  LREI_FP64 = 0,        /* complex128 storage and arithmetic */
+  LREI_FP64 = 0,        /* complex128 storage and arithmetic; tall-skinny products of more than 4096
+                         * rows as integer digit products at the accuracy of FP64 sums: a Gram entry
+                         * relative to the norms of its columns, a row of a new block relative to the
+                         * largest of that row's entries (each times its largest coefficient) */
   LREI_MIXED_C64 = 1,   /* complex64 storage and FP32 arithmetic, FP64 small solves */
   LREI_MIXED_BF16X = 2  /* BF16-split tensor-core products: declared, not built in this version;
                          * lrei_create returns LREI_ERR_UNSUPPORTED for it */
@@ -185,8 +188,10 @@ int lrei_apply_h(lrei_ctx *ctx, const void *V_dev, void *Y_dev, int r);
  * block), by the same fused tile pass and deterministic reduction the step uses.
  * blocks_dev: m device pointers (1 <= m <= 13), each N x r row-major with the
  * context's r and precision; G_dev: device complex128 (m r) x r, column-major,
- * written on the context's stream (no host sync).  Compensated FP32 sums in
- * mixed precision, FP64 otherwise. */
+ * written on the context's stream (no host sync).  Mixed precision: FP32 sums of 8 to
+ * 256 rows, compensated beyond.  LREI_FP64: an entry is as close as FP64 sums are,
+ * relative to the norms of its two columns (2^-55 or so of their product): a value
+ * that is small beside others of its column does not keep 53 bits of its own. */
 int lrei_gram(lrei_ctx *ctx, const void *const *blocks_dev, int nblocks, void *G_dev);
 
 /* Low-rank right-hand side at the current state: f(rho) = Z V^* + V W^*

@@ -812,9 +812,9 @@ int tsx_run(const TSArgs &a, bool proj, const XPlan &p, int nsm, cudaStream_t st
 // as fast (about 20 us, all latency) and its sums a little closer).  Modes 1 and 2 are a projection and the Gram of what it
 // wrote: in one kernel the projection's planes, the coefficients' and the Gram's sums leave shared memory for
 // 16-row tiles only, and the pass was slower than the two (n = 20, r = 16, five blocks: 7.1 ms against 2.6 + 1.9).
-// Measured against the general kernel (ts2_kernel) at n = 20, r = 16: Gram of 1 / 2 / 3 / 5 blocks 1.83 / 3.66 / 5.55 /
-// 10.96 ms there and 0.26 / 0.49 / 0.67 / 0.99 ms here (the five blocks' tensor work alone is 0.47 ms), the projection of
-// five blocks onto one 2.2 ms, an RK4 step 96.0 and 22.2 ms.
+// Measured against the general kernel (ts2_kernel) at n = 20, r = 16: Gram of 1 / 2 / 3 / 5 Krylov blocks 1.83 / 3.66 / 5.55 /
+// 10.96 ms there and 0.27 / 0.51 / 0.64 / 0.98 ms here (the five blocks' tensor work alone is 0.47 ms), an RK4 step 96.0 and
+// 15.3 ms.
 int launch_tsx(const TSArgs &a, int nsm, cudaStream_t st) {
   if ((a.mode == 0 && a.out) || (a.mode != 0 && !a.out) || a.r > MAX_R || a.N < 256) return 0;
   auto off = [](const void *x) { return (reinterpret_cast<uintptr_t>(x) & 15) != 0; };
