@@ -11,9 +11,9 @@
 // others are below 2^-55 of the largest); those of equal s + t share an accumulator (a "class").  Every 128 complex summands
 // (the rows of a Gram, the columns of a projection: 2 x 128 x 4 x 2^14 = 2^24 for the first four classes; a class beyond
 // the fourth carries less than 2^-32 of the result) the classes go into two 64-bit integers per entry, without rounding.
-// In a Gram a column keeps its exponent from tile to tile while the tile's largest entry stays within ten bits below it;
-// when it does not, the sums so far are flushed to the CTA's FP64 partial at the old exponents and the column
-// gets a new one.  A value is off by 2^-56 of the power of two above the largest of its column so far, an entry of the Gram by
+// In a Gram a column keeps its exponent from tile to tile while the tile's largest entry stays within ten bits below it.
+// Above it, the column's exponent rises and the sums so far are shifted down; further below, they are flushed to the CTA's
+// FP64 partial at the old exponents and the column gets a new one.  A value is off by 2^-56 of the power of two above the largest of its column so far, an entry of the Gram by
 // some 2^-55 of its columns' norms: a value beside a larger one keeps fewer bits, which the sum over the rows does not see.
 // A projection does: each of its rows is a result.  There the exponents are those of the rows, after the columns are
 // weighted: with 2^(g_k) the largest coefficient of input column k,
@@ -63,10 +63,12 @@ constexpr int NS = 7;                 // digits
 constexpr int CUT_UNITS = 4;          // units a cutting warp holds in registers
 constexpr int X_THREADS = 512;        // most threads of a CTA (128 registers)
 constexpr int X_DRAIN = 128;          // complex summands between drains
-// Gram: bits that a column's tiles may stay below its exponent.  H V of a spin chain varies by 2^7 from tile to tile (the diagonal
-// and the number of flips do), so with 2 bits 60 to 97 of 100 tiles flushed the sums of their CTA, with 10 three to thirteen do
-// (a tile above the largest so far).  A new exponent is the tile's own: a bit above it would halve the flushes, at twice the error.
-constexpr int X_SLACK = 10;
+// Gram: bits that a column's tiles may stay below its exponent, and what tells the multiplying warps that one changed.  H V of a
+// spin chain varies by 2^7 from tile to tile (the diagonal and the number of flips do): with 2 bits 60 to 97 of 100 tiles flushed
+// the sums of their CTA, 7 us each.  With 10, and a tile above the largest so far shifting the sums in shared memory, hardly any does.
+// A column's first exponent is a bit above its tile's, which spares most columns without structure any shift (6 random blocks at
+// n = 14, r = 16: 66 us against 73), later ones are the tile's own.
+constexpr int X_SLACK = 10, X_RAISED = 1, X_LOWERED = 2;
 constexpr int X_EMIN = 530, X_EMAX = 1510;   // exponent fields that are cut; others take the direct path
 constexpr int E_UNSET = -100000;
 // projections: exponents of the rows that are cut, of the coefficients' largest (either side); a zero coefficient row; the
@@ -189,6 +191,19 @@ struct Sum {
   }
   __device__ __forceinline__ void store(uint32_t at) const {
     asm volatile("st.shared.v2.s64 [%0], {%1, %2};\n" ::"r"(at), "l"(h), "l"(l));
+  }
+  __device__ __forceinline__ void down(int k) {   // h 2^32 + l, k > 0 bits down
+    if (k >= 32) {
+      l = h + (l >> 32);
+      h = 0;
+      k -= 32;
+    }
+    if (k >= 32) {
+      l >>= min(k, 63);
+      return;
+    }
+    l = (l >> k) + ((h & ((1ll << k) - 1)) << (32 - k));
+    h >>= k;
   }
 };
 
@@ -500,8 +515,8 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
               if (k != 0 && (E < X_EMIN || E > X_EMAX)) {
                 flag[1] = 1;
               } else if (k != 0 && (ex > e || ex < e - X_SLACK)) {
-                e = ex;
-                flag[0] = 1;
+                atomicOr(flag, ex > e ? X_RAISED : X_LOWERED);
+                e = e == E_UNSET ? ex + 1 : ex;
               }
               G.ecol[(i & 3) * ncl + ucol[x]] = e;
               if (e == E_UNSET) e = 0;   // zero so far: any exponent gives zero digits
@@ -687,13 +702,36 @@ __global__ void __launch_bounds__(X_THREADS, 1) tsx_kernel(const __grid_constant
       for (int c = tid; c < ncl; c += nt) G.eacc[c] = el[c];
       clear_sums();
     };
+    // the sums for larger exponents el: down by the bits that an entry's two columns rose
+    auto shift = [&](const int *el) {
+      bar_sync(BAR_MUL, nt);
+      if (has_item)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int c0 = (x < 2 ? ga : gb) * 8 + g, c1 = gg * 8 + in0 * 8 + 2 * q + (x & 1);
+          if (G.eacc[c0] == E_UNSET || G.eacc[c1] == E_UNSET) continue;   // zero so far
+          const int k = el[c0] - G.eacc[c0] + el[c1] - G.eacc[c1];
+          if (k == 0) continue;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            Sum v;
+            v.load(sums + (h * 4 + x) * sum_step);
+            v.down(k);
+            v.store(sums + (h * 4 + x) * sum_step);
+          }
+        }
+      bar_sync(BAR_MUL, nt);
+      for (int c = tid; c < ncl; c += nt) G.eacc[c] = el[c];
+    };
     int since = 0;                // rows in the accumulators since the last drain or flush
     for (int i = 0; i < mine; ++i) {
       bar_sync(BAR_FULL + (i & 1), all);
-      const bool changed = G.flags[4 + 2 * (i & 3)] != 0, direct = G.flags[5 + 2 * (i & 3)] != 0;
+      const int changed = G.flags[4 + 2 * (i & 3)];
+      const bool direct = G.flags[5 + 2 * (i & 3)] != 0;
       if (changed) {
         if (since > 0) drain();
-        flush(G.ecol + (i & 3) * ncl);
+        if (changed & X_LOWERED) flush(G.ecol + (i & 3) * ncl);
+        else shift(G.ecol + (i & 3) * ncl);
         since = 0;
       }
       if (direct) {
@@ -813,8 +851,8 @@ int tsx_run(const TSArgs &a, bool proj, const XPlan &p, int nsm, cudaStream_t st
 // wrote: in one kernel the projection's planes, the coefficients' and the Gram's sums leave shared memory for
 // 16-row tiles only, and the pass was slower than the two (n = 20, r = 16, five blocks: 7.1 ms against 2.6 + 1.9).
 // Measured against the general kernel (ts2_kernel) at n = 20, r = 16: Gram of 1 / 2 / 3 / 5 Krylov blocks 1.83 / 3.66 / 5.55 /
-// 10.96 ms there and 0.27 / 0.51 / 0.64 / 0.98 ms here (the five blocks' tensor work alone is 0.47 ms), an RK4 step 96.0 and
-// 15.3 ms.
+// 10.96 ms there and 0.24 / 0.47 / 0.62 / 0.91 ms here (the five blocks' tensor work alone is 0.47 ms), an RK4 step 96.0 and
+// 15.1 ms.
 int launch_tsx(const TSArgs &a, int nsm, cudaStream_t st) {
   if ((a.mode == 0 && a.out) || (a.mode != 0 && !a.out) || a.r > MAX_R || a.N < 256) return 0;
   auto off = [](const void *x) { return (reinterpret_cast<uintptr_t>(x) & 15) != 0; };
