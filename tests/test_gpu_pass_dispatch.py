@@ -1,5 +1,5 @@
-"""Passes on both sides of the lines between the kernels: rows summed entry by entry or tiled (64, 256 and 4096 rows, by precision and
-width), projections of ranks 1 and 2 in complex128 below and from 2^16 rows on, and blocks whose rows are no whole
+"""Passes on both sides of the lines between the kernels: rows summed entry by entry or tiled (4096 rows, and 2^20 multiply-adds of a
+Gram), projections of ranks 1 and 2 in complex128 below and from 2^16 rows on, and blocks whose rows are no whole
 groups of four columns (loaded by elements).
 
 Steps against the same step from a factor with its columns turned by phases, which every path must carry through: the density
